@@ -88,7 +88,14 @@ typedef struct {
                            dividing every f[x] - f_min (LABS: at least 2); 0
                            for float costs and for a constant vector.  0 is
                            always valid. */
-    uint32_t reserved;  /* 0 */
+    uint32_t reserved;  /* 0 in a struct filled by hand.  qaoa_cost_stats_compute
+                           leaves a mark here where f[x] == f[2^n - 1 - x] for
+                           every x (LABS, MaxCut, even-order polynomials);
+                           simulations from |+>^n and gradients of such a
+                           vector then evolve only the amplitudes whose top
+                           qubit is 0, with the same results.  The mark covers
+                           n and the fields above: changing any of them, or
+                           setting it to 0, takes the path of any vector. */
 } qaoa_cost_stats;
 
 /* Human-readable name of a status code (static string, never NULL). */
@@ -378,7 +385,8 @@ qaoa_status qaoa_overlap(int n, const void *d_state, qaoa_state_type st,
  * Environment variables, read at each call: QAOA_ADJOINT_PAIRS = "never" (no
  * such groups) or "always" (every group above the lowest 12 qubits is one);
  * QAOA_ADJOINT_WIDE = "pair" (every pass of those groups on CTA pairs) or
- * "all" (every pass, the last one too, on the 512-thread CTA).
+ * "all" (every pass, the last one too, on the 512-thread CTA).  Any of them
+ * takes the plan of the full vector (see qaoa_cost_stats.reserved).
  * Results agree across plans to rounding.
  */
 qaoa_status qaoa_grad(int n, const void *d_costs, qaoa_cost_type ct,

@@ -263,7 +263,8 @@ struct Group {
   bool high;
   int c, h;          // geometry
   uint32_t rot;      // tile bits rotated
-  bool cl = false;   // adjoint cluster pair: also rotates the qubit h + TB - c
+  bool cl = false;   // adjoint 9-qubit group: a tile of 2^(TB+1) amplitudes
+  bool comp = false; // complement pair: the top tile bit selects the box (half vectors)
 };
 
 // LOW group + HIGH groups covering qubits [TB, n), TB - chigh per pass
@@ -405,6 +406,94 @@ std::vector<Group> bwd_groups(int n, int TB) {
   return gs;
 }
 
+// ------------------------------------------------------- half vectors
+//
+// A cost vector with f(x) = f(~x) for all x (LABS, MaxCut, every polynomial of
+// even-order terms) keeps psi(x) = psi(~x) from |+> on, and lambda = f psi the
+// same, so the passes need only the m = n - 1 index bits of the amplitudes whose
+// top qubit is 0: half the traffic and half the arithmetic of every pass, for
+// the same n rotations per layer.  The top qubit's rotation pairs x with its
+// m-bit complement and takes one slot of the last group (Group::comp, see
+// kernels.h); the last pass writes both halves of the state.  Bound by HBM
+// traffic before and after: LABS n = 30 p = 10 objective and gradient 218.6 ->
+// 113.8 ms, weighted MaxCut n = 28 p = 20 113.6 -> 61.6 ms; complex128, bound by
+// the FP64 pipe, LABS n = 23 p = 4 14.45 -> 7.36 ms.
+// qaoa_cost_stats_compute finds the symmetry in the scan that it makes anyway
+// and records it in `reserved` as a mark over the other fields and n, so that a
+// struct filled or changed by hand, or used for another n, takes the full path.
+uint32_t comp_mark(int n, const qaoa_cost_stats *st) {
+  uint64_t h = 0x9E3779B97F4A7C15ull * (uint64_t)(n + 1), w[4];
+  memcpy(&w[0], &st->f_min, 8);
+  memcpy(&w[1], &st->f_max, 8);
+  w[2] = st->n_min;
+  w[3] = st->step_log2;
+  for (uint64_t v : w) {
+    h ^= v;
+    h *= 0xBF58476D1CE4E5B9ull;
+    h ^= h >> 29;
+  }
+  return (uint32_t)(h >> 32) | 1u;
+}
+
+// The smallest n of the half-vector passes: from there the full vector has more
+// tiles than the GPU has SMs, so half of them take half the time.  Below, the
+// passes are as long as one tile takes, and the box pairs make that longer:
+// complex64 n = 18 p = 20 gradient 717 us on half vectors, 653 us on full ones.
+constexpr int kHalfMinN64 = 21, kHalfMinN128 = 20;
+
+// (an adjoint plan asked for by environment variable is one of the full vector)
+bool adjoint_override() { return adjoint_wide_mode() != 1 || adjoint_pairs_mode() != 0; }
+
+bool half_vector(int n, qaoa_state_type st, const qaoa_cost_stats *stats, int init_plus) {
+  return n >= (st == QAOA_C64 ? kHalfMinN64 : kHalfMinN128) && init_plus && stats && stats->reserved != 0 && stats->reserved == comp_mark(n, stats);
+}
+
+// Groups of a half vector of m index bits: the LOW group, then HIGH groups of
+// at most `cap` rotations (`wide`: up to as many groups of one more, on tiles
+// of 2^(TB+1) amplitudes, as save a group), the last of which also takes the
+// complement.  Segments of 2^c amplitudes, the widest that the rotations leave room
+// for (cmax at most).
+std::vector<Group> half_groups(int m, int TB, int cmax, bool wide) {
+  std::vector<Group> gs;
+  gs.push_back(Group{false, TB, TB, (1u << TB) - 1u});
+  const int span = TB - 4;
+  int left = m - TB + 1;  // rotations: the rows and the complement
+  int k = (left + span - 1) / span, nwide = 0;
+  if (wide && (left + span) / (span + 1) < k) {
+    k = (left + span) / (span + 1);
+    nwide = left - span * k;
+  }
+  int q0 = TB;
+  for (int g = 0; g < k; ++g) {
+    const bool last = g == k - 1, w = g >= k - nwide;
+    const int tb = TB + (w ? 1 : 0);
+    // as few as the others can take over, but a wide-segment group's fill where that holds them all
+    int cap = tb - 4;
+    if (!w && nwide == 0 && left <= (k - g) * (TB - cmax)) cap = TB - cmax;
+    const int take = std::min(cap, left);
+    const int rows_new = take - (last ? 1 : 0);
+    Group G;
+    G.high = true;
+    G.cl = w;
+    G.comp = last;
+    const int box = tb - (last ? 1 : 0);
+    int c = 4;
+    while (!w && c < cmax && rows_new <= box - (c + 1)) ++c;
+    G.c = c;
+    const int rows = box - c;
+    G.h = q0 < m - rows ? q0 : m - rows;
+    G.rot = last ? 1u << (tb - 1) : 0u;
+    for (int j = c; j < box; ++j) {
+      const int q = G.h + j - c;
+      if (q >= q0 && q < q0 + rows_new) G.rot |= 1u << j;
+    }
+    gs.push_back(G);
+    q0 += rows_new;
+    left -= take;
+  }
+  return gs;
+}
+
 Geom make_geom(int n, const Group &G, int TB) {
   Geom g;
   g.n = n;
@@ -412,6 +501,7 @@ Geom make_geom(int n, const Group &G, int TB) {
   g.c = G.c;
   g.h = G.h;
   g.ntiles = 1ull << (n - TB);
+  g.comp = G.comp ? (1ull << n) - 1ull : 0ull;
   return g;
 }
 
@@ -624,10 +714,11 @@ int popc8(uint8_t m) { return __builtin_popcount((unsigned)m); }
 template <typename Real, class Low, class High>
 qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                              const double *gam, const double *bet, int p, void *state, int init_plus,
-                             const Ws &ws, double *d_out, cudaStream_t s) {
+                             const Ws &ws, double *d_out, bool half, bool whole, cudaStream_t s) {
   using C2 = typename C2T<Real>::type;
   const int TB = Low::TB;
-  const std::vector<Group> gs = plan_groups(n, TB, kHighC);
+  const int m = half ? n - 1 : n;  // index bits of the vector that the passes hold
+  const std::vector<Group> gs = half ? half_groups(m, TB, kHighC, false) : plan_groups(n, TB, kHighC);
   const std::vector<PassOp> ops = forward_schedule((int)gs.size(), p, init_plus != 0, d_out != nullptr);
   const int nsm = num_sms();
   if (d_out) CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
@@ -641,7 +732,9 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
     P.psi = reinterpret_cast<C2 *>(state);
     P.cost = cost;
     P.cost_kind = cost_kind(ct);
-    P.g = make_geom(n, G, TB);
+    P.g = make_geom(m, G, TB);
+    P.out_scale = half ? 2.0 : 1.0;
+    P.mirror = half && whole && &op == &ops.back() ? (1ull << n) - 1ull : 0ull;
     const bool two = op.l1 >= 0 && op.l2 >= 0;  // both sweeps: s1 ascends, s2 descends
     // (these plans hold every rotated bit in registers: no lane rotations)
     if (op.l1 >= 0) {
@@ -676,8 +769,8 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
     P.partials = ws.partials;
     P.counter = ws.counter;
     P.out = d_out;
-    const double N = (double)(1ull << n);
-    const double bytes = (P.init_plus ? 1.0 : 2.0) * sizeof(C2) * N +
+    const double N = (double)(1ull << m);
+    const double bytes = ((P.init_plus ? 1.0 : 2.0) + (P.mirror ? 1.0 : 0.0)) * sizeof(C2) * N +
                          ((P.has_phase || P.reduce) ? cost_bytes(ct) * N : 0.0);
     if (G.high)
       LAUNCH("fwd_high", bytes, s, launch_fwd(P, true, TB, s, nsm));
@@ -690,29 +783,31 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
 // complex128 at n <= 16: tiles small enough to spread the FP64-bound passes
 // over more SMs, with no more groups than the 4096-amplitude tiles (the
 // partial sums of the tiles fit the workspace: 2^(16-9) * 3 doubles)
+// half: a half vector (half_vector); whole: the last pass writes both halves
 template <typename Real>
 qaoa_status tiled_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                           const double *gam, const double *bet, int p, void *state, int init_plus,
-                          const Ws &ws, double *d_out, cudaStream_t s) {
+                          const Ws &ws, double *d_out, bool half, bool whole, cudaStream_t s) {
   if constexpr (sizeof(Real) == 8) {
     if (n <= 14)
       return tiled_forward_pl<Real, PlanT9Low, PlanT9High>(n, cost, ct, stats, gam, bet, p, state, init_plus,
-                                                           ws, d_out, s);
+                                                           ws, d_out, half, whole, s);
     if (n <= 16)
       return tiled_forward_pl<Real, PlanT10Low, PlanT10High>(n, cost, ct, stats, gam, bet, p, state,
-                                                             init_plus, ws, d_out, s);
+                                                             init_plus, ws, d_out, half, whole, s);
   }
   return tiled_forward_pl<Real, typename FwdTB<Real>::Low, typename FwdTB<Real>::High>(
-      n, cost, ct, stats, gam, bet, p, state, init_plus, ws, d_out, s);
+      n, cost, ct, stats, gam, bet, p, state, init_plus, ws, d_out, half, whole, s);
 }
 
 template <typename Real, class Low, class High>
 qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                               const double *gam, const double *bet, int p, void *state, void *lam,
-                              const Ws &ws, double *d_grad_g, double *d_grad_b, cudaStream_t s) {
+                              const Ws &ws, double *d_grad_g, double *d_grad_b, bool half, cudaStream_t s) {
   using C2 = typename C2T<Real>::type;
   const int TB = Low::TB;
-  const std::vector<Group> gs = plan_groups(n, TB, kHighC);
+  const int m = half ? n - 1 : n;
+  const std::vector<Group> gs = half ? half_groups(m, TB, kHighC, false) : plan_groups(n, TB, kHighC);
   const std::vector<PassOp> ops = adjoint_schedule((int)gs.size(), p);
   const int nsm = num_sms();
   CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
@@ -725,7 +820,9 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
     P.lam = reinterpret_cast<C2 *>(lam);
     P.cost = cost;
     P.cost_kind = cost_kind(ct);
-    P.g = make_geom(n, G, TB);
+    P.g = make_geom(m, G, TB);
+    P.out_scale = half ? 4.0 : 2.0;
+    P.mirror = half && &op == &ops.back() ? (1ull << n) - 1ull : 0ull;
     // psi and lambda are stored divided by sig; un-rotations are the reduced
     // forms of exp(-i (-beta) X)
     P.s1 = G.high ? make_sweep<High>(G.rot, true) : make_sweep<Low>(G.rot, true);
@@ -768,8 +865,8 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
     P.init_lambda = op.init;
     P.partials = ws.partials;
     P.counter = ws.counter;
-    const double N = (double)(1ull << n);
-    const double bytes = (P.init_lambda ? 3.0 : 4.0) * sizeof(C2) * N +
+    const double N = (double)(1ull << m);
+    const double bytes = ((P.init_lambda ? 3.0 : 4.0) + (P.mirror ? 1.0 : 0.0)) * sizeof(C2) * N +
                          ((P.has_phase || P.init_lambda) ? cost_bytes(ct) * N : 0.0);
     if (G.high)
       LAUNCH("bwd_high", bytes, s, launch_bwd(P, true, TB, s, nsm));
@@ -782,17 +879,17 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
 template <typename Real>
 qaoa_status tiled_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                            const double *gam, const double *bet, int p, void *state, void *lam,
-                           const Ws &ws, double *d_grad_g, double *d_grad_b, cudaStream_t s) {
+                           const Ws &ws, double *d_grad_g, double *d_grad_b, bool half, cudaStream_t s) {
   if constexpr (sizeof(Real) == 8) {
     if (n <= 14)
       return tiled_backward_pl<Real, PlanT9Low, PlanT9High>(n, cost, ct, stats, gam, bet, p, state, lam, ws,
-                                                            d_grad_g, d_grad_b, s);
+                                                            d_grad_g, d_grad_b, half, s);
     if (n <= 16)
       return tiled_backward_pl<Real, PlanT10Low, PlanT10High>(n, cost, ct, stats, gam, bet, p, state, lam,
-                                                              ws, d_grad_g, d_grad_b, s);
+                                                              ws, d_grad_g, d_grad_b, half, s);
   }
   return tiled_backward_pl<Real, typename BwdTB<Real>::Low, typename BwdTB<Real>::High>(
-      n, cost, ct, stats, gam, bet, p, state, lam, ws, d_grad_g, d_grad_b, s);
+      n, cost, ct, stats, gam, bet, p, state, lam, ws, d_grad_g, d_grad_b, half, s);
 }
 
 // ---------------------------------------------------- TMA (complex64) path
@@ -837,15 +934,16 @@ TanRot tan_rot(double beta, bool adjoint) {
 
 float2 f2c(std::complex<double> z) { return make_float2((float)z.real(), (float)z.imag()); }
 
-// untwist: leave the final state in the standard basis (the adjoint instead
-// continues from the twisted one).
+// untwist: leave the final state in the standard basis, whole (the adjoint
+// instead continues from the twisted one); half: a half vector (half_vector).
 qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                         const double *gam, const double *bet, int p, void *state, int init_plus,
-                        const Ws &ws, double *d_out, bool untwist, cudaStream_t s) {
+                        const Ws &ws, double *d_out, bool untwist, bool half, cudaStream_t s) {
   using Low = PlanTmaF13Low;
   using High = PlanTmaF13High;
   const int TB = Low::TB;
-  const std::vector<Group> gs = tma_groups(n, TB);
+  const int m = half ? n - 1 : n;  // index bits of the vector that the passes hold
+  const std::vector<Group> gs = half ? half_groups(m, TB, kMaxSegBits, false) : tma_groups(n, TB);
   const std::vector<PassOp> ops = forward_schedule((int)gs.size(), p, init_plus != 0, d_out != nullptr);
   const int nsm = num_sms();
   if (d_out) CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
@@ -856,14 +954,17 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
   for (const PassOp &op : ops) {
     const Group &G = gs[op.group];
     memset(&P, 0, sizeof(P));
-    const int h = G.high ? G.h : 4, c = G.high ? G.c : 4;
-    CK(make_tile_map(&P.map_psi, state, n, TB, h, c, 8, 128), "tensor map (state)");
+    const int h = G.high ? G.h : 4, c = G.high ? G.c : 4, box = TB - (G.comp ? 1 : 0);
+    CK(make_tile_map(&P.map_psi, state, m, box, h, c, 8, 128), "tensor map (state)");
     P.psi = reinterpret_cast<float2 *>(state);
-    CK(make_tile_map(&P.map_cost, const_cast<void *>(cost), n, TB, h, c, (int)cost_bytes(ct), 0),
+    CK(make_tile_map(&P.map_cost, const_cast<void *>(cost), m, box, h, c, (int)cost_bytes(ct), 0),
        "tensor map (cost)");
-    P.ntiles = 1ull << (n - TB);
+    P.ntiles = 1ull << (m - TB);
     P.h = h;
     P.c = c;
+    P.mid2 = tile_map_mid2(box, c);
+    P.comp = G.comp ? m : 0;
+    P.out_scale = half ? 2.0 : 1.0;
     P.cost_kind = cost_kind(ct);
     const bool two = op.l1 >= 0 && op.l2 >= 0;
     const int nrot = __builtin_popcount(G.rot);
@@ -892,6 +993,7 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
       P.end_scale = 1;
       P.scl_end = f2c(sig);
       P.untwist = untwist;
+      if (half && untwist) P.mirror = (1ull << n) - 1ull;
       sig = 1.0;
     }
     if (uses_lanes(P.s1) || uses_lanes(P.s2)) return fail(QAOA_ERR_INVALID_ARG, "internal: plan needs lane rotations");
@@ -904,8 +1006,9 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
     P.counter = ws.counter;
     P.out = d_out;
     P.err = ws.err;
-    const double N = (double)(1ull << n);
-    const double bytes = (P.init_plus ? 8.0 : 16.0) * N + ((P.has_phase || P.reduce) ? cost_bytes(ct) * N : 0.0);
+    const double N = (double)(1ull << m);
+    const double bytes = ((P.init_plus ? 8.0 : 16.0) + (P.mirror ? 8.0 : 0.0)) * N +
+                         ((P.has_phase || P.reduce) ? cost_bytes(ct) * N : 0.0);
     const int kind = (op.l1 >= 0 ? 1 : 0) | (P.has_phase ? 2 : 0) | (op.l2 >= 0 ? 4 : 0) | (P.reduce ? 8 : 0);
     LAUNCH_N(tma_pass_name(true, G.high ? 1 : 0, kind), bytes, s,
              ct == QAOA_COST_U16 ? launch_fwd_tma_u16(P, G.high, s, nsm) : launch_fwd_tma(P, G.high, s, nsm));
@@ -915,12 +1018,13 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
 
 qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                          const double *gam, const double *bet, int p, void *state, void *lam,
-                         const Ws &ws, double *d_grad_g, double *d_grad_b, cudaStream_t s) {
+                         const Ws &ws, double *d_grad_g, double *d_grad_b, bool half, cudaStream_t s) {
   using Low = PlanTmaB12Low;
   using High = PlanTmaB12High;
   const int TB = Low::TB;
-  // HIGH groups of 9 new qubits on cluster pairs where they save a group
-  const std::vector<Group> gs = bwd_groups(n, TB);
+  const int m = half ? n - 1 : n;
+  // HIGH groups of 9 new qubits where they save a group
+  const std::vector<Group> gs = half ? half_groups(m, TB, kMaxSegBits, true) : bwd_groups(n, TB);
   const std::vector<PassOp> ops = adjoint_schedule((int)gs.size(), p);
   const int nsm = num_sms();
   CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
@@ -934,24 +1038,25 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
     memset(&P, 0, sizeof(P));
     const int h = G.high ? G.h : 4, c = G.high ? G.c : 4;
     // a 9-qubit group's pass: one 512-thread CTA per tile, or the cluster pair
-    const bool wide = G.cl && (wide_mode == 2 || (wide_mode == 1 && !(op.lp >= 0 && op.l2 < 0)));
-    const int TBg = wide ? PlanTmaB13High::TB : TB;
-    CK(make_tile_map(&P.map_psi, state, n, TBg, h, c, 8, 128), "tensor map (psi)");
-    CK(make_tile_map(&P.map_lam, lam, n, TBg, h, c, 8, 128), "tensor map (lambda)");
+    // (half vectors: always the 512-thread CTA)
+    const bool wide = G.cl && (half || wide_mode == 2 || (wide_mode == 1 && !(op.lp >= 0 && op.l2 < 0)));
+    const int TBg = wide ? PlanTmaB13High::TB : TB, box = TBg - (G.comp ? 1 : 0);
+    CK(make_tile_map(&P.map_psi, state, m, box, h, c, 8, 128), "tensor map (psi)");
+    CK(make_tile_map(&P.map_lam, lam, m, box, h, c, 8, 128), "tensor map (lambda)");
     P.psi = reinterpret_cast<float2 *>(state);
     P.lam = reinterpret_cast<float2 *>(lam);
-    if (wide)
-      CK(make_tile_map(&P.map_cost, const_cast<void *>(cost), n, TBg, h, c, (int)cost_bytes(ct), 0),
-         "tensor map (cost)");
-    else if (G.cl && op.lp >= 0)
+    if (G.cl && !wide && op.lp >= 0)
       CK(make_pair_cost_map(&P.map_cost, const_cast<void *>(cost), n, h, (int)cost_bytes(ct)),
          "tensor map (pair cost)");
     else
-      CK(make_tile_map(&P.map_cost, const_cast<void *>(cost), n, TB, h, c, (int)cost_bytes(ct), 0),
+      CK(make_tile_map(&P.map_cost, const_cast<void *>(cost), m, box, h, c, (int)cost_bytes(ct), 0),
          "tensor map (cost)");
-    P.ntiles = 1ull << (n - TBg);
+    P.ntiles = 1ull << (m - TBg);
     P.h = h;
     P.c = c;
+    P.mid2 = tile_map_mid2(box, c);
+    P.comp = G.comp ? m : 0;
+    P.out_scale = half ? 4.0 : 2.0;
     P.cost_kind = cost_kind(ct);
     // A cluster pair rotates tile bits 8..11 in round 0 (layout L0), tile
     // bits 4..7 in round 1's registers and tile bit 12 at its lane bit 4
@@ -962,9 +1067,14 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
     pair_sweep.m[1] = (uint8_t)((G.rot >> 4) & 0xFu);
     pair_sweep.lm[1] = (uint8_t)(((G.rot >> TB) & 1u) << 4);
     P.cluster = wide ? 2 : G.cl ? 1 : 0;
-    P.s1 = wide   ? make_sweep<PlanTmaB13High>(G.rot, true)
-           : G.cl ? pair_sweep
-           : G.high ? make_sweep<High>(G.rot, true) : make_sweep<Low>(G.rot, true);
+    auto sweep = [&](bool up) {
+      return wide && G.comp ? make_sweep<PlanTmaB13Comp>(G.rot, up)
+             : wide         ? make_sweep<PlanTmaB13High>(G.rot, up)
+             : G.cl         ? pair_sweep
+             : G.high       ? make_sweep<High>(G.rot, up)
+                            : make_sweep<Low>(G.rot, up);
+    };
+    P.s1 = sweep(true);
     {
       const TanRot R = tan_rot(bet[op.l1], true);
       P.tau1 = R.tau;
@@ -987,9 +1097,7 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
       P.out_g = d_grad_g + op.lp;
     }
     if (op.l2 >= 0) {
-      P.s2 = wide   ? make_sweep<PlanTmaB13High>(G.rot, false)
-             : G.cl ? pair_sweep
-             : G.high ? make_sweep<High>(G.rot, false) : make_sweep<Low>(G.rot, false);
+      P.s2 = sweep(false);
       const TanRot R = tan_rot(bet[op.l2], true);
       P.tau2 = R.tau;
       P.form2 = R.form;
@@ -1004,13 +1112,14 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
       return fail(QAOA_ERR_INVALID_ARG, "internal: plan needs lane rotations");
     P.init_lambda = op.init;
     P.untwist = &op == &ops.back();
+    if (half && P.untwist) P.mirror = (1ull << n) - 1ull;
     P.partials = ws.partials;
     P.counter = ws.counter;
     P.err = ws.err;
-    const double N = (double)(1ull << n);
+    const double N = (double)(1ull << m);
     // psi and lambda read and written (lambda not read by the first pass, not
     // written by the last), plus the cost vector where the pass reads it
-    const double bytes = (32.0 - (P.init_lambda ? 8.0 : 0.0) - (P.untwist ? 8.0 : 0.0)) * N +
+    const double bytes = (32.0 - (P.init_lambda ? 8.0 : 0.0) - (P.untwist ? 8.0 : 0.0) + (P.mirror ? 8.0 : 0.0)) * N +
                          ((P.has_phase || P.init_lambda) ? cost_bytes(ct) * N : 0.0);
     const int kind = (P.has_phase ? 2 : 0) | (op.l2 >= 0 ? 4 : 0) | (P.init_lambda ? 8 : 0);
     LAUNCH_N(tma_pass_name(false, wide ? 3 : G.cl ? 2 : G.high ? 1 : 0, kind), bytes, s,
@@ -1322,7 +1431,7 @@ qaoa_status qaoa_cost_stats_compute(int n, const void *d_costs, qaoa_cost_type c
   CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
   LAUNCH("cost_stats", cost_bytes(ct) * (double)(1ull << n), s,
          launch_cost_stats(n, d_costs, cost_kind(ct), ws.partials, ws.counter, ws.small, s, num_sms()));
-  double h[4];
+  double h[5];
   CK(cudaMemcpyAsync(h, ws.small, sizeof(h), cudaMemcpyDeviceToHost, s), "cost stats copy");
   CK(cudaStreamSynchronize(s), "cost stats sync");
   h_out->f_min = h[0];
@@ -1331,6 +1440,7 @@ qaoa_status qaoa_cost_stats_compute(int n, const void *d_costs, qaoa_cost_type c
   const uint32_t bits = (uint32_t)h[3];
   h_out->step_log2 = bits ? (uint32_t)__builtin_ctz(bits) : 0u;
   h_out->reserved = 0u;
+  if (h[4] != 0.0) h_out->reserved = comp_mark(n, h_out);
   return QAOA_OK;
 }
 
@@ -1354,11 +1464,13 @@ qaoa_status qaoa_simulate(int n, const void *d_costs, qaoa_cost_type ct, const q
                : small_forward<double>(n, d_costs, ct, stats->f_min, gammas, betas, p, d_state, init_plus, d_out, s);
   }
   CK(cudaMemsetAsync(ws.err, 0, sizeof(unsigned), s), "memset error word");
+  const bool half = half_vector(n, st, stats, init_plus);
   if (st == QAOA_C64 && tma_ok(ct))
-    return tma_forward(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws, d_out, true, s);
-  return st == QAOA_C64
-             ? tiled_forward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws, d_out, s)
-             : tiled_forward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws, d_out, s);
+    return tma_forward(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws, d_out, true, half, s);
+  return st == QAOA_C64 ? tiled_forward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws,
+                                               d_out, half, true, s)
+                        : tiled_forward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws,
+                                                d_out, half, true, s);
 }
 
 // ------------------------------------------------------------- XY mixers
@@ -1677,21 +1789,24 @@ qaoa_status qaoa_grad(int n, const void *d_costs, qaoa_cost_type ct, const qaoa_
   }
   CK(cudaMemsetAsync(d_out + 2, 0, sizeof(double) * 2 * (size_t)p, s), "memset grad");
   CK(cudaMemsetAsync(ws.err, 0, sizeof(unsigned), s), "memset error word");
+  bool half = half_vector(n, st, stats, 1);
   if (st == QAOA_C64 && tma_ok(ct)) {
-    r = tma_forward(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, false, s);
+    half = half && !adjoint_override();
+    r = tma_forward(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, false, half, s);
     if (r != QAOA_OK) return r;
     return tma_backward(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws, d_out + 2,
-                        d_out + 2 + p, s);
+                        d_out + 2 + p, half, s);
   }
-  r = st == QAOA_C64
-          ? tiled_forward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, s)
-          : tiled_forward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, s);
+  r = st == QAOA_C64 ? tiled_forward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, half,
+                                            false, s)
+                     : tiled_forward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, half,
+                                             false, s);
   if (r != QAOA_OK) return r;
   return st == QAOA_C64
              ? tiled_backward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws,
-                                     d_out + 2, d_out + 2 + p, s)
+                                     d_out + 2, d_out + 2 + p, half, s)
              : tiled_backward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws,
-                                      d_out + 2, d_out + 2 + p, s);
+                                      d_out + 2, d_out + 2 + p, half, s);
 }
 
 }  // extern "C"

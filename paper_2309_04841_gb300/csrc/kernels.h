@@ -77,6 +77,25 @@ static_assert(PlanTmaB12Low::valid() && PlanTmaB12High::valid(), "bad TMA B12 pl
 // round 1 tile bits 4-7 and tile bit 12 as lane bit 4 (a shuffle rotation).
 using PlanTmaB13High = Plan<13, 4, 512, 0, 2, 0x0F00, 0x001F, 0x10E0, 0x00F0, 0x100F, 0x0F00>;
 static_assert(PlanTmaB13High::valid(), "bad TMA B13 plan");
+// The same group with a complement pair (below): tile bit 12 in registers in
+// round 0 and a warp bit in round 1, tile bit 8 the lane rotation of round 1.
+using PlanTmaB13Comp = Plan<13, 4, 512, 0, 2, 0x1E00, 0x001F, 0x01E0, 0x00F0, 0x010F, 0x1E00>;
+static_assert(PlanTmaB13Comp::valid(), "bad TMA B13 complement plan");
+// Complement pairs: on a cost vector with f(x) = f(~x) the state keeps
+// psi(x) = psi(~x), so the passes hold the 2^(n-1) amplitudes with the top
+// qubit 0 (m = n - 1 index bits).  The rotation of the top qubit pairs x with
+// its m-bit complement.  The one group that carries it has tiles of two boxes,
+// T and ~T, of 2^(TB-1) amplitudes: tile bit TB - 1 selects the box, and tile
+// offset t of box 1 is the amplitude ~x of the x at offset t of box 0.  The
+// shared-memory slot of (box 1, t) is the bitwise complement of t, a constant
+// XOR, so the loads stay two plain boxes.  Tile bit TB - 1 must be the last
+// register bit of round 0 and a warp bit of round 1.
+template <class PL>
+constexpr bool comp_plan() {
+  return PL::NR == 2 && (PL::reg(0) >> (PL::TB - 1)) == 1u && (PL::warp(1) >> (PL::TB - 1)) == 1u;
+}
+static_assert(comp_plan<PlanTmaF13High>() && comp_plan<PlanTmaB12High>() && comp_plan<PlanTmaB13Comp>(),
+              "complement tile bit: last register bit of round 0, warp bit of round 1");
 
 // The TMA passes hold vectors in the twisted basis s(x) = (-i)^popc(x) psi(x),
 // where exp(-i b X_q) acts on a pair as the real rotation
@@ -118,6 +137,8 @@ struct alignas(64) TmaFwdParams {
   float2 *psi;           // the state (finished tiles are stored from registers)
   uint64_t ntiles;
   int h, c, cost_kind;  // tile = 2^c contiguous amplitudes x rows at qubits h..
+  int mid2;             // the outer bits c..h-1 are view dimension 2 (else 1), see make_tile_map
+  int comp;             // complement pair: the index bits m of the half vector, else 0
   Sweep s1, s2;
   float tau1, tau2;
   int form1, form2;
@@ -126,6 +147,8 @@ struct alignas(64) TmaFwdParams {
   int has_phase, init_plus, reduce;
   int twist_in;  // first pass on a caller's state: into the twisted basis
   int untwist;   // last pass (with end_scale): back to the standard basis
+  uint64_t mirror;   // with untwist, nonzero (2^n - 1): amplitude x is also stored at its complement
+  double out_scale;  // E and O times this (2 where half of the amplitudes are held)
   float amp;
   uint32_t fmin_word;  // f_min as the cost vector stores it (int32 or float32 bits)
   double *partials;
@@ -140,6 +163,7 @@ struct alignas(64) TmaBwdParams {
   float2 *psi, *lam;                       // stores, from registers
   uint64_t ntiles;
   int h, c, cost_kind;
+  int mid2, comp;     // as in TmaFwdParams
   Sweep s1, s2;
   float tau1, tau2;
   int form1, form2;
@@ -148,6 +172,8 @@ struct alignas(64) TmaBwdParams {
   float wg;           // |scale|^2 weight of the d/d gamma inner product
   int has_phase, init_lambda;
   int untwist;  // last pass: psi back to the standard basis, lambda not stored
+  uint64_t mirror;   // with untwist, nonzero (2^n - 1): psi[x] is also stored at its complement
+  double out_scale;  // inner products times this before they are added
   // HIGH group of 9 new qubits (c = 4) on a 2^13-amplitude tile: 1 = cluster
   // pair, two CTAs holding its two halves (k_bwd_pair; map_cost is then the
   // pair cost map of the phase layout for passes with a phase); 2 = one
@@ -160,6 +186,9 @@ struct alignas(64) TmaBwdParams {
   PhaseDigits ph;
 };
 
+// The tile view whose outer bits c..h-1 are dimension 2 (else dimension 1): segments
+// of 32 amplitudes and more, and tiles of fewer than 256 rows.
+constexpr bool tile_map_mid2(int tb, int c) { return c >= 5 || tb - c < 8; }
 cudaError_t make_tile_map(CUtensorMap *map, void *base, int n, int tb, int h, int c, int esz,
                           int swizzle_bytes);
 // Cost tile of one CTA of a pair in the phase layout: 16 contiguous elements

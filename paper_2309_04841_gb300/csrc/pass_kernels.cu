@@ -235,44 +235,75 @@ __device__ __forceinline__ double2 phase_factor(const PhaseData<double> &ph, con
   return make_double2(cs * ph.scl, -sn * ph.scl);
 }
 
-template <class PL, int R, typename Real, typename C2>
+// Index of this thread's amplitude in register r of round R of the tile at
+// `base`: base + offset, and in box 1 of a complement pair (CP) the complement
+// of that.  The box bit is a register bit (a constant of r) or a thread bit.
+template <class PL, int R, bool CP>
+struct AmpIndex {
+  static constexpr uint32_t TOP = CP ? 1u << (PL::TB - 1) : 0u;
+  const Geom &g;
+  uint64_t xt;
+  bool neg = false;
+  __device__ __forceinline__ AmpIndex(const Geom &g_, uint64_t base) : g(g_) {
+    const uint32_t t = thr_toff<PL, R>();
+    xt = base + tile_off(g, t & ~TOP);
+    if constexpr (CP && (PL::reg(R) & TOP) == 0u) {
+      neg = (t & TOP) != 0u;
+      if (neg) xt = g.comp - xt;
+    }
+  }
+  __device__ __forceinline__ uint64_t at(int r) const {
+    const uint32_t t = pdep(r, PL::reg(R));
+    const uint64_t off = tile_off(g, t & ~TOP);
+    if constexpr (!CP) return xt + off;
+    if constexpr ((PL::reg(R) & TOP) != 0u) return (t & TOP) ? g.comp - (xt + off) : xt + off;
+    return neg ? xt - off : xt + off;
+  }
+};
+
+template <class PL, int R, bool CP, typename Real, typename C2>
 __device__ __forceinline__ void apply_phase(C2 (&v)[PL::NREG], const PhaseData<Real> &ph,
                                             const C2 *tlo, const C2 *thi, const void *cost,
                                             int kind, const Geom &g, uint64_t base) {
-  const uint64_t xt = base + tile_off(g, thr_toff<PL, R>());
+  const AmpIndex<PL, R, CP> ix(g, base);
 #pragma unroll
   for (int r = 0; r < PL::NREG; ++r) {
-    const uint64_t x = xt + tile_off(g, pdep(r, PL::reg(R)));
+    const uint64_t x = ix.at(r);
     v[r] = cmul(v[r], phase_factor(ph, tlo, thi, cost, kind, x));
   }
 }
 
-template <class PL, int R, typename C2>
+template <class PL, int R, bool CP, typename C2>
 __device__ __forceinline__ void load_tile(C2 (&v)[PL::NREG], const C2 *__restrict__ src,
                                           const Geom &g, uint64_t base) {
-  const uint64_t xt = base + tile_off(g, thr_toff<PL, R>());
+  const AmpIndex<PL, R, CP> ix(g, base);
 #pragma unroll
-  for (int r = 0; r < PL::NREG; ++r) v[r] = src[xt + tile_off(g, pdep(r, PL::reg(R)))];
+  for (int r = 0; r < PL::NREG; ++r) v[r] = src[ix.at(r)];
 }
 
-template <class PL, int R, typename C2>
+// mirror nonzero (2^n - 1): every amplitude is also stored at its complement.
+template <class PL, int R, bool CP, typename C2>
 __device__ __forceinline__ void store_tile(const C2 (&v)[PL::NREG], C2 *__restrict__ dst,
-                                           const Geom &g, uint64_t base) {
-  const uint64_t xt = base + tile_off(g, thr_toff<PL, R>());
+                                           const Geom &g, uint64_t base, uint64_t mirror = 0) {
+  const AmpIndex<PL, R, CP> ix(g, base);
 #pragma unroll
-  for (int r = 0; r < PL::NREG; ++r) dst[xt + tile_off(g, pdep(r, PL::reg(R)))] = v[r];
+  for (int r = 0; r < PL::NREG; ++r) dst[ix.at(r)] = v[r];
+  if (mirror) {
+#pragma unroll
+    for (int r = 0; r < PL::NREG; ++r) dst[mirror - ix.at(r)] = v[r];
+  }
 }
 
 // Energy and overlap terms of this thread's amplitudes in round-R layout.
-template <class PL, int R, typename C2>
+template <class PL, int R, bool CP, typename C2>
 __device__ __forceinline__ void accum_eo(const C2 (&v)[PL::NREG], const void *cost, int kind,
                                          double fmin, const Geom &g, uint64_t base,
                                          typename Scal<C2>::R &e, typename Scal<C2>::R &o) {
   using Real = typename Scal<C2>::R;
-  const uint64_t xt = base + tile_off(g, thr_toff<PL, R>());
+  const AmpIndex<PL, R, CP> ix(g, base);
 #pragma unroll
   for (int r = 0; r < PL::NREG; ++r) {
-    const uint64_t x = xt + tile_off(g, pdep(r, PL::reg(R)));
+    const uint64_t x = ix.at(r);
     const double f = cost_d(cost, kind, x);
     const Real pr = v[r].x * v[r].x + v[r].y * v[r].y;
     e += pr * (Real)f;
@@ -337,7 +368,7 @@ __device__ __forceinline__ void last_block_reduce(const double *partials, uint64
 
 // ------------------------------------------------------------ forward pass
 
-template <class PL, typename Real>
+template <class PL, typename Real, bool CP>
 __global__ void __launch_bounds__(PL::NT, 2) k_fwd(const __grid_constant__ FwdParams<Real> P) {
   using C2 = typename C2T<Real>::type;
   constexpr int NREG = PL::NREG, NR = PL::NR, EB = PL::EB;
@@ -365,7 +396,7 @@ __global__ void __launch_bounds__(PL::NT, 2) k_fwd(const __grid_constant__ FwdPa
 #pragma unroll
       for (int r = 0; r < NREG; ++r) v[r] = mk<C2>(P.amp, (Real)0);
     } else {
-      load_tile<PL, 0>(v, P.psi, g, base);
+      load_tile<PL, 0, CP>(v, P.psi, g, base);
     }
     bool final0;
     if (has1) {
@@ -376,7 +407,7 @@ __global__ void __launch_bounds__(PL::NT, 2) k_fwd(const __grid_constant__ FwdPa
         xpose<PL, 1, 2>(v, tile);
         rot_regs<EB>(v, P.s1.m[2], P.t1, P.form1);
       }
-      if (P.has_phase) apply_phase<PL, NR - 1>(v, P.ph, tlo, thi, P.cost, P.cost_kind, g, base);
+      if (P.has_phase) apply_phase<PL, NR - 1, CP>(v, P.ph, tlo, thi, P.cost, P.cost_kind, g, base);
       if (has2) {
         rot_regs<EB>(v, P.s2.m[NR - 1], P.t2, P.form2);
         if constexpr (NR == 3) {
@@ -390,7 +421,7 @@ __global__ void __launch_bounds__(PL::NT, 2) k_fwd(const __grid_constant__ FwdPa
         final0 = false;
       }
     } else {
-      if (P.has_phase) apply_phase<PL, 0>(v, P.ph, tlo, thi, P.cost, P.cost_kind, g, base);
+      if (P.has_phase) apply_phase<PL, 0, CP>(v, P.ph, tlo, thi, P.cost, P.cost_kind, g, base);
       rot_regs<EB>(v, P.s2.m[0], P.t2, P.form2);
       xpose<PL, 0, 1>(v, tile);
       rot_regs<EB>(v, P.s2.m[1], P.t2, P.form2);
@@ -407,9 +438,9 @@ __global__ void __launch_bounds__(PL::NT, 2) k_fwd(const __grid_constant__ FwdPa
     if (P.reduce) {
       Real e = 0, o = 0;
       if (final0)
-        accum_eo<PL, 0>(v, P.cost, P.cost_kind, P.fmin_d, g, base, e, o);
+        accum_eo<PL, 0, CP>(v, P.cost, P.cost_kind, P.fmin_d, g, base, e, o);
       else
-        accum_eo<PL, NR - 1>(v, P.cost, P.cost_kind, P.fmin_d, g, base, e, o);
+        accum_eo<PL, NR - 1, CP>(v, P.cost, P.cost_kind, P.fmin_d, g, base, e, o);
       double a[2] = {(double)e, (double)o};
       block_sum<PL::NT, 2>(a, red);
       if (threadIdx.x == 0) {
@@ -418,22 +449,23 @@ __global__ void __launch_bounds__(PL::NT, 2) k_fwd(const __grid_constant__ FwdPa
       }
     }
     if (final0)
-      store_tile<PL, 0>(v, P.psi, g, base);
+      store_tile<PL, 0, CP>(v, P.psi, g, base, P.mirror);
     else
-      store_tile<PL, NR - 1>(v, P.psi, g, base);
+      store_tile<PL, NR - 1, CP>(v, P.psi, g, base, P.mirror);
   }
   if (P.reduce) {
     double *out = P.out;
-    last_block_reduce<PL::NT, 2>(P.partials, g.ntiles, P.counter, red, [out](double(&a)[2]) {
-      out[0] = a[0];
-      out[1] = a[1];
+    const double sc = P.out_scale;
+    last_block_reduce<PL::NT, 2>(P.partials, g.ntiles, P.counter, red, [out, sc](double(&a)[2]) {
+      out[0] = sc * a[0];
+      out[1] = sc * a[1];
     });
   }
 }
 
 // ----------------------------------------------------------- backward pass
 
-template <class PL, typename Real>
+template <class PL, typename Real, bool CP>
 __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdParams<Real> P) {
   using C2 = typename C2T<Real>::type;
   constexpr int NREG = PL::NREG, NR = PL::NR, EB = PL::EB;
@@ -458,17 +490,17 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
     const uint64_t base = tile_base(g, T);
     __syncthreads();
     C2 v[NREG], w[NREG];
-    load_tile<PL, 0>(v, P.psi, g, base);
+    load_tile<PL, 0, CP>(v, P.psi, g, base);
     if (P.init_lambda) {
       // lambda = f psi: the gradient of E = <psi|f|psi> with respect to psi^*
-      const uint64_t xt = base + tile_off(g, thr_toff<PL, 0>());
+      const AmpIndex<PL, 0, CP> ix(g, base);
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
-        const Real f = (Real)cost_d(P.cost, P.cost_kind, xt + tile_off(g, pdep(r, PL::reg(0))));
+        const Real f = (Real)cost_d(P.cost, P.cost_kind, ix.at(r));
         w[r] = mk<C2>(f * v[r].x, f * v[r].y);
       }
     } else {
-      load_tile<PL, 0>(w, P.lam, g, base);
+      load_tile<PL, 0, CP>(w, P.lam, g, base);
     }
     Real a1 = 0, ag = 0, a2 = 0;
     // sweep 1 ascending through the rounds
@@ -481,11 +513,11 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
     }
     if (P.has_phase) {
       // d/d gamma: Im <lambda| f |psi>, then un-phase both vectors
-      const uint64_t xt = base + tile_off(g, thr_toff<PL, NR - 1>());
+      const AmpIndex<PL, NR - 1, CP> ix(g, base);
       Real raw = 0;
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
-        const uint64_t x = xt + tile_off(g, pdep(r, PL::reg(NR - 1)));
+        const uint64_t x = ix.at(r);
         const Real f = (Real)cost_d(P.cost, P.cost_kind, x);
         raw += f * (w[r].x * v[r].y - w[r].y * v[r].x);
         const C2 ph = phase_factor(P.ph, tlo, thi, P.cost, P.cost_kind, x);
@@ -521,18 +553,19 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
       }
     }
     if (final0) {
-      store_tile<PL, 0>(v, P.psi, g, base);
-      store_tile<PL, 0>(w, P.lam, g, base);
+      store_tile<PL, 0, CP>(v, P.psi, g, base, P.mirror);
+      store_tile<PL, 0, CP>(w, P.lam, g, base);
     } else {
-      store_tile<PL, NR - 1>(v, P.psi, g, base);
-      store_tile<PL, NR - 1>(w, P.lam, g, base);
+      store_tile<PL, NR - 1, CP>(v, P.psi, g, base, P.mirror);
+      store_tile<PL, NR - 1, CP>(w, P.lam, g, base);
     }
   }
   double *o1 = P.out_b1, *og = P.out_g, *o2 = P.out_b2;
+  const double sc = P.out_scale;
   last_block_reduce<PL::NT, 3>(P.partials, g.ntiles, P.counter, red, [=](double(&a)[3]) {
-    if (o1) *o1 += 2.0 * a[0];
-    if (og) *og += 2.0 * a[1];
-    if (o2) *o2 += 2.0 * a[2];
+    if (o1) *o1 += sc * a[0];
+    if (og) *og += sc * a[1];
+    if (o2) *o2 += sc * a[2];
   });
 }
 
@@ -545,11 +578,11 @@ static int blocks_per_sm(K kernel, int nt, size_t smem) {
   return nb < 1 ? 1 : nb;
 }
 
-template <class PL, typename Real>
+template <class PL, typename Real, bool CP = false>
 static cudaError_t launch_fwd_t(const FwdParams<Real> &P, cudaStream_t s, int nsm) {
   using C2 = typename C2T<Real>::type;
   const size_t smem = ((size_t)(1 << PL::TB) + 512) * sizeof(C2) + (PL::NT / 32) * 3 * sizeof(double);
-  auto kern = k_fwd<PL, Real>;
+  auto kern = k_fwd<PL, Real, CP>;
   static int nb = -1;  // per instantiation; the device is fixed per process
   if (nb < 0) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -562,11 +595,11 @@ static cudaError_t launch_fwd_t(const FwdParams<Real> &P, cudaStream_t s, int ns
   return cudaGetLastError();
 }
 
-template <class PL, typename Real>
+template <class PL, typename Real, bool CP = false>
 static cudaError_t launch_bwd_t(const BwdParams<Real> &P, cudaStream_t s, int nsm) {
   using C2 = typename C2T<Real>::type;
   const size_t smem = ((size_t)(2 << PL::TB) + 512) * sizeof(C2) + (PL::NT / 32) * 3 * sizeof(double);
-  auto kern = k_bwd<PL, Real>;
+  auto kern = k_bwd<PL, Real, CP>;
   static int nb = -1;
   if (nb < 0) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -579,36 +612,40 @@ static cudaError_t launch_bwd_t(const BwdParams<Real> &P, cudaStream_t s, int ns
   return cudaGetLastError();
 }
 
+// LOW pass, HIGH pass, or HIGH pass on complement-pair tiles.
+template <class Low, class High, typename Real>
+static cudaError_t dispatch_fwd(const FwdParams<Real> &P, bool high, cudaStream_t s, int nsm) {
+  if (!high) return P.g.comp ? cudaErrorInvalidValue : launch_fwd_t<Low, Real>(P, s, nsm);
+  return P.g.comp ? launch_fwd_t<High, Real, true>(P, s, nsm) : launch_fwd_t<High, Real>(P, s, nsm);
+}
+template <class Low, class High, typename Real>
+static cudaError_t dispatch_bwd(const BwdParams<Real> &P, bool high, cudaStream_t s, int nsm) {
+  if (!high) return P.g.comp ? cudaErrorInvalidValue : launch_bwd_t<Low, Real>(P, s, nsm);
+  return P.g.comp ? launch_bwd_t<High, Real, true>(P, s, nsm) : launch_bwd_t<High, Real>(P, s, nsm);
+}
+
 cudaError_t launch_fwd(const FwdParams<float> &P, bool high, int tb, cudaStream_t s, int nsm) {
   if (tb != PlanF13Low::TB) return cudaErrorInvalidValue;
-  return high ? launch_fwd_t<PlanF13High, float>(P, s, nsm) : launch_fwd_t<PlanF13Low, float>(P, s, nsm);
+  return dispatch_fwd<PlanF13Low, PlanF13High>(P, high, s, nsm);
 }
 cudaError_t launch_fwd(const FwdParams<double> &P, bool high, int tb, cudaStream_t s, int nsm) {
   switch (tb) {
-    case 9:
-      return high ? launch_fwd_t<PlanT9High, double>(P, s, nsm) : launch_fwd_t<PlanT9Low, double>(P, s, nsm);
-    case 10:
-      return high ? launch_fwd_t<PlanT10High, double>(P, s, nsm) : launch_fwd_t<PlanT10Low, double>(P, s, nsm);
-    case 12:
-      return high ? launch_fwd_t<PlanT12High, double>(P, s, nsm) : launch_fwd_t<PlanT12Low, double>(P, s, nsm);
-    default:
-      return cudaErrorInvalidValue;
+    case 9: return dispatch_fwd<PlanT9Low, PlanT9High>(P, high, s, nsm);
+    case 10: return dispatch_fwd<PlanT10Low, PlanT10High>(P, high, s, nsm);
+    case 12: return dispatch_fwd<PlanT12Low, PlanT12High>(P, high, s, nsm);
+    default: return cudaErrorInvalidValue;
   }
 }
 cudaError_t launch_bwd(const BwdParams<float> &P, bool high, int tb, cudaStream_t s, int nsm) {
   if (tb != PlanT12Low::TB) return cudaErrorInvalidValue;
-  return high ? launch_bwd_t<PlanT12High, float>(P, s, nsm) : launch_bwd_t<PlanT12Low, float>(P, s, nsm);
+  return dispatch_bwd<PlanT12Low, PlanT12High>(P, high, s, nsm);
 }
 cudaError_t launch_bwd(const BwdParams<double> &P, bool high, int tb, cudaStream_t s, int nsm) {
   switch (tb) {
-    case 9:
-      return high ? launch_bwd_t<PlanT9High, double>(P, s, nsm) : launch_bwd_t<PlanT9Low, double>(P, s, nsm);
-    case 10:
-      return high ? launch_bwd_t<PlanT10High, double>(P, s, nsm) : launch_bwd_t<PlanT10Low, double>(P, s, nsm);
-    case 11:
-      return high ? launch_bwd_t<PlanT11High, double>(P, s, nsm) : launch_bwd_t<PlanT11Low, double>(P, s, nsm);
-    default:
-      return cudaErrorInvalidValue;
+    case 9: return dispatch_bwd<PlanT9Low, PlanT9High>(P, high, s, nsm);
+    case 10: return dispatch_bwd<PlanT10Low, PlanT10High>(P, high, s, nsm);
+    case 11: return dispatch_bwd<PlanT11Low, PlanT11High>(P, high, s, nsm);
+    default: return cudaErrorInvalidValue;
   }
 }
 

@@ -110,17 +110,22 @@ constexpr int kHighC = 4;
 
 enum CostKind : int { kCostI32 = 0, kCostF32 = 1, kCostF64 = 2, kCostU16 = 3 };
 
-// Tile geometry of one pass (see file comment).
+// Tile geometry of one pass (see file comment).  A complement pair (comp != 0,
+// the all-ones mask of the vector's index): tile bit tb - 1 is no index bit but
+// selects one of two boxes of 2^(tb-1) amplitudes, tile offset t with that bit
+// set being the amplitude whose index is the complement of the one at t without
+// it, so the rotation that pairs x with ~x acts on that tile bit.
 struct Geom {
   int n, c, h, tb;
   uint64_t ntiles;
+  uint64_t comp;
 };
 
 __device__ __forceinline__ uint64_t tile_base(const Geom &g, uint64_t T) {
   const int mid = g.h - g.c;  // outer bits between the two segments
   const uint64_t lo = T & ((1ull << mid) - 1ull);
   const uint64_t hi = T >> mid;
-  return (lo << g.c) | (hi << (g.h + g.tb - g.c));
+  return (lo << g.c) | (hi << (g.h + g.tb - g.c - (g.comp ? 1 : 0)));
 }
 
 __device__ __forceinline__ uint64_t tile_off(const Geom &g, uint32_t t) {
@@ -174,6 +179,8 @@ struct FwdParams {
   double *partials;     // [ntiles][2]
   unsigned *counter;
   double *out;          // [2]: E, O
+  double out_scale;     // E and O times this (2 where half of the amplitudes are held)
+  uint64_t mirror;      // nonzero (2^n - 1): amplitude x is also stored at its complement
   PhaseData<Real> ph;
 };
 
@@ -197,6 +204,8 @@ struct BwdParams {
   double *partials;       // [ntiles][3]
   unsigned *counter;
   double *out_b1, *out_g, *out_b2;  // gradient slots (accumulated: +=)
+  double out_scale;       // inner products times this before they are added
+  uint64_t mirror;        // nonzero (2^n - 1): psi[x] is also stored at its complement
   PhaseData<Real> ph;     // un-phase data (exp(+i g f))
 };
 

@@ -247,6 +247,107 @@ __device__ __forceinline__ void rot_tw(float2 (&v)[1 << EB], uint32_t m, float t
   }
 }
 
+// ---- complement pairs
+// Box 1 of a tile holds the amplitude ~x at the offset of x, so the members of
+// a pair change roles there: its rotations run with the angle negated.  The
+// rotation that pairs x (box 0) with ~x (box 1) is, in the twisted basis, with
+// k = popc(x) and kappa = i^(m-1) (-1)^k,
+//   m odd:   (a, b) <- (a + t kappa b, b - t kappa a),  kappa = eps = +-1
+//   m even:  (a, b) <- (a + t kappa b, b + t kappa a),  kappa = i eps
+// and Im <lambda| X |psi> of the pair is eps (l_a . s_b - l_b . s_a), or
+// -eps Im(conj(l_a) s_b + conj(l_b) s_a).  eps here is this thread's sign for
+// register 0 of round 0 (the register's own parity is a constant).
+struct CompCtx {
+  float eps = 1.f;
+  bool odd = false, box1 = false;  // box1: this thread's amplitudes of round 1 are in box 1
+};
+
+// rot_tw on a round of a complement-pair tile: UB >= 0, the box is register
+// bit UB (left to rot_comp); UB = -1, the whole thread is in one box.
+template <int EB, int UB>
+__device__ __forceinline__ void rot_tw_comp(float2 (&v)[1 << EB], uint32_t m, float tau, int form, bool box1) {
+  if (form == 0) {
+    const float ts = UB < 0 && box1 ? -tau : tau;
+    const float2 tp = f2(ts, ts), tn = f2(-ts, -ts);
+#pragma unroll
+    for (int i = 0; i < EB; ++i)
+      if (i != UB && ((m >> i) & 1u)) {
+#pragma unroll
+        for (int r = 0; r < (1 << EB); ++r)
+          if (!((r >> i) & 1)) {
+            const bool rev = UB >= 0 && ((r >> (UB < 0 ? 0 : UB)) & 1);
+            const float2 a = v[r], b = v[r | (1 << i)];
+            v[r] = __ffma2_rn(rev ? tn : tp, b, a);
+            v[r | (1 << i)] = __ffma2_rn(rev ? tp : tn, a, b);
+          }
+      }
+  } else {
+    const float2 tp = f2(tau, tau);
+    auto sweep = [&](bool all_rev) {
+#pragma unroll
+      for (int i = 0; i < EB; ++i)
+        if (i != UB && ((m >> i) & 1u)) {
+#pragma unroll
+          for (int r = 0; r < (1 << EB); ++r)
+            if (!((r >> i) & 1)) {
+              const bool rev = UB >= 0 ? ((r >> (UB < 0 ? 0 : UB)) & 1) != 0 : all_rev;
+              const float2 a = v[r], b = v[r | (1 << i)];
+              v[r] = __ffma2_rn(tp, a, rev ? f2(-b.x, -b.y) : b);
+              v[r | (1 << i)] = __ffma2_rn(tp, b, rev ? a : f2(-a.x, -a.y));
+            }
+        }
+    };
+    if (UB < 0 && box1)
+      sweep(true);
+    else
+      sweep(false);
+  }
+}
+
+// The rotation of the pairs (x, ~x): register bit UB.
+template <int EB, int UB>
+__device__ __forceinline__ void rot_comp(float2 (&v)[1 << EB], float tau, int form, const CompCtx &cx) {
+#pragma unroll
+  for (int r = 0; r < (1 << EB); ++r)
+    if (!((r >> UB) & 1)) {
+      const float e = (popc_c(r) & 1) ? -cx.eps : cx.eps;
+      const float2 a = v[r], b = v[r | (1 << UB)];
+      if (cx.odd) {
+        if (form == 0) {
+          v[r] = __ffma2_rn(f2(e * tau, e * tau), b, a);
+          v[r | (1 << UB)] = __ffma2_rn(f2(-e * tau, -e * tau), a, b);
+        } else {
+          v[r] = __ffma2_rn(f2(tau, tau), a, f2(e * b.x, e * b.y));
+          v[r | (1 << UB)] = __ffma2_rn(f2(tau, tau), b, f2(-e * a.x, -e * a.y));
+        }
+      } else {
+        const float et = e * tau;
+        if (form == 0) {
+          v[r] = f2(fmaf(-et, b.y, a.x), fmaf(et, b.x, a.y));
+          v[r | (1 << UB)] = f2(fmaf(-et, a.y, b.x), fmaf(et, a.x, b.y));
+        } else {
+          v[r] = f2(fmaf(tau, a.x, -e * b.y), fmaf(tau, a.y, e * b.x));
+          v[r | (1 << UB)] = f2(fmaf(tau, b.x, -e * a.y), fmaf(tau, b.y, e * a.x));
+        }
+      }
+    }
+}
+
+// Rotations of round R of a forward pass.
+template <class PL, int R, bool CP>
+__device__ __forceinline__ void rot_round(float2 (&v)[PL::NREG], uint32_t m, float tau, int form,
+                                          const CompCtx &cx) {
+  if constexpr (!CP) {
+    rot_tw<PL::EB>(v, m, tau, form);
+  } else if constexpr (R == 0) {
+    constexpr int UB = PL::EB - 1;
+    rot_tw_comp<PL::EB, UB>(v, m, tau, form, false);
+    if ((m >> UB) & 1u) rot_comp<PL::EB, UB>(v, tau, form, cx);
+  } else {
+    rot_tw_comp<PL::EB, -1>(v, m, tau, form, cx.box1);
+  }
+}
+
 // Adjoint: un-rotation of psi (v) and lambda (w), adding first the raw
 // Im <lambda| X_q |psi> of each pair, which in the twisted basis is
 // lambda_a . psi_b - lambda_b . psi_a (real dot products of the complex
@@ -304,6 +405,91 @@ __device__ __forceinline__ void unrot_tw(float2 (&v)[1 << EB], float2 (&w)[1 << 
   rot_tw<EB>(w, m, tau, form);
 }
 
+// unrot_tw on a round of a complement-pair tile (UB as in rot_tw_comp).
+template <int EB, int UB, bool LANES>
+__device__ __forceinline__ void unrot_tw_comp(float2 (&v)[1 << EB], float2 (&w)[1 << EB], uint32_t m,
+                                              uint32_t lm, float tau, int form, float wr, float &acc,
+                                              const CompCtx &cx) {
+  if (m == 0u && (!LANES || lm == 0u)) return;
+  float2 pp[2] = {f2(0.f, 0.f), f2(0.f, 0.f)}, pm[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
+#pragma unroll
+  for (int i = 0; i < EB; ++i)
+    if (i != UB && ((m >> i) & 1u)) {
+#pragma unroll
+      for (int r = 0; r < (1 << EB); ++r)
+        if (!((r >> i) & 1)) {
+          const int k = (r >> (i == 0 ? 1 : 0)) & 1;
+          const bool rev = UB >= 0 && ((r >> (UB < 0 ? 0 : UB)) & 1);
+          const int a = rev ? r | (1 << i) : r, b = rev ? r : r | (1 << i);
+          pp[k] = __ffma2_rn(w[a], v[b], pp[k]);
+          pm[k] = __ffma2_rn(w[b], v[a], pm[k]);
+        }
+    }
+  const float2 sp = __fadd2_rn(pp[0], pp[1]), sm = __fadd2_rn(pm[0], pm[1]);
+  const float sgn = UB < 0 && cx.box1 ? -1.f : 1.f;
+  float term = sgn * ((sp.x + sp.y) - (sm.x + sm.y));
+  if constexpr (UB >= 0) {
+    if ((m >> UB) & 1u) {
+      float q[2] = {0.f, 0.f};  // by the register's parity
+#pragma unroll
+      for (int r = 0; r < (1 << EB); ++r)
+        if (!((r >> UB) & 1)) {
+          const int k = popc_c(r) & 1;
+          const float2 va = v[r], vb = v[r | (1 << UB)], wa = w[r], wb = w[r | (1 << UB)];
+          if (cx.odd)
+            q[k] += fmaf(wa.x, vb.x, wa.y * vb.y) - fmaf(wb.x, va.x, wb.y * va.y);
+          else
+            q[k] -= fmaf(wa.x, vb.y, -wa.y * vb.x) + fmaf(wb.x, va.y, -wb.y * va.x);
+        }
+      term = fmaf(cx.eps, q[0] - q[1], term);
+    }
+  }
+  float lane_term = 0.f;
+  if constexpr (LANES) {
+    if (lm != 0u) {
+      const int lb = __ffs((int)lm) - 1;
+      const float sg = ((threadIdx.x >> lb) & 1u) ? -sgn : sgn;  // sgn * (-1 for the pair's upper element)
+      const float2 st = f2(sg * tau, sg * tau), tt = f2(tau, tau);
+      float2 q = f2(0.f, 0.f);
+#pragma unroll
+      for (int r = 0; r < (1 << EB); ++r) {
+        const float2 pv = f2(__shfl_xor_sync(0xffffffffu, v[r].x, 1 << lb),
+                             __shfl_xor_sync(0xffffffffu, v[r].y, 1 << lb));
+        const float2 pw = f2(__shfl_xor_sync(0xffffffffu, w[r].x, 1 << lb),
+                             __shfl_xor_sync(0xffffffffu, w[r].y, 1 << lb));
+        q = __ffma2_rn(w[r], pv, q);
+        if (form == 0) {
+          v[r] = __ffma2_rn(st, pv, v[r]);
+          w[r] = __ffma2_rn(st, pw, w[r]);
+        } else {
+          v[r] = __ffma2_rn(tt, v[r], f2(sg * pv.x, sg * pv.y));
+          w[r] = __ffma2_rn(tt, w[r], f2(sg * pw.x, sg * pw.y));
+        }
+      }
+      lane_term = sg * (q.x + q.y);
+    }
+  }
+  acc = fmaf(term + lane_term, wr, acc);
+  rot_tw_comp<EB, UB>(v, m, tau, form, cx.box1);
+  rot_tw_comp<EB, UB>(w, m, tau, form, cx.box1);
+  if constexpr (UB >= 0) {
+    if ((m >> UB) & 1u) {
+      rot_comp<EB, UB>(v, tau, form, cx);
+      rot_comp<EB, UB>(w, tau, form, cx);
+    }
+  }
+}
+
+// Un-rotations of round R of an adjoint pass.
+template <class PL, int R, bool CP, bool LANES>
+__device__ __forceinline__ void unrot_round(float2 (&v)[PL::NREG], float2 (&w)[PL::NREG], const Sweep &s,
+                                            float tau, int form, float wr, float &acc, const CompCtx &cx) {
+  if constexpr (!CP)
+    unrot_tw<PL::EB, LANES>(v, w, s.m[R], s.lm[R], tau, form, wr, acc);
+  else
+    unrot_tw_comp<PL::EB, R == 0 ? PL::EB - 1 : -1, LANES && R != 0>(v, w, s.m[R], s.lm[R], tau, form, wr, acc, cx);
+}
+
 // z * i^k (k folds to a constant where the register index is one)
 __device__ __forceinline__ float2 ipow(float2 z, int k) {
   k &= 3;
@@ -336,11 +522,48 @@ __device__ __forceinline__ int twist_base(uint64_t T) {
   return __popc(thr_tile<PL, R>()) + __popcll(T);
 }
 
+// Shared-memory slot of tile offset t before the swizzle: t itself, or in a
+// complement-pair tile the complement of t inside box 1 (linear over XOR).
+template <class PL, bool CP>
+__host__ __device__ constexpr uint32_t slot(uint32_t t) {
+  return CP && ((t >> (PL::TB - 1)) & 1u) ? t ^ ((1u << (PL::TB - 1)) - 1u) : t;
+}
+
+// v <- scale * i^popc(x) * v: from the twisted to the standard basis (round R
+// layout; m = the vector's index bits, complement pairs only).
+template <class PL, int R, bool CP>
+__device__ __forceinline__ void untwist_round(float2 (&v)[PL::NREG], uint64_t T, float2 scale, int m) {
+  if constexpr (!CP) {
+    const float2 z = cmulf(scale, ipow(f2(1.f, 0.f), twist_base<PL, R>(T)));
+#pragma unroll
+    for (int r = 0; r < PL::NREG; ++r) v[r] = ipow(cmulf(v[r], z), popc_c(r));
+  } else {
+    // box 1: popc(~x) = m - popc(x)
+    const uint32_t t = thr_tile<PL, R>() & ((1u << (PL::TB - 1)) - 1u);
+    const int k = __popc(t) + __popcll(T);
+    const bool thr1 = thr_tile<PL, R>() != t;
+    const float2 z0 = cmulf(scale, ipow(f2(1.f, 0.f), thr1 ? m - k : k));
+    const float2 z1 = cmulf(scale, ipow(f2(1.f, 0.f), m - k));
+#pragma unroll
+    for (int r = 0; r < PL::NREG; ++r) {
+      if constexpr (R == 0) {
+        if ((r >> (PL::EB - 1)) & 1)
+          v[r] = ipow(cmulf(v[r], z1), 1 - popc_c(r));
+        else
+          v[r] = ipow(cmulf(v[r], z0), popc_c(r));
+      } else {
+        const float2 q = cmulf(v[r], z0);
+        v[r] = thr1 ? ipow(q, -popc_c(r)) : ipow(q, popc_c(r));
+      }
+    }
+  }
+}
+
 // Registers <- shared tile in round-R layout (16-byte accesses when the
 // round holds tile bit 0 in registers).
-template <class PL, int R, int SW>
+template <class PL, int R, int SW, bool CP = false>
 __device__ __forceinline__ void lds_round(float2 (&v)[PL::NREG], const float2 *buf) {
-  const uint32_t st = tswz<SW>(thr_tile<PL, R>());
+  const uint32_t st = tswz<SW>(slot<PL, CP>(thr_tile<PL, R>()));
   if constexpr ((PL::reg(R) & 1u) != 0u) {
 #pragma unroll
     for (int r = 0; r < PL::NREG; r += 2) {
@@ -350,13 +573,13 @@ __device__ __forceinline__ void lds_round(float2 (&v)[PL::NREG], const float2 *b
     }
   } else {
 #pragma unroll
-    for (int r = 0; r < PL::NREG; ++r) v[r] = buf[st ^ tswz<SW>(pdep(r, PL::reg(R)))];
+    for (int r = 0; r < PL::NREG; ++r) v[r] = buf[st ^ tswz<SW>(slot<PL, CP>(pdep(r, PL::reg(R))))];
   }
 }
 
-template <class PL, int R, int SW>
+template <class PL, int R, int SW, bool CP = false>
 __device__ __forceinline__ void sts_round(const float2 (&v)[PL::NREG], float2 *buf) {
-  const uint32_t st = tswz<SW>(thr_tile<PL, R>());
+  const uint32_t st = tswz<SW>(slot<PL, CP>(thr_tile<PL, R>()));
   if constexpr ((PL::reg(R) & 1u) != 0u) {
 #pragma unroll
     for (int r = 0; r < PL::NREG; r += 2)
@@ -364,37 +587,37 @@ __device__ __forceinline__ void sts_round(const float2 (&v)[PL::NREG], float2 *b
           make_float4(v[r].x, v[r].y, v[r + 1].x, v[r + 1].y);
   } else {
 #pragma unroll
-    for (int r = 0; r < PL::NREG; ++r) buf[st ^ tswz<SW>(pdep(r, PL::reg(R)))] = v[r];
+    for (int r = 0; r < PL::NREG; ++r) buf[st ^ tswz<SW>(slot<PL, CP>(pdep(r, PL::reg(R))))] = v[r];
   }
 }
 
-template <class PL, int RF, int RT, int SW>
+template <class PL, int RF, int RT, int SW, bool CP = false>
 __device__ __forceinline__ void xp(float2 (&v)[PL::NREG], float2 *buf) {
-  sts_round<PL, RF, SW>(v, buf);
+  sts_round<PL, RF, SW, CP>(v, buf);
   cbar<PL::NT>();
-  lds_round<PL, RT, SW>(v, buf);
+  lds_round<PL, RT, SW, CP>(v, buf);
 }
 
 // xp with `at_barrier()` run right after the barrier (all reads of the
 // previous round done), before the loads.
-template <class PL, int RF, int RT, int SW, class F>
+template <class PL, int RF, int RT, int SW, bool CP = false, class F>
 __device__ __forceinline__ void xp_hook(float2 (&v)[PL::NREG], float2 *buf, F at_barrier) {
-  sts_round<PL, RF, SW>(v, buf);
+  sts_round<PL, RF, SW, CP>(v, buf);
   cbar<PL::NT>();
   at_barrier();
-  lds_round<PL, RT, SW>(v, buf);
+  lds_round<PL, RT, SW, CP>(v, buf);
 }
 
 // The same for psi and lambda together (one barrier).
-template <class PL, int RF, int RT, int SW, class F>
+template <class PL, int RF, int RT, int SW, bool CP = false, class F>
 __device__ __forceinline__ void xp_pair(float2 (&v)[PL::NREG], float2 (&w)[PL::NREG], float2 *bv,
                                         float2 *bw, F at_barrier) {
-  sts_round<PL, RF, SW>(v, bv);
-  sts_round<PL, RF, SW>(w, bw);
+  sts_round<PL, RF, SW, CP>(v, bv);
+  sts_round<PL, RF, SW, CP>(w, bw);
   cbar<PL::NT>();
   at_barrier();
-  lds_round<PL, RT, SW>(v, bv);
-  lds_round<PL, RT, SW>(w, bw);
+  lds_round<PL, RT, SW, CP>(v, bv);
+  lds_round<PL, RT, SW, CP>(w, bw);
 }
 
 struct NoHook {
@@ -460,29 +683,38 @@ __device__ __forceinline__ float cost_val(int kind, uint32_t word) {
 }
 
 // v <- v * exp(-i g f) (* scl in computed mode; table mode has it folded in).
-template <class PL, int R, int M>
+// Cost-tile slot of register r's amplitude in round R (tt = thr_tile).
+template <class PL, int R, bool CP>
+__device__ __forceinline__ uint32_t cost_slot(uint32_t tt, int r) {
+  if constexpr (CP)
+    return slot<PL, true>(tt) ^ slot<PL, true>(pdep(r, PL::reg(R)));
+  else
+    return tt | pdep(r, PL::reg(R));
+}
+
+template <class PL, int R, bool CP, int M>
 __device__ __forceinline__ void phase_round_m(float2 (&v)[PL::NREG], const CostWord *cb,
                                               const PhaseDigits &ph, int kind, const float2 *tab,
                                               float2 scl) {
   const uint32_t tt = thr_tile<PL, R>();
 #pragma unroll
   for (int r = 0; r < PL::NREG; ++r) {
-    const float2 z = phase_of<M>(ph, kind, tab, cb[tt | pdep(r, PL::reg(R))]);
+    const float2 z = phase_of<M>(ph, kind, tab, cb[cost_slot<PL, R, CP>(tt, r)]);
     v[r] = cmulf(v[r], M == 1 ? cmulf(scl, z) : z);
   }
 }
 
-template <class PL, int R>
+template <class PL, int R, bool CP = false>
 __device__ __forceinline__ void phase_round(float2 (&v)[PL::NREG], const CostWord *cb,
                                             const PhaseDigits &ph, int kind, const float2 *tab,
                                             float2 scl) {
   const int m = phase_m(ph);
   if (m == 2)
-    phase_round_m<PL, R, 2>(v, cb, ph, kind, tab, scl);
+    phase_round_m<PL, R, CP, 2>(v, cb, ph, kind, tab, scl);
   else if (m == 3)
-    phase_round_m<PL, R, 3>(v, cb, ph, kind, tab, scl);
+    phase_round_m<PL, R, CP, 3>(v, cb, ph, kind, tab, scl);
   else
-    phase_round_m<PL, R, 1>(v, cb, ph, kind, tab, scl);
+    phase_round_m<PL, R, CP, 1>(v, cb, ph, kind, tab, scl);
 }
 
 // Float-float running sum (Knuth's TwoSum adds each term exactly into hi + lo):
@@ -497,7 +729,7 @@ struct FF {
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
-template <class PL, int R>
+template <class PL, int R, bool CP>
 __device__ __forceinline__ void eo_round(const float2 (&v)[PL::NREG], const CostWord *cb, int kind,
                                          uint32_t fmin_word, float &e, float &o) {
   // f == f_min is tested on the raw words (exact for integer costs; for
@@ -505,7 +737,7 @@ __device__ __forceinline__ void eo_round(const float2 (&v)[PL::NREG], const Cost
   const uint32_t tt = thr_tile<PL, R>();
 #pragma unroll
   for (int r = 0; r < PL::NREG; ++r) {
-    const uint32_t w = cb[tt | pdep(r, PL::reg(R))];
+    const uint32_t w = cb[cost_slot<PL, R, CP>(tt, r)];
     const float f = cost_val(kind, w);
     const float pr = v[r].x * v[r].x + v[r].y * v[r].y;
     e += pr * f;
@@ -608,6 +840,44 @@ __device__ __forceinline__ void stg_round(const float2 (&v)[PL::NREG], float2 *g
   }
 }
 
+// The same for a tile of a half vector (index bits m): a complement-pair tile
+// where CP (box 1 at the complemented indices), and with mirror every
+// amplitude at its n-bit complement mirror - x too.
+template <class PL, int R, bool CP>
+__device__ __forceinline__ void stg_half(const float2 (&v)[PL::NREG], float2 *g, uint64_t T, int h, int c,
+                                         int m, uint64_t mirror) {
+  constexpr uint32_t RM = PL::reg(R), BM = CP ? (1u << (PL::TB - 1)) - 1u : (1u << PL::TB) - 1u;
+  const int midbits = h - c, box = PL::TB - (CP ? 1 : 0);
+  const uint32_t cm = (1u << c) - 1u;
+  auto f = [&](uint32_t t) -> int64_t { return (int64_t)((uint64_t)(t & cm) | ((uint64_t)(t >> c) << h)); };
+  const uint64_t mid = T & ((1ull << midbits) - 1ull), top = T >> midbits;
+  const uint32_t thr = thr_tile<PL, R>();
+  const int64_t x0 = (int64_t)((mid << c) | (top << (h + box - c))) + f(thr & BM);
+  const int64_t all = (int64_t)((1ull << m) - 1ull);
+  const bool thr1 = CP && (thr & ~BM) != 0u;  // this thread's amplitudes are in box 1
+  int64_t u[PL::EB];
+#pragma unroll
+  for (int k = 0; k < PL::EB; ++k) {
+    const uint32_t b = pdep(1u << k, RM);
+    u[k] = (b & ~BM) ? 0 : f(b);  // the box bit is no index bit
+  }
+  auto put = [&](int64_t xa, int64_t xb, bool neg) {  // box 0 / box 1 start; neg: box 0 descends
+    int64_t s[PL::EB];
+#pragma unroll
+    for (int k = 0; k < PL::EB; ++k) s[k] = neg ? -u[k] : u[k];
+#pragma unroll
+    for (int r = 0; r < PL::NREG; ++r) {
+      int64_t off = 0;
+#pragma unroll
+      for (int k = 0; k < PL::EB; ++k)
+        if ((r >> k) & 1) off += s[k];
+      g[(pdep(r, RM) & ~BM) != 0u ? xb - off : xa + off] = v[r];
+    }
+  };
+  put(thr1 ? all - x0 : x0, all - x0, thr1);
+  if (mirror) put((int64_t)mirror - (thr1 ? all - x0 : x0), (int64_t)mirror - (all - x0), !thr1);
+}
+
 __device__ __forceinline__ unsigned char *aligned_base(unsigned char *raw) {
   const uint32_t a = smem_u32(raw);
   return raw + ((1024u - (a & 1023u)) & 1023u);
@@ -649,13 +919,17 @@ __device__ __forceinline__ void drain(int aborted, uint64_t *full, int i) {
 // own path: forward  K = kH1 | kPH | kH2 | kRED,  adjoint  K = kPH | kH2 | kINIT.
 constexpr int kH1 = 1, kPH = 2, kH2 = 4, kRED = 8, kINIT = 8;
 
-template <class PL, int K>
+// CP: the tiles are complement pairs of a half vector (P.comp index bits).
+template <class PL, int K, bool CP>
 __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__ TmaFwdParams P) {
-  constexpr int NREG = PL::NREG, NR = PL::NR, EB = PL::EB, SW = 128;
+  constexpr int NREG = PL::NREG, NR = PL::NR, SW = 128;
   constexpr bool H1 = (K & kH1) != 0, PH = (K & kPH) != 0, H2 = (K & kH2) != 0, RED = (K & kRED) != 0;
   static_assert(!(H1 && PH && !H2), "a first sweep with the phase always has a second sweep");
   constexpr bool need_cost = PH || RED;
   constexpr int RS = (H1 && H2) ? 0 : NR - 1;  // the round the tile is stored from
+  // pass kinds that can end a sweep (the schedule's last pass: k >= 2 groups
+  // H1, one group PH + H2); the others carry no code for it
+  constexpr bool END = RED || (H1 && !PH) || (PH && !H1);
   extern __shared__ unsigned char smem_raw[];
   unsigned char *base = aligned_base(smem_raw);
   const Lay L = layout(1u << PL::TB, false, need_cost);
@@ -676,31 +950,40 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
   }
   __syncthreads();
 
-  // 8- or 16-amplitude segments: the outer bits between the segments are view
-  // dimension 1; wider segments (bits 4.. are view dimension 1): dimension 2
-  auto coords = [&](uint64_t T) {
+  // the outer bits between the segments are view dimension 1 or 2 (mid2);
+  // box 1 of a complement pair sits at the complemented tile number
+  auto coords = [&](uint64_t T, bool box1) {
+    if (CP && box1) T = ~T & ((1ull << (P.comp - (PL::TB - 1))) - 1ull);
     const int mid = (int)(T & ((1ull << midbits) - 1ull));
     TC c;
-    c.x1 = P.c <= 4 ? mid : 0;
-    c.x2 = P.c <= 4 ? 0 : mid;
+    c.x1 = P.mid2 ? 0 : mid;
+    c.x2 = P.mid2 ? mid : 0;
     c.x4 = (int)(T >> midbits);
     return c;
+  };
+  auto load_state = [&](uint64_t T, TC c) {
+    tma_load(buf, &P.map_psi, c, full);
+    if (CP) tma_load(buf + (1u << (PL::TB - 1)), &P.map_psi, coords(T, true), full);
+  };
+  auto load_cost = [&](uint64_t T, TC c) {
+    tma_load(base + L.cost_off, &P.map_cost, c, full);
+    if (CP) tma_load(base + L.cost_off + L.cost_bytes / 2u, &P.map_cost, coords(T, true), full);
   };
   // Phase passes that read the cost tile before their last barrier load the
   // next tile's costs as soon as that barrier passes, the state later.
   constexpr bool early_cost = PH && !RED;
   auto issue = [&](uint64_t T, bool cost) {
-    const TC c = coords(T);
+    const TC c = coords(T, false);
     mbar_expect_tx(full, (P.init_plus ? 0u : L.tile_bytes) + (cost ? L.cost_bytes : 0u));
-    if (!P.init_plus) tma_load(buf, &P.map_psi, c, full);
-    if (cost) tma_load(base + L.cost_off, &P.map_cost, c, full);
+    if (!P.init_plus) load_state(T, c);
+    if (cost) load_cost(T, c);
   };
   int abort_now = 0;  // uniform over the CTA: read after the tile's first barrier
   auto read_abort = [&]() { abort_now = s_abort; };
   auto cost_next = [&](uint64_t T) {
     if (tid == 0 && T + gridDim.x < P.ntiles && !abort_now) {
       mbar_add_tx(full, L.cost_bytes);
-      tma_load(base + L.cost_off, &P.map_cost, coords(T + gridDim.x), full);
+      load_cost(T + gridDim.x, coords(T + gridDim.x, false));
     }
   };
   // after the tile's last shared-memory read: the buffers go to the next load
@@ -712,6 +995,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
   if (tid == 0 && blockIdx.x < P.ntiles) issue(blockIdx.x, need_cost);
 
   FF acc_e, acc_o;  // this thread's energy / overlap terms
+  CompCtx cx;
+  if constexpr (CP) {
+    cx.odd = (P.comp & 1) != 0;
+    cx.box1 = (thr_tile<PL, 1>() >> (PL::TB - 1)) != 0u;
+  }
   int i = 0;
   for (;; ++i) {
     const uint64_t T = blockIdx.x + (uint64_t)i * gridDim.x;
@@ -725,13 +1013,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
       atomicExch(P.err, 1u);
     }
     float2 v[NREG];
+    if constexpr (CP) cx.eps = ((((P.comp - 1) >> 1) + twist_base<PL, 0>(T)) & 1) ? -1.f : 1.f;
     if (P.init_plus) {
       // |+>^n in the twisted basis: amp (-i)^popc(x)
       const float2 z0 = ipow(f2(P.amp, 0.f), -twist_base<PL, 0>(T));
 #pragma unroll
       for (int r = 0; r < NREG; ++r) v[r] = ipow(z0, -popc_c(r));
     } else {
-      lds_round<PL, 0, SW>(v, buf);
+      lds_round<PL, 0, SW, CP>(v, buf);
       if (P.twist_in) {
         const float2 z = ipow(f2(1.f, 0.f), -twist_base<PL, 0>(T));
 #pragma unroll
@@ -739,56 +1028,54 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
       }
     }
     if constexpr (H1) {
-      rot_tw<EB>(v, P.s1.m[0], P.tau1, P.form1);
-      xp_hook<PL, 0, 1, SW>(v, buf, read_abort);
+      rot_round<PL, 0, CP>(v, P.s1.m[0], P.tau1, P.form1, cx);
+      xp_hook<PL, 0, 1, SW, CP>(v, buf, read_abort);
       if constexpr (NR == 2 && !H2 && !RED) release(T);
-      rot_tw<EB>(v, P.s1.m[1], P.tau1, P.form1);
+      rot_round<PL, 1, CP>(v, P.s1.m[1], P.tau1, P.form1, cx);
       if constexpr (NR == 3) {
         xp<PL, 1, 2, SW>(v, buf);
         if constexpr (!H2 && !RED) release(T);
-        rot_tw<EB>(v, P.s1.m[2], P.tau1, P.form1);
+        rot_round<PL, 2, CP>(v, P.s1.m[2], P.tau1, P.form1, cx);
       }
-      if constexpr (PH) phase_round<PL, NR - 1>(v, cb, P.ph, P.cost_kind, tab, P.scl_phase);
+      if constexpr (PH) phase_round<PL, NR - 1, CP>(v, cb, P.ph, P.cost_kind, tab, P.scl_phase);
       if constexpr (H2) {
-        rot_tw<EB>(v, P.s2.m[NR - 1], P.tau2, P.form2);
+        rot_round<PL, NR - 1, CP>(v, P.s2.m[NR - 1], P.tau2, P.form2, cx);
         if constexpr (NR == 3) {
           if constexpr (early_cost)
             xp_hook<PL, 2, 1, SW>(v, buf, [&] { cost_next(T); });
           else
             xp<PL, 2, 1, SW>(v, buf);
-          rot_tw<EB>(v, P.s2.m[1], P.tau2, P.form2);
+          rot_round<PL, 1, CP>(v, P.s2.m[1], P.tau2, P.form2, cx);
         }
         if constexpr (NR == 3) {
           xp<PL, 1, 0, SW>(v, buf);
         } else if constexpr (early_cost) {
-          xp_hook<PL, 1, 0, SW>(v, buf, [&] { cost_next(T); });
+          xp_hook<PL, 1, 0, SW, CP>(v, buf, [&] { cost_next(T); });
         } else {
-          xp<PL, 1, 0, SW>(v, buf);
+          xp<PL, 1, 0, SW, CP>(v, buf);
         }
         if constexpr (!RED) release(T);
-        rot_tw<EB>(v, P.s2.m[0], P.tau2, P.form2);
+        rot_round<PL, 0, CP>(v, P.s2.m[0], P.tau2, P.form2, cx);
       }
     } else {
-      if constexpr (PH) phase_round<PL, 0>(v, cb, P.ph, P.cost_kind, tab, P.scl_phase);
-      rot_tw<EB>(v, P.s2.m[0], P.tau2, P.form2);
+      if constexpr (PH) phase_round<PL, 0, CP>(v, cb, P.ph, P.cost_kind, tab, P.scl_phase);
+      rot_round<PL, 0, CP>(v, P.s2.m[0], P.tau2, P.form2, cx);
       if constexpr (early_cost)
-        xp_hook<PL, 0, 1, SW>(v, buf, [&] { read_abort(); cost_next(T); });
+        xp_hook<PL, 0, 1, SW, CP>(v, buf, [&] { read_abort(); cost_next(T); });
       else
-        xp_hook<PL, 0, 1, SW>(v, buf, read_abort);
+        xp_hook<PL, 0, 1, SW, CP>(v, buf, read_abort);
       if constexpr (NR == 2 && !RED) release(T);
-      rot_tw<EB>(v, P.s2.m[1], P.tau2, P.form2);
+      rot_round<PL, 1, CP>(v, P.s2.m[1], P.tau2, P.form2, cx);
       if constexpr (NR == 3) {
         xp<PL, 1, 2, SW>(v, buf);
         if constexpr (!RED) release(T);
-        rot_tw<EB>(v, P.s2.m[2], P.tau2, P.form2);
+        rot_round<PL, 2, CP>(v, P.s2.m[2], P.tau2, P.form2, cx);
       }
     }
-    if (P.end_scale) {
+    if (END && P.end_scale) {
       if (P.untwist) {
         // back to the standard basis: psi(x) = i^popc(x) s(x)
-        const float2 z = cmulf(P.scl_end, ipow(f2(1.f, 0.f), twist_base<PL, RS>(T)));
-#pragma unroll
-        for (int r = 0; r < NREG; ++r) v[r] = ipow(cmulf(v[r], z), popc_c(r));
+        untwist_round<PL, RS, CP>(v, T, P.scl_end, P.comp);
       } else {
 #pragma unroll
         for (int r = 0; r < NREG; ++r) v[r] = cmulf(v[r], P.scl_end);
@@ -796,12 +1083,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
     }
     if constexpr (RED) {
       float e = 0.f, o = 0.f;
-      eo_round<PL, RS>(v, cb, P.cost_kind, P.fmin_word, e, o);
+      eo_round<PL, RS, CP>(v, cb, P.cost_kind, P.fmin_word, e, o);
       acc_e.add(e);
       acc_o.add(o);
       release(T);
     }
-    stg_round<PL, RS>(v, P.psi, T, P.h, P.c);
+    if constexpr (CP)
+      stg_half<PL, RS, true>(v, P.psi, T, P.h, P.c, P.comp, END ? P.mirror : 0);
+    else if (END && P.mirror)
+      stg_half<PL, RS, false>(v, P.psi, T, P.h, P.c, 0, P.mirror);
+    else
+      stg_round<PL, RS>(v, P.psi, T, P.h, P.c);
   }
   drain(abort_now, full, i);
   if constexpr (RED) {
@@ -812,9 +1104,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
       P.partials[blockIdx.x * 2 + 1] = a[1];
     }
     double *out = P.out;
-    final_reduce<2>(P.partials, gridDim.x, P.counter, red, [out](double(&a)[2]) {
-      out[0] = a[0];
-      out[1] = a[1];
+    const double sc = P.out_scale;
+    final_reduce<2>(P.partials, gridDim.x, P.counter, red, [out, sc](double(&a)[2]) {
+      out[0] = sc * a[0];
+      out[1] = sc * a[1];
     });
   }
 }
@@ -828,14 +1121,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
 struct CostIdx {
   __device__ __forceinline__ uint32_t operator()(uint32_t t) const { return t; }
 };
-template <class PL, int R, int M, class CI = CostIdx>
+template <class PL, int R, bool CP, int M, class CI>
 __device__ __forceinline__ void unphase_round(float2 (&v)[PL::NREG], float2 (&w)[PL::NREG],
                                               const CostWord *cb, const TmaBwdParams &P,
-                                              const float2 *tab, float &ag, CI ci = CI()) {
+                                              const float2 *tab, float &ag, CI ci) {
   const uint32_t tt = thr_tile<PL, R>();
 #pragma unroll
   for (int r = 0; r < PL::NREG; ++r) {
-    const uint32_t word = cb[ci(tt | pdep(r, PL::reg(R)))];
+    const uint32_t word = cb[ci(cost_slot<PL, R, CP>(tt, r))];
     const float f = cost_val(P.cost_kind, word);
     ag += P.wg * f * (w[r].x * v[r].y - w[r].y * v[r].x);
     float2 ph = phase_of<M>(P.ph, P.cost_kind, tab, word);
@@ -845,27 +1138,29 @@ __device__ __forceinline__ void unphase_round(float2 (&v)[PL::NREG], float2 (&w)
   }
 }
 
-template <class PL, int R, class CI = CostIdx>
+template <class PL, int R, bool CP = false, class CI = CostIdx>
 __device__ __forceinline__ void unphase_any(float2 (&v)[PL::NREG], float2 (&w)[PL::NREG],
                                             const CostWord *cb, const TmaBwdParams &P,
                                             const float2 *tab, float &ag, CI ci = CI()) {
   const int m = phase_m(P.ph);
   if (m == 2)
-    unphase_round<PL, R, 2>(v, w, cb, P, tab, ag, ci);
+    unphase_round<PL, R, CP, 2>(v, w, cb, P, tab, ag, ci);
   else if (m == 3)
-    unphase_round<PL, R, 3>(v, w, cb, P, tab, ag, ci);
+    unphase_round<PL, R, CP, 3>(v, w, cb, P, tab, ag, ci);
   else
-    unphase_round<PL, R, 1>(v, w, cb, P, tab, ag, ci);
+    unphase_round<PL, R, CP, 1>(v, w, cb, P, tab, ag, ci);
 }
 
 // The state tiles use the TMA 128-byte swizzle (16- to 64-amplitude segments).
-template <class PL, int K>
+// CP: complement-pair tiles (see k_fwd_tma).
+template <class PL, int K, bool CP>
 __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_constant__ TmaBwdParams P) {
-  constexpr int NREG = PL::NREG, NR = PL::NR, EB = PL::EB, SW = 128;
-  constexpr bool LN = PL::NT == 512;  // the 512-thread plan rotates tile bit 12 across lanes
+  constexpr int NREG = PL::NREG, NR = PL::NR, SW = 128;
+  constexpr bool LN = PL::NT == 512;  // the 512-thread plans rotate one tile bit across lanes
   constexpr bool PH = (K & kPH) != 0, H2 = (K & kH2) != 0, INIT = (K & kINIT) != 0;
   constexpr bool need_cost = PH || INIT;
   constexpr int RS = H2 ? 0 : NR - 1;  // the round the tiles are stored from
+  constexpr bool END = PH && !H2;      // the kind of the last pass (untwist, mirror)
   extern __shared__ unsigned char smem_raw[];
   unsigned char *base = aligned_base(smem_raw);
   const Lay L = layout(1u << PL::TB, true, need_cost);
@@ -887,15 +1182,22 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
   }
   __syncthreads();
 
-  // 8- or 16-amplitude segments: the outer bits between the segments are view
-  // dimension 1; wider segments (bits 4.. are view dimension 1): dimension 2
-  auto coords = [&](uint64_t T) {
+  auto coords = [&](uint64_t T, bool box1) {  // as in k_fwd_tma
+    if (CP && box1) T = ~T & ((1ull << (P.comp - (PL::TB - 1))) - 1ull);
     const int mid = (int)(T & ((1ull << midbits) - 1ull));
     TC c;
-    c.x1 = P.c <= 4 ? mid : 0;
-    c.x2 = P.c <= 4 ? 0 : mid;
+    c.x1 = P.mid2 ? 0 : mid;
+    c.x2 = P.mid2 ? mid : 0;
     c.x4 = (int)(T >> midbits);
     return c;
+  };
+  auto load_vec = [&](float2 *dst, const CUtensorMap *map, uint64_t T, TC c) {
+    tma_load(dst, map, c, full);
+    if (CP) tma_load(dst + (1u << (PL::TB - 1)), map, coords(T, true), full);
+  };
+  auto load_cost = [&](uint64_t T, TC c) {
+    tma_load(base + L.cost_off, &P.map_cost, c, full);
+    if (CP) tma_load(base + L.cost_off + L.cost_bytes / 2u, &P.map_cost, coords(T, true), full);
   };
   // Passes whose cost reads end before a later barrier (lambda = f psi in the
   // first round; the phase of a pivot) load the next tile's costs at that
@@ -905,16 +1207,16 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
   int abort_now = 0;  // uniform over the CTA: read after the tile's first barrier
   auto read_abort = [&]() { abort_now = s_abort; };
   auto issue = [&](uint64_t T, bool cost) {
-    const TC c = coords(T);
+    const TC c = coords(T, false);
     mbar_expect_tx(full, L.tile_bytes + (INIT ? 0u : L.tile_bytes) + (cost ? L.cost_bytes : 0u));
-    tma_load(bv, &P.map_psi, c, full);
-    if (!INIT) tma_load(bw, &P.map_lam, c, full);
-    if (cost) tma_load(base + L.cost_off, &P.map_cost, c, full);
+    load_vec(bv, &P.map_psi, T, c);
+    if (!INIT) load_vec(bw, &P.map_lam, T, c);
+    if (cost) load_cost(T, c);
   };
   auto cost_next = [&](uint64_t T) {
     if (tid == 0 && T + gridDim.x < P.ntiles && !abort_now) {
       mbar_add_tx(full, L.cost_bytes);
-      tma_load(base + L.cost_off, &P.map_cost, coords(T + gridDim.x), full);
+      load_cost(T + gridDim.x, coords(T + gridDim.x, false));
     }
   };
   // after the tile's last shared-memory read: the buffers go to the next load
@@ -930,23 +1232,28 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
   auto release_vectors = [&](uint64_t T) {
     cbar<PL::NT>();
     if (tid == 0 && T + gridDim.x < P.ntiles && !abort_now) {
-      const TC c = coords(T + gridDim.x);
+      const TC c = coords(T + gridDim.x, false);
       mbar_add_tx(full, 2u * L.tile_bytes);
-      tma_load(bv, &P.map_psi, c, full);
-      tma_load(bw, &P.map_lam, c, full);
+      load_vec(bv, &P.map_psi, T + gridDim.x, c);
+      load_vec(bw, &P.map_lam, T + gridDim.x, c);
     }
   };
   auto release_cost = [&](uint64_t T) {
     cbar<PL::NT>();
     if (tid == 0 && T + gridDim.x < P.ntiles && !abort_now) {
       mbar_expect_tx(full, L.cost_bytes);
-      tma_load(base + L.cost_off, &P.map_cost, coords(T + gridDim.x), full);
+      load_cost(T + gridDim.x, coords(T + gridDim.x, false));
     }
   };
 
   if (tid == 0 && blockIdx.x < P.ntiles) issue(blockIdx.x, need_cost);
 
   FF acc1, accg, acc2;  // this thread's gradient terms
+  CompCtx cx;
+  if constexpr (CP) {
+    cx.odd = (P.comp & 1) != 0;
+    cx.box1 = (thr_tile<PL, 1>() >> (PL::TB - 1)) != 0u;
+  }
   int i = 0;
   for (;; ++i) {
     const uint64_t T = blockIdx.x + (uint64_t)i * gridDim.x;
@@ -960,66 +1267,71 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
       atomicExch(P.err, 1u);
     }
     float2 v[NREG], w[NREG];
-    lds_round<PL, 0, SW>(v, bv);
+    if constexpr (CP) cx.eps = ((((P.comp - 1) >> 1) + twist_base<PL, 0>(T)) & 1) ? -1.f : 1.f;
+    lds_round<PL, 0, SW, CP>(v, bv);
     if constexpr (INIT) {
       // lambda = f psi: the derivative of E = <psi|f|psi> with respect to psi^*
       const uint32_t tt = thr_tile<PL, 0>();
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
-        const float f = cost_val(P.cost_kind, cb[tt | pdep(r, PL::reg(0))]);
+        const float f = cost_val(P.cost_kind, cb[cost_slot<PL, 0, CP>(tt, r)]);
         w[r] = f2(f * v[r].x, f * v[r].y);
       }
     } else {
-      lds_round<PL, 0, SW>(w, bw);
+      lds_round<PL, 0, SW, CP>(w, bw);
     }
     float a1 = 0.f, ag = 0.f, a2 = 0.f;
-    unrot_tw<EB, LN>(v, w, P.s1.m[0], P.s1.lm[0], P.tau1, P.form1, P.w1[0], a1);
+    unrot_round<PL, 0, CP, LN>(v, w, P.s1, P.tau1, P.form1, P.w1[0], a1, cx);
     if constexpr (INIT && early_cost)
-      xp_pair<PL, 0, 1, SW>(v, w, bv, bw, [&] { read_abort(); cost_next(T); });
+      xp_pair<PL, 0, 1, SW, CP>(v, w, bv, bw, [&] { read_abort(); cost_next(T); });
     else
-      xp_pair<PL, 0, 1, SW>(v, w, bv, bw, [&] { read_abort(); });
+      xp_pair<PL, 0, 1, SW, CP>(v, w, bv, bw, [&] { read_abort(); });
     if constexpr (NR == 2 && !PH && !H2) release(T);
     if constexpr (NR == 2 && late_cost) release_vectors(T);
-    unrot_tw<EB, LN>(v, w, P.s1.m[1], P.s1.lm[1], P.tau1, P.form1, P.w1[1], a1);
+    unrot_round<PL, 1, CP, LN>(v, w, P.s1, P.tau1, P.form1, P.w1[1], a1, cx);
     if constexpr (NR == 3) {
       xp_pair<PL, 1, 2, SW>(v, w, bv, bw, NoHook());
       if constexpr (!PH && !H2) release(T);
       if constexpr (late_cost) release_vectors(T);
-      unrot_tw<EB, LN>(v, w, P.s1.m[2], P.s1.lm[2], P.tau1, P.form1, P.w1[2], a1);
+      unrot_round<PL, 2, CP, LN>(v, w, P.s1, P.tau1, P.form1, P.w1[2], a1, cx);
     }
     if constexpr (PH) {
       // d/d gamma: Im <lambda| f |psi>, then un-phase both vectors
-      unphase_any<PL, NR - 1>(v, w, cb, P, tab, ag);
+      unphase_any<PL, NR - 1, CP>(v, w, cb, P, tab, ag);
       if constexpr (late_cost)
         release_cost(T);
       else if constexpr (!H2)
         release(T);
     }
     if constexpr (H2) {
-      unrot_tw<EB, LN>(v, w, P.s2.m[NR - 1], P.s2.lm[NR - 1], P.tau2, P.form2, P.w2[NR - 1], a2);
+      unrot_round<PL, NR - 1, CP, LN>(v, w, P.s2, P.tau2, P.form2, P.w2[NR - 1], a2, cx);
       if constexpr (NR == 3) {
         if constexpr (PH && early_cost)
           xp_pair<PL, 2, 1, SW>(v, w, bv, bw, [&] { cost_next(T); });
         else
           xp_pair<PL, 2, 1, SW>(v, w, bv, bw, NoHook());
-        unrot_tw<EB, LN>(v, w, P.s2.m[1], P.s2.lm[1], P.tau2, P.form2, P.w2[1], a2);
+        unrot_round<PL, 1, CP, LN>(v, w, P.s2, P.tau2, P.form2, P.w2[1], a2, cx);
         xp_pair<PL, 1, 0, SW>(v, w, bv, bw, NoHook());
       } else if constexpr (PH && early_cost) {
-        xp_pair<PL, 1, 0, SW>(v, w, bv, bw, [&] { cost_next(T); });
+        xp_pair<PL, 1, 0, SW, CP>(v, w, bv, bw, [&] { cost_next(T); });
       } else {
-        xp_pair<PL, 1, 0, SW>(v, w, bv, bw, NoHook());
+        xp_pair<PL, 1, 0, SW, CP>(v, w, bv, bw, NoHook());
       }
       release(T);
-      unrot_tw<EB, LN>(v, w, P.s2.m[0], P.s2.lm[0], P.tau2, P.form2, P.w2[0], a2);
+      unrot_round<PL, 0, CP, LN>(v, w, P.s2, P.tau2, P.form2, P.w2[0], a2, cx);
     }
-    if (P.untwist) {
-      // psi back to the standard basis (lambda is scratch from here on)
-      const float2 z = ipow(f2(1.f, 0.f), twist_base<PL, RS>(T));
-#pragma unroll
-      for (int r = 0; r < NREG; ++r) v[r] = ipow(cmulf(v[r], z), popc_c(r));
+    if (END && P.untwist)  // psi back to the standard basis (lambda is scratch from here on)
+      untwist_round<PL, RS, CP>(v, T, f2(1.f, 0.f), P.comp);
+    if constexpr (CP) {
+      stg_half<PL, RS, true>(v, P.psi, T, P.h, P.c, P.comp, END ? P.mirror : 0);
+      if (!END || !P.untwist) stg_half<PL, RS, true>(w, P.lam, T, P.h, P.c, P.comp, 0);
+    } else {
+      if (END && P.mirror)
+        stg_half<PL, RS, false>(v, P.psi, T, P.h, P.c, 0, P.mirror);
+      else
+        stg_round<PL, RS>(v, P.psi, T, P.h, P.c);
+      if (!END || !P.untwist) stg_round<PL, RS>(w, P.lam, T, P.h, P.c);  // the last pass: lambda is spent
     }
-    stg_round<PL, RS>(v, P.psi, T, P.h, P.c);
-    if (!P.untwist) stg_round<PL, RS>(w, P.lam, T, P.h, P.c);  // the last pass: lambda is spent
     acc1.add(a1);
     accg.add(ag);
     acc2.add(a2);
@@ -1033,10 +1345,11 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
     P.partials[blockIdx.x * 3 + 2] = a[2];
   }
   double *o1 = P.out_b1, *og = P.out_g, *o2 = P.out_b2;
+  const double sc = P.out_scale;
   final_reduce<3>(P.partials, gridDim.x, P.counter, red, [=](double(&a)[3]) {
-    if (o1) *o1 += 2.0 * a[0];
-    if (og) *og += 2.0 * a[1];
-    if (o2) *o2 += 2.0 * a[2];
+    if (o1) *o1 += sc * a[0];
+    if (og) *og += sc * a[1];
+    if (o2) *o2 += sc * a[2];
   });
 }
 
@@ -1521,7 +1834,8 @@ EncodeFn encode_fn() {
 
 // 5-D tile view of a 2^n vector of `esz`-byte elements for tiles of 2^tb
 // elements with 2^c contiguous ones:
-// [2^c][2^(h-c)][256][2^(tb-c-8)][2^(n-h-(tb-c))]; one box = one tile.
+// [2^c][2^(h-c)][256][2^(tb-c-8)][2^(n-h-(tb-c))], or where tile_map_mid2
+// [16][2^(c-4)][2^(h-c)][2^(tb-c)][2^(n-h-(tb-c))]; one box = one tile.
 cudaError_t make_tile_map(CUtensorMap *map, void *base, int n, int tb, int h, int c, int esz,
                           int swizzle_bytes) {
   EncodeFn fn = encode_fn();
@@ -1529,7 +1843,7 @@ cudaError_t make_tile_map(CUtensorMap *map, void *base, int n, int tb, int h, in
   const cuuint64_t e = (cuuint64_t)esz;
   cuuint64_t dims[5], strides[4];
   cuuint32_t box[5];
-  if (c >= 5) {
+  if (tile_map_mid2(tb, c)) {
     // 2^c contiguous amplitudes as [16][2^(c-4)] (a swizzled box row is at
     // most 128 bytes), then the outer bits c..h-1, the rows, the rest
     const int rows = tb - c;
@@ -1612,10 +1926,10 @@ cudaError_t launch_wait_selftest(unsigned *err, cudaStream_t s) {
 }
 #endif  // QAOA_TMA_CW == 4
 
-template <class PL, int K>
+template <class PL, int K, bool CP>
 static cudaError_t launch_fwd_tma_t(const TmaFwdParams &P, cudaStream_t s, int nsm) {
   const size_t smem = smem_bytes(PL::TB, false, (K & (kPH | kRED)) != 0);
-  auto kern = k_fwd_tma<PL, K>;
+  auto kern = k_fwd_tma<PL, K, CP>;
   static int nb = 0;
   if (nb == 0) {
     const size_t mx = smem_bytes(PL::TB, false, true);
@@ -1631,10 +1945,10 @@ static cudaError_t launch_fwd_tma_t(const TmaFwdParams &P, cudaStream_t s, int n
   return cudaGetLastError();
 }
 
-template <class PL, int K>
+template <class PL, int K, bool CP>
 static cudaError_t launch_bwd_tma_t(const TmaBwdParams &P, cudaStream_t s, int nsm) {
   const size_t smem = smem_bytes(PL::TB, true, (K & (kPH | kINIT)) != 0);
-  auto kern = k_bwd_tma<PL, K>;
+  auto kern = k_bwd_tma<PL, K, CP>;
   static int nb = 0;
   if (nb == 0) {
     const size_t mx = smem_bytes(PL::TB, true, true);
@@ -1706,12 +2020,28 @@ static cudaError_t dispatch_fwd(const TmaFwdParams &P, cudaStream_t s, int nsm) 
   const bool h2 = (P.s2.m[0] | P.s2.m[1] | P.s2.m[2]) != 0;
   const int k = (h1 ? kH1 : 0) | (P.has_phase ? kPH : 0) | (h2 ? kH2 : 0) | (P.reduce ? kRED : 0);
   switch (k) {  // the kinds the forward schedules produce
-    case kPH | kH2: return launch_fwd_tma_t<PL, kPH | kH2>(P, s, nsm);
-    case kPH | kH2 | kRED: return launch_fwd_tma_t<PL, kPH | kH2 | kRED>(P, s, nsm);
-    case kH2: return launch_fwd_tma_t<PL, kH2>(P, s, nsm);
-    case kH1 | kPH | kH2: return launch_fwd_tma_t<PL, kH1 | kPH | kH2>(P, s, nsm);
-    case kH1: return launch_fwd_tma_t<PL, kH1>(P, s, nsm);
-    case kH1 | kRED: return launch_fwd_tma_t<PL, kH1 | kRED>(P, s, nsm);
+    case kPH | kH2: return launch_fwd_tma_t<PL, kPH | kH2, false>(P, s, nsm);
+    case kPH | kH2 | kRED: return launch_fwd_tma_t<PL, kPH | kH2 | kRED, false>(P, s, nsm);
+    case kH2: return launch_fwd_tma_t<PL, kH2, false>(P, s, nsm);
+    case kH1 | kPH | kH2: return launch_fwd_tma_t<PL, kH1 | kPH | kH2, false>(P, s, nsm);
+    case kH1: return launch_fwd_tma_t<PL, kH1, false>(P, s, nsm);
+    case kH1 | kRED: return launch_fwd_tma_t<PL, kH1 | kRED, false>(P, s, nsm);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// The complement-pair group is always the last of the order: it carries the
+// pivots and may end the sweep, and never starts one.
+template <class PL>
+static cudaError_t dispatch_fwd_comp(const TmaFwdParams &P, cudaStream_t s, int nsm) {
+  static_assert(comp_plan<PL>(), "complement tile bit");
+  const bool h1 = (P.s1.m[0] | P.s1.m[1]) != 0, h2 = (P.s2.m[0] | P.s2.m[1]) != 0;
+  const int k = (h1 ? kH1 : 0) | (P.has_phase ? kPH : 0) | (h2 ? kH2 : 0) | (P.reduce ? kRED : 0);
+  if (P.comp < PL::TB || P.init_plus || P.twist_in) return cudaErrorInvalidValue;
+  switch (k) {
+    case kH1 | kPH | kH2: return launch_fwd_tma_t<PL, kH1 | kPH | kH2, true>(P, s, nsm);
+    case kH1: return launch_fwd_tma_t<PL, kH1, true>(P, s, nsm);
+    case kH1 | kRED: return launch_fwd_tma_t<PL, kH1 | kRED, true>(P, s, nsm);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1721,11 +2051,24 @@ static cudaError_t dispatch_bwd(const TmaBwdParams &P, cudaStream_t s, int nsm) 
   const bool h2 = (P.s2.m[0] | P.s2.m[1] | P.s2.m[2] | P.s2.lm[0] | P.s2.lm[1] | P.s2.lm[2]) != 0;
   const int k = (P.has_phase ? kPH : 0) | (h2 ? kH2 : 0) | (P.init_lambda ? kINIT : 0);
   switch (k) {  // the kinds the adjoint schedules produce
-    case 0: return launch_bwd_tma_t<PL, 0>(P, s, nsm);
-    case kINIT: return launch_bwd_tma_t<PL, kINIT>(P, s, nsm);
-    case kPH | kH2: return launch_bwd_tma_t<PL, kPH | kH2>(P, s, nsm);
-    case kPH: return launch_bwd_tma_t<PL, kPH>(P, s, nsm);
-    case kPH | kINIT: return launch_bwd_tma_t<PL, kPH | kINIT>(P, s, nsm);
+    case 0: return launch_bwd_tma_t<PL, 0, false>(P, s, nsm);
+    case kINIT: return launch_bwd_tma_t<PL, kINIT, false>(P, s, nsm);
+    case kPH | kH2: return launch_bwd_tma_t<PL, kPH | kH2, false>(P, s, nsm);
+    case kPH: return launch_bwd_tma_t<PL, kPH, false>(P, s, nsm);
+    case kPH | kINIT: return launch_bwd_tma_t<PL, kPH | kINIT, false>(P, s, nsm);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <class PL>
+static cudaError_t dispatch_bwd_comp(const TmaBwdParams &P, cudaStream_t s, int nsm) {
+  static_assert(comp_plan<PL>(), "complement tile bit");
+  const bool h2 = (P.s2.m[0] | P.s2.m[1] | P.s2.lm[1]) != 0;
+  const int k = (P.has_phase ? kPH : 0) | (h2 ? kH2 : 0) | (P.init_lambda ? kINIT : 0);
+  if (P.comp < PL::TB) return cudaErrorInvalidValue;
+  switch (k) {
+    case kPH | kH2: return launch_bwd_tma_t<PL, kPH | kH2, true>(P, s, nsm);
+    case kPH: return launch_bwd_tma_t<PL, kPH, true>(P, s, nsm);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -1758,6 +2101,7 @@ static cudaError_t launch_xy_tma_t(const XyTmaParams &P, cudaStream_t s, int nsm
 cudaError_t QAOA_TMA_FN(launch_fwd_tma)(const TmaFwdParams &P, bool high, cudaStream_t s, int nsm) {
   if (P.c < 4 || P.c > 6) return cudaErrorInvalidValue;  // 16- to 64-amplitude segments
   if (!P.psi || ((uintptr_t)P.psi & 15u)) return cudaErrorInvalidValue;
+  if (P.comp) return high ? dispatch_fwd_comp<PlanTmaF13High>(P, s, nsm) : cudaErrorInvalidValue;
   return high ? dispatch_fwd<PlanTmaF13High>(P, s, nsm) : dispatch_fwd<PlanTmaF13Low>(P, s, nsm);
 }
 
@@ -1777,6 +2121,11 @@ cudaError_t QAOA_TMA_FN(launch_bwd_tma)(const TmaBwdParams &P, bool high, cudaSt
     if ((!P.cluster && (P.s1.lm[r] | P.s2.lm[r]) != 0) || __builtin_popcount(P.s1.lm[r]) > 1 ||
         __builtin_popcount(P.s2.lm[r]) > 1)
       return cudaErrorInvalidValue;
+  if (P.comp) {
+    if (!high || P.cluster == 1) return cudaErrorInvalidValue;
+    return P.cluster == 2 ? dispatch_bwd_comp<PlanTmaB13Comp>(P, s, nsm)
+                          : dispatch_bwd_comp<PlanTmaB12High>(P, s, nsm);
+  }
   if (P.cluster == 2) {  // a HIGH group of up to 9 qubits on one 512-thread CTA
     if (!high || P.c != 4 || P.h < 4) return cudaErrorInvalidValue;
     return dispatch_bwd<PlanTmaB13High>(P, s, nsm);
