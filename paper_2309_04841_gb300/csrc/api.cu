@@ -683,18 +683,25 @@ std::vector<PassOp> adjoint_schedule(int k, int p) {
   return ops;
 }
 
-// Reduced form of exp(-i b X) for the tiled passes (rot_tan): the form with
-// |t| <= 1 and the real factor it drops.
+// Reduced form of exp(-i b X) (rot_tan; kernels.h): the form with |t| <= 1 and
+// the real factor it drops.  The factor belongs to the multiplier as the kernels
+// hold it, rounded to Real: with 1 / sqrt(1 + t^2) of that t every rotation is
+// unitary (by an angle a rounding off), whereas the cosine of the exact angle
+// left the norm off by up to 3e-8 a rotation, the same for all n rotations of a
+// layer -- most of the error of a complex64 energy (LABS n = 27 p = 10:
+// 2.2e-6 -> 2.1e-7 relative).
 struct RedRot {
   double t;
   int form;
   double sigma;
 };
 
+template <typename Real>
 RedRot red_rot(double b) {
   const double c = cos(b), s = sin(b);
-  if (fabs(c) >= fabs(s)) return RedRot{s / c, 0, c};
-  return RedRot{c / s, 1, s};
+  const int form = fabs(c) >= fabs(s) ? 0 : 1;
+  const double t = (double)(Real)(form ? c / s : s / c);
+  return RedRot{t, form, copysign(1.0 / sqrt(1.0 + t * t), form ? s : c)};
 }
 
 double ipow_d(double x, int k) {
@@ -739,14 +746,14 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
     // (these plans hold every rotated bit in registers: no lane rotations)
     if (op.l1 >= 0) {
       P.s1 = G.high ? make_sweep<High>(G.rot, true) : make_sweep<Low>(G.rot, true);
-      const RedRot R = red_rot(bet[op.l1]);
+      const RedRot R = red_rot<Real>(bet[op.l1]);
       P.t1 = (Real)R.t;
       P.form1 = R.form;
       sig *= ipow_d(R.sigma, sweep_qubits(P.s1));
     }
     if (op.l2 >= 0) {
       P.s2 = G.high ? make_sweep<High>(G.rot, !two) : make_sweep<Low>(G.rot, !two);
-      const RedRot R = red_rot(bet[op.l2]);
+      const RedRot R = red_rot<Real>(bet[op.l2]);
       P.t2 = (Real)R.t;
       P.form2 = R.form;
     }
@@ -756,7 +763,7 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
       make_phase<Real>(P.ph, gam[op.lp], ct, stats, sig);
       sig = 1.0;
     }
-    if (op.l2 >= 0) sig *= ipow_d(red_rot(bet[op.l2]).sigma, sweep_qubits(P.s2));
+    if (op.l2 >= 0) sig *= ipow_d(red_rot<Real>(bet[op.l2]).sigma, sweep_qubits(P.s2));
     P.post_scale = (Real)1;
     if (&op == &ops.back()) {
       P.post_scale = (Real)sig;
@@ -803,7 +810,8 @@ qaoa_status tiled_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa
 template <typename Real, class Low, class High>
 qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                               const double *gam, const double *bet, int p, void *state, void *lam,
-                              const Ws &ws, double *d_grad_g, double *d_grad_b, bool half, cudaStream_t s) {
+                              const Ws &ws, const double *d_energy, double *d_grad_g, double *d_grad_b, bool half,
+                           cudaStream_t s) {
   using C2 = typename C2T<Real>::type;
   const int TB = Low::TB;
   const int m = half ? n - 1 : n;
@@ -827,7 +835,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
     // forms of exp(-i (-beta) X)
     P.s1 = G.high ? make_sweep<High>(G.rot, true) : make_sweep<Low>(G.rot, true);
     {
-      const RedRot R = red_rot(-bet[op.l1]);
+      const RedRot R = red_rot<Real>(-bet[op.l1]);
       P.t1 = (Real)R.t;
       P.form1 = R.form;
       for (int r = 0; r < Low::NR; ++r) {  // the kernel walks s1 upward
@@ -845,7 +853,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
     }
     if (op.l2 >= 0) {
       P.s2 = G.high ? make_sweep<High>(G.rot, false) : make_sweep<Low>(G.rot, false);
-      const RedRot R = red_rot(-bet[op.l2]);
+      const RedRot R = red_rot<Real>(-bet[op.l2]);
       P.t2 = (Real)R.t;
       P.form2 = R.form;
       for (int k = 0; k < Low::NR; ++k) {  // and s2 downward
@@ -863,6 +871,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
     if (uses_lanes(P.s1) || uses_lanes(P.s2))
       return fail(QAOA_ERR_INVALID_ARG, "internal: plan needs lane rotations");
     P.init_lambda = op.init;
+    P.energy = d_energy;
     P.partials = ws.partials;
     P.counter = ws.counter;
     const double N = (double)(1ull << m);
@@ -879,17 +888,18 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
 template <typename Real>
 qaoa_status tiled_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                            const double *gam, const double *bet, int p, void *state, void *lam,
-                           const Ws &ws, double *d_grad_g, double *d_grad_b, bool half, cudaStream_t s) {
+                           const Ws &ws, const double *d_energy, double *d_grad_g, double *d_grad_b, bool half,
+                           cudaStream_t s) {
   if constexpr (sizeof(Real) == 8) {
     if (n <= 14)
       return tiled_backward_pl<Real, PlanT9Low, PlanT9High>(n, cost, ct, stats, gam, bet, p, state, lam, ws,
-                                                            d_grad_g, d_grad_b, half, s);
+                                                            d_energy, d_grad_g, d_grad_b, half, s);
     if (n <= 16)
       return tiled_backward_pl<Real, PlanT10Low, PlanT10High>(n, cost, ct, stats, gam, bet, p, state, lam,
-                                                              ws, d_grad_g, d_grad_b, half, s);
+                                                              ws, d_energy, d_grad_g, d_grad_b, half, s);
   }
   return tiled_backward_pl<Real, typename BwdTB<Real>::Low, typename BwdTB<Real>::High>(
-      n, cost, ct, stats, gam, bet, p, state, lam, ws, d_grad_g, d_grad_b, half, s);
+      n, cost, ct, stats, gam, bet, p, state, lam, ws, d_energy, d_grad_g, d_grad_b, half, s);
 }
 
 // ---------------------------------------------------- TMA (complex64) path
@@ -917,19 +927,8 @@ struct TanRot {
 // Reduced form of exp(-i b X) in the twisted basis (b = -beta for the
 // adjoint): form 0 t = tan b, sigma = cos b; form 1 u = cot b, sigma = sin b.
 TanRot tan_rot(double beta, bool adjoint) {
-  const double b = adjoint ? -beta : beta;
-  const double c = cos(b), s = sin(b);
-  TanRot r;
-  if (fabs(c) >= fabs(s)) {
-    r.form = 0;
-    r.tau = (float)(s / c);
-    r.sigma = c;
-  } else {
-    r.form = 1;
-    r.tau = (float)(c / s);
-    r.sigma = s;
-  }
-  return r;
+  const RedRot r = red_rot<float>(adjoint ? -beta : beta);
+  return TanRot{(float)r.t, r.form, r.sigma};
 }
 
 float2 f2c(std::complex<double> z) { return make_float2((float)z.real(), (float)z.imag()); }
@@ -1018,7 +1017,8 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
 
 qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                          const double *gam, const double *bet, int p, void *state, void *lam,
-                         const Ws &ws, double *d_grad_g, double *d_grad_b, bool half, cudaStream_t s) {
+                         const Ws &ws, const double *d_energy, double *d_grad_g, double *d_grad_b, bool half,
+                           cudaStream_t s) {
   using Low = PlanTmaB12Low;
   using High = PlanTmaB12High;
   const int TB = Low::TB;
@@ -1111,6 +1111,7 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
     if ((uses_lanes(P.s1) || uses_lanes(P.s2)) && !G.cl)
       return fail(QAOA_ERR_INVALID_ARG, "internal: plan needs lane rotations");
     P.init_lambda = op.init;
+    P.energy = d_energy;
     P.untwist = &op == &ops.back();
     if (half && P.untwist) P.mirror = (1ull << n) - 1ull;
     P.partials = ws.partials;
@@ -1794,7 +1795,7 @@ qaoa_status qaoa_grad(int n, const void *d_costs, qaoa_cost_type ct, const qaoa_
     half = half && !adjoint_override();
     r = tma_forward(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, false, half, s);
     if (r != QAOA_OK) return r;
-    return tma_backward(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws, d_out + 2,
+    return tma_backward(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws, d_out, d_out + 2,
                         d_out + 2 + p, half, s);
   }
   r = st == QAOA_C64 ? tiled_forward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, half,
@@ -1804,9 +1805,9 @@ qaoa_status qaoa_grad(int n, const void *d_costs, qaoa_cost_type ct, const qaoa_
   if (r != QAOA_OK) return r;
   return st == QAOA_C64
              ? tiled_backward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws,
-                                     d_out + 2, d_out + 2 + p, half, s)
+                                     d_out, d_out + 2, d_out + 2 + p, half, s)
              : tiled_backward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws,
-                                      d_out + 2, d_out + 2 + p, half, s);
+                                      d_out, d_out + 2, d_out + 2 + p, half, s);
 }
 
 }  // extern "C"

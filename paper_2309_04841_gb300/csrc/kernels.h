@@ -171,6 +171,7 @@ struct alignas(64) TmaBwdParams {
   float w1[4], w2[4]; // |scale|^2 weights of the inner products taken in each round
   float wg;           // |scale|^2 weight of the d/d gamma inner product
   int has_phase, init_lambda;
+  const double *energy;  // E of the forward sweep (cost_shift)
   int untwist;  // last pass: psi back to the standard basis, lambda not stored
   uint64_t mirror;   // with untwist, nonzero (2^n - 1): psi[x] is also stored at its complement
   double out_scale;  // inner products times this before they are added

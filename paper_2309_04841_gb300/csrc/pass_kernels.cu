@@ -483,6 +483,7 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
     }
   }
   const Geom g = P.g;
+  const double fc = cost_shift(P.energy);
   const bool has1 = (P.s1.m[0] | P.s1.m[1] | P.s1.m[2]) != 0;
   const bool has2 = (P.s2.m[0] | P.s2.m[1] | P.s2.m[2]) != 0;
 
@@ -492,11 +493,11 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
     C2 v[NREG], w[NREG];
     load_tile<PL, 0, CP>(v, P.psi, g, base);
     if (P.init_lambda) {
-      // lambda = f psi: the gradient of E = <psi|f|psi> with respect to psi^*
+      // lambda = (f - E) psi: the gradient of <psi|f - E|psi> with respect to psi^*
       const AmpIndex<PL, 0, CP> ix(g, base);
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
-        const Real f = (Real)cost_d(P.cost, P.cost_kind, ix.at(r));
+        const Real f = (Real)(cost_d(P.cost, P.cost_kind, ix.at(r)) - fc);
         w[r] = mk<C2>(f * v[r].x, f * v[r].y);
       }
     } else {
@@ -518,7 +519,7 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
         const uint64_t x = ix.at(r);
-        const Real f = (Real)cost_d(P.cost, P.cost_kind, x);
+        const Real f = (Real)(cost_d(P.cost, P.cost_kind, x) - fc);
         raw += f * (w[r].x * v[r].y - w[r].y * v[r].x);
         const C2 ph = phase_factor(P.ph, tlo, thi, P.cost, P.cost_kind, x);
         v[r] = cmul(v[r], ph);

@@ -1124,12 +1124,12 @@ struct CostIdx {
 template <class PL, int R, bool CP, int M, class CI>
 __device__ __forceinline__ void unphase_round(float2 (&v)[PL::NREG], float2 (&w)[PL::NREG],
                                               const CostWord *cb, const TmaBwdParams &P,
-                                              const float2 *tab, float &ag, CI ci) {
+                                              const float2 *tab, float fc, float &ag, CI ci) {
   const uint32_t tt = thr_tile<PL, R>();
 #pragma unroll
   for (int r = 0; r < PL::NREG; ++r) {
     const uint32_t word = cb[ci(cost_slot<PL, R, CP>(tt, r))];
-    const float f = cost_val(P.cost_kind, word);
+    const float f = cost_val(P.cost_kind, word) - fc;
     ag += P.wg * f * (w[r].x * v[r].y - w[r].y * v[r].x);
     float2 ph = phase_of<M>(P.ph, P.cost_kind, tab, word);
     if constexpr (M == 1) ph = cmulf(ph, P.scl_phase);
@@ -1141,14 +1141,14 @@ __device__ __forceinline__ void unphase_round(float2 (&v)[PL::NREG], float2 (&w)
 template <class PL, int R, bool CP = false, class CI = CostIdx>
 __device__ __forceinline__ void unphase_any(float2 (&v)[PL::NREG], float2 (&w)[PL::NREG],
                                             const CostWord *cb, const TmaBwdParams &P,
-                                            const float2 *tab, float &ag, CI ci = CI()) {
+                                            const float2 *tab, float fc, float &ag, CI ci = CI()) {
   const int m = phase_m(P.ph);
   if (m == 2)
-    unphase_round<PL, R, CP, 2>(v, w, cb, P, tab, ag, ci);
+    unphase_round<PL, R, CP, 2>(v, w, cb, P, tab, fc, ag, ci);
   else if (m == 3)
-    unphase_round<PL, R, CP, 3>(v, w, cb, P, tab, ag, ci);
+    unphase_round<PL, R, CP, 3>(v, w, cb, P, tab, fc, ag, ci);
   else
-    unphase_round<PL, R, CP, 1>(v, w, cb, P, tab, ag, ci);
+    unphase_round<PL, R, CP, 1>(v, w, cb, P, tab, fc, ag, ci);
 }
 
 // The state tiles use the TMA 128-byte swizzle (16- to 64-amplitude segments).
@@ -1248,6 +1248,7 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
 
   if (tid == 0 && blockIdx.x < P.ntiles) issue(blockIdx.x, need_cost);
 
+  const float fc = need_cost ? (float)cost_shift(P.energy) : 0.f;
   FF acc1, accg, acc2;  // this thread's gradient terms
   CompCtx cx;
   if constexpr (CP) {
@@ -1270,11 +1271,11 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
     if constexpr (CP) cx.eps = ((((P.comp - 1) >> 1) + twist_base<PL, 0>(T)) & 1) ? -1.f : 1.f;
     lds_round<PL, 0, SW, CP>(v, bv);
     if constexpr (INIT) {
-      // lambda = f psi: the derivative of E = <psi|f|psi> with respect to psi^*
+      // lambda = (f - E) psi: the derivative of <psi|f - E|psi> with respect to psi^*
       const uint32_t tt = thr_tile<PL, 0>();
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
-        const float f = cost_val(P.cost_kind, cb[cost_slot<PL, 0, CP>(tt, r)]);
+        const float f = cost_val(P.cost_kind, cb[cost_slot<PL, 0, CP>(tt, r)]) - fc;
         w[r] = f2(f * v[r].x, f * v[r].y);
       }
     } else {
@@ -1297,7 +1298,7 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
     }
     if constexpr (PH) {
       // d/d gamma: Im <lambda| f |psi>, then un-phase both vectors
-      unphase_any<PL, NR - 1, CP>(v, w, cb, P, tab, ag);
+      unphase_any<PL, NR - 1, CP>(v, w, cb, P, tab, fc, ag);
       if constexpr (late_cost)
         release_cost(T);
       else if constexpr (!H2)
@@ -1548,6 +1549,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_pair(const __grid_constant_
 
   if (tid == 0 && first < nunits) issue(first, need_cost);
 
+  const float fc = need_cost ? (float)cost_shift(P.energy) : 0.f;
   FF acc1, accg, acc2;
   int i = 0;
   for (;; ++i) {
@@ -1567,7 +1569,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_pair(const __grid_constant_
       const uint32_t tt = thr_tile<PL, 0>();
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
-        const float f = cost_val(P.cost_kind, cb[tt | pdep(r, PL::reg(0))]);
+        const float f = cost_val(P.cost_kind, cb[tt | pdep(r, PL::reg(0))]) - fc;
         w[r] = f2(f * v[r].x, f * v[r].y);
       }
     } else {
@@ -1591,7 +1593,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_pair(const __grid_constant_
     if constexpr (H2) signal(remote(&xbar[2]), (P.s1.m[1] | P.s1.lm[1]) ? __float_as_uint(a1) : fold_bits(v, w));
     if constexpr (!PH && !H2) release(U);
     if constexpr (PH) {
-      unphase_any<PL, 1>(v, w, cb, P, tab, ag, PairCostIdx());
+      unphase_any<PL, 1>(v, w, cb, P, tab, fc, ag, PairCostIdx());
       if constexpr (!H2) release(U);
     }
     if constexpr (H2) {
