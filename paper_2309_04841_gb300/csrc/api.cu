@@ -440,12 +440,21 @@ uint32_t comp_mark(int n, const qaoa_cost_stats *st) {
 // passes are as long as one tile takes, and the box pairs make that longer:
 // complex64 n = 18 p = 20 gradient 717 us on half vectors, 653 us on full ones.
 constexpr int kHalfMinN64 = 21, kHalfMinN128 = 20;
+// On chip (small_kernels.cu) from the smallest register tile on.
+constexpr int kHalfMinN = 4;
 
 // (an adjoint plan asked for by environment variable is one of the full vector)
 bool adjoint_override() { return adjoint_wide_mode() != 1 || adjoint_pairs_mode() != 0; }
 
-bool half_vector(int n, qaoa_state_type st, const qaoa_cost_stats *stats, int init_plus) {
-  return n >= (st == QAOA_C64 ? kHalfMinN64 : kHalfMinN128) && init_plus && stats && stats->reserved != 0 && stats->reserved == comp_mark(n, stats);
+bool comp_symmetric(int n, const qaoa_cost_stats *stats, int init_plus) {
+  return n >= kHalfMinN && init_plus && stats && stats->reserved != 0 && stats->reserved == comp_mark(n, stats);
+}
+
+bool half_tiled(int n, qaoa_state_type st) { return n >= (st == QAOA_C64 ? kHalfMinN64 : kHalfMinN128); }
+
+// The on-chip kernels: n <= 12, and complex64 n = 13 where half of it is 12 bits.
+bool small_path(int n, qaoa_state_type st, bool symmetric) {
+  return n <= kSmallMaxN || (n == kSmallMaxN + 1 && symmetric && st == QAOA_C64);
 }
 
 // Groups of a half vector of m index bits: the LOW group, then HIGH groups of
@@ -505,18 +514,6 @@ Geom make_geom(int n, const Group &G, int TB) {
   return g;
 }
 
-template <typename Real>
-SmallLayer<Real> small_layer(double gamma, double beta) {
-  SmallLayer<Real> L;
-  L.cb = (Real)cos(beta);
-  L.sb = (Real)sin(beta);
-  const double g2 = gamma / kTwoPi;
-  L.g2pi = g2;
-  L.g_hi = (float)g2;
-  L.g_lo = (float)(g2 - (double)L.g_hi);
-  return L;
-}
-
 int cost_kind(qaoa_cost_type ct) { return (int)ct; }
 
 double cost_bytes(qaoa_cost_type ct) {
@@ -526,83 +523,79 @@ double cost_bytes(qaoa_cost_type ct) {
 // ----------------------------------------------------------- small path
 
 template <typename Real>
-qaoa_status small_forward(int n, const void *cost, qaoa_cost_type ct, double fmin,
-                          const double *gam, const double *bet, int p, void *state, int init_plus,
-                          double *d_out, cudaStream_t s) {
+SmallJob<Real> small_job(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats, void *state,
+                         bool half) {
   using C2 = typename C2T<Real>::type;
-  for (int l0 = 0; l0 < p; l0 += kSmallMaxLayers) {
-    const int nl = (p - l0) < kSmallMaxLayers ? (p - l0) : kSmallMaxLayers;
-    SmallParams<Real> P;
-    memset(&P, 0, sizeof(P));
-    P.psi = reinterpret_cast<C2 *>(state);
-    P.lam = nullptr;
-    P.cost = cost;
-    P.cost_kind = cost_kind(ct);
-    P.n = n;
-    P.nl = nl;
-    P.mode = 0;
-    P.init_plus = (l0 == 0) && init_plus;
-    P.amp = (Real)(1.0 / sqrt(ldexp(1.0, n)));
-    P.reduce = (l0 + nl == p) && d_out != nullptr;
-    P.fmin_d = fmin;
-    P.out = d_out;
-    for (int i = 0; i < nl; ++i) P.L[i] = small_layer<Real>(gam[l0 + i], bet[l0 + i]);
-    LAUNCH("small", 2.0 * sizeof(C2) * (double)(1 << n), s, launch_small(P, s));
+  SmallJob<Real> J;
+  memset(&J, 0, sizeof(J));
+  J.psi = reinterpret_cast<C2 *>(state);
+  J.cost = cost;
+  J.cost_kind = cost_kind(ct);
+  J.n = n;
+  J.half = half;
+  J.amp = (Real)(1.0 / sqrt(ldexp(1.0, n)));
+  J.fmin_d = stats->f_min;
+  small_digits(J, stats->f_min, stats->f_max, stats->step_log2);
+  return J;
+}
+
+template <typename Real>
+qaoa_status small_launch(SmallJob<Real> &J, const double *gam, const double *bet, int nl, double vectors,
+                         cudaStream_t s) {
+  SmallLayer<Real> L[SmallTile<Real>::kMaxLayers];
+  for (int i = 0; i < nl; ++i) L[i] = small_layer<Real>(gam[i], bet[i], J.n, J.half);
+  J.nl = nl;
+  LAUNCH("small", vectors * 2.0 * sizeof(Real) * (double)(1 << J.n), s, launch_small(J, L, s));
+  return QAOA_OK;
+}
+
+template <typename Real>
+qaoa_status small_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
+                          const double *gam, const double *bet, int p, void *state, int init_plus,
+                          double *d_out, bool half, cudaStream_t s) {
+  constexpr int ML = SmallTile<Real>::kMaxLayers;
+  for (int l0 = 0; l0 < p; l0 += ML) {
+    const int nl = (p - l0) < ML ? (p - l0) : ML;
+    SmallJob<Real> J = small_job<Real>(n, cost, ct, stats, state, half);
+    J.init_plus = (l0 == 0) && init_plus;
+    J.reduce = (l0 + nl == p) && d_out != nullptr;
+    J.out = d_out;
+    const qaoa_status st = small_launch(J, gam + l0, bet + l0, nl, 2.0, s);
+    if (st != QAOA_OK) return st;
   }
   return QAOA_OK;
 }
 
 template <typename Real>
-qaoa_status small_grad(int n, const void *cost, qaoa_cost_type ct, double fmin, const double *gam,
-                       const double *bet, int p, void *state, void *lam, double *d_out,
+qaoa_status small_grad(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
+                       const double *gam, const double *bet, int p, void *state, void *lam, double *d_out, bool half,
                        cudaStream_t s) {
   using C2 = typename C2T<Real>::type;
-  const Real amp = (Real)(1.0 / sqrt(ldexp(1.0, n)));
-  if (p <= kSmallMaxLayers) {
-    SmallParams<Real> P;
-    memset(&P, 0, sizeof(P));
-    P.psi = reinterpret_cast<C2 *>(state);
-    P.lam = reinterpret_cast<C2 *>(lam);
-    P.cost = cost;
-    P.cost_kind = cost_kind(ct);
-    P.n = n;
-    P.nl = p;
-    P.mode = 1;
-    P.init_plus = 1;
-    P.amp = amp;
-    P.reduce = 1;
-    P.fmin_d = fmin;
-    P.out = d_out;
-    P.out_dg = d_out + 2;
-    P.out_db = d_out + 2 + p;
-    for (int i = 0; i < p; ++i) P.L[i] = small_layer<Real>(gam[i], bet[i]);
-    LAUNCH("small", 3.0 * sizeof(C2) * (double)(1 << n), s, launch_small(P, s));
-    return QAOA_OK;
+  constexpr int ML = SmallTile<Real>::kMaxLayers;
+  SmallJob<Real> J = small_job<Real>(n, cost, ct, stats, state, half);
+  J.lam = reinterpret_cast<C2 *>(lam);
+  if (p <= ML) {
+    J.mode = 1;
+    J.init_plus = 1;
+    J.reduce = 1;
+    J.out = d_out;
+    J.out_dg = d_out + 2;
+    J.out_db = d_out + 2 + p;
+    return small_launch(J, gam, bet, p, 3.0, s);
   }
-  qaoa_status st = small_forward<Real>(n, cost, ct, fmin, gam, bet, p, state, 1, d_out, s);
-  if (st != QAOA_OK) return st;
-  const int nchunks = (p + kSmallMaxLayers - 1) / kSmallMaxLayers;
-  for (int ci = nchunks - 1; ci >= 0; --ci) {
-    const int l0 = ci * kSmallMaxLayers;
-    const int nl = (p - l0) < kSmallMaxLayers ? (p - l0) : kSmallMaxLayers;
-    SmallParams<Real> P;
-    memset(&P, 0, sizeof(P));
-    P.psi = reinterpret_cast<C2 *>(state);
-    P.lam = reinterpret_cast<C2 *>(lam);
-    P.cost = cost;
-    P.cost_kind = cost_kind(ct);
-    P.n = n;
-    P.nl = nl;
-    P.mode = 2;
-    P.init_lambda = (ci == nchunks - 1);
-    P.amp = amp;
-    P.fmin_d = fmin;
-    P.out_dg = d_out + 2 + l0;
-    P.out_db = d_out + 2 + p + l0;
-    for (int i = 0; i < nl; ++i) P.L[i] = small_layer<Real>(gam[l0 + i], bet[l0 + i]);
-    LAUNCH("small", 4.0 * sizeof(C2) * (double)(1 << n), s, launch_small(P, s));
+  qaoa_status st = small_forward<Real>(n, cost, ct, stats, gam, bet, p, state, 1, d_out, half, s);
+  const int nchunks = (p + ML - 1) / ML;
+  for (int ci = nchunks - 1; ci >= 0 && st == QAOA_OK; --ci) {
+    const int l0 = ci * ML;
+    const int nl = (p - l0) < ML ? (p - l0) : ML;
+    J.mode = 2;
+    J.out = d_out;
+    J.init_lambda = (ci == nchunks - 1);
+    J.out_dg = d_out + 2 + l0;
+    J.out_db = d_out + 2 + p + l0;
+    st = small_launch(J, gam + l0, bet + l0, nl, 4.0, s);
   }
-  return QAOA_OK;
+  return st;
 }
 
 // ----------------------------------------------------------- tiled path
@@ -790,7 +783,7 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
 // complex128 at n <= 16: tiles small enough to spread the FP64-bound passes
 // over more SMs, with no more groups than the 4096-amplitude tiles (the
 // partial sums of the tiles fit the workspace: 2^(16-9) * 3 doubles)
-// half: a half vector (half_vector); whole: the last pass writes both halves
+// half: a half vector (comp_symmetric); whole: the last pass writes both halves
 template <typename Real>
 qaoa_status tiled_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                           const double *gam, const double *bet, int p, void *state, int init_plus,
@@ -934,7 +927,7 @@ TanRot tan_rot(double beta, bool adjoint) {
 float2 f2c(std::complex<double> z) { return make_float2((float)z.real(), (float)z.imag()); }
 
 // untwist: leave the final state in the standard basis, whole (the adjoint
-// instead continues from the twisted one); half: a half vector (half_vector).
+// instead continues from the twisted one); half: a half vector (comp_symmetric).
 qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                         const double *gam, const double *bet, int p, void *state, int init_plus,
                         const Ws &ws, double *d_out, bool untwist, bool half, cudaStream_t s) {
@@ -1169,6 +1162,7 @@ bool dyadic_scale(const double *w, size_t m, int *e_out) {
 
 namespace qaoa {
 void set_last_error(const char *msg) { fail(QAOA_OK, msg); }
+bool comp_symmetric_stats(int n, const qaoa_cost_stats *stats) { return comp_symmetric(n, stats, 1); }
 qaoa_status builtin_scratch(void **ptr, size_t *bytes);  // noalloc.cu
 }  // namespace qaoa
 
@@ -1459,13 +1453,15 @@ qaoa_status qaoa_simulate(int n, const void *d_costs, qaoa_cost_type ct, const q
   r = get_ws(n, d_work, work_bytes, ws);
   if (r != QAOA_OK) return r;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (n <= kSmallMaxN) {
-    return st == QAOA_C64
-               ? small_forward<float>(n, d_costs, ct, stats->f_min, gammas, betas, p, d_state, init_plus, d_out, s)
-               : small_forward<double>(n, d_costs, ct, stats->f_min, gammas, betas, p, d_state, init_plus, d_out, s);
+  bool half = comp_symmetric(n, stats, init_plus);
+  if (small_path(n, st, half)) {
+    return st == QAOA_C64 ? small_forward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus,
+                                                 d_out, half, s)
+                          : small_forward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus,
+                                                  d_out, half, s);
   }
   CK(cudaMemsetAsync(ws.err, 0, sizeof(unsigned), s), "memset error word");
-  const bool half = half_vector(n, st, stats, init_plus);
+  half = half && half_tiled(n, st);
   if (st == QAOA_C64 && tma_ok(ct))
     return tma_forward(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws, d_out, true, half, s);
   return st == QAOA_C64 ? tiled_forward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws,
@@ -1783,16 +1779,17 @@ qaoa_status qaoa_grad(int n, const void *d_costs, qaoa_cost_type ct, const qaoa_
   r = get_ws(n, d_work, work_bytes, ws);
   if (r != QAOA_OK) return r;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (n <= kSmallMaxN) {
+  bool half = comp_symmetric(n, stats, 1);
+  if (st == QAOA_C64 && tma_ok(ct) && n > kSmallMaxN) half = half && !adjoint_override();
+  if (small_path(n, st, half)) {
     return st == QAOA_C64
-               ? small_grad<float>(n, d_costs, ct, stats->f_min, gammas, betas, p, d_state, d_lambda, d_out, s)
-               : small_grad<double>(n, d_costs, ct, stats->f_min, gammas, betas, p, d_state, d_lambda, d_out, s);
+               ? small_grad<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, d_out, half, s)
+               : small_grad<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, d_out, half, s);
   }
+  half = half && half_tiled(n, st);
   CK(cudaMemsetAsync(d_out + 2, 0, sizeof(double) * 2 * (size_t)p, s), "memset grad");
   CK(cudaMemsetAsync(ws.err, 0, sizeof(unsigned), s), "memset error word");
-  bool half = half_vector(n, st, stats, 1);
   if (st == QAOA_C64 && tma_ok(ct)) {
-    half = half && !adjoint_override();
     r = tma_forward(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, false, half, s);
     if (r != QAOA_OK) return r;
     return tma_backward(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws, d_out, d_out + 2,

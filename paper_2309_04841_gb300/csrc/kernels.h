@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include "qaoa_common.cuh"
 
 namespace qaoa {
@@ -260,9 +262,73 @@ cudaError_t launch_xy_gate(void *psi, bool c128, int n, int i, int j, double tb2
                            cudaStream_t s, int nsm);
 cudaError_t launch_dicke(void *psi, bool c128, int n, int k, double amp, cudaStream_t s, int nsm);
 
-cudaError_t launch_small_batch(const SmallJob<float> *d_jobs, int count, int max_n, cudaStream_t s);
-cudaError_t launch_small_batch(const SmallJob<double> *d_jobs, int count, int max_n, cudaStream_t s);
-cudaError_t launch_small(const SmallParams<float> &P, cudaStream_t s);
-cudaError_t launch_small(const SmallParams<double> &P, cudaStream_t s);
+// The phase tables of a job (entries, ndig, shift, fmin) from its cost type and
+// statistics.  Computing a phase takes about as long as 10 of the products that
+// two tables add per amplitude: the cheapest of computing all N, one table and two.
+template <typename Real>
+void small_digits(SmallJob<Real> &J, double f_min, double f_max, unsigned step_log2) {
+  J.entries = J.ndig = 0;
+  const int d = small_dims(J.n, J.half);
+  // one warp with fewer threads at work than it has lanes: they compute the phases for each other
+  J.by_x = 1 << (d - SmallTile<Real>::eb(d)) < 32;
+  if (J.by_x) {
+    J.entries = 1 << d;
+    return;
+  }
+  if (J.cost_kind != kCostI32 && J.cost_kind != kCostU16) return;
+  const int shift = step_log2 < 31u ? (int)step_log2 : 0;
+  const double top = std::floor((f_max - f_min) / std::ldexp(1.0, shift));  // the largest d
+  if (!(top >= 0.0 && top < 8192.0 && f_min >= -2147483648.0 && f_max <= 2147483647.0)) return;
+  const int N = 1 << d, one = (int)top + 1, hi = (int)top / 64 + 1;
+  const int t1 = 10 * one, t2 = 10 * (64 + hi) + N, most = kSmallTableBytes / (2 * (int)sizeof(Real));
+  if (t1 <= t2 && t1 < 10 * N && one <= most) {
+    J.entries = one;
+  } else if (t2 < 10 * N && 64 + hi <= most) {
+    J.entries = 64 + hi;
+    J.ndig = hi;
+  }
+  J.shift = shift;
+  J.fmin = (int)f_min;
+}
+// count jobs on d index bits (small_dims) each, of max_nl layers at most
+cudaError_t launch_small_batch(const SmallJob<float> *d_jobs, int count, int d, int max_nl, cudaStream_t s);
+cudaError_t launch_small(const SmallJob<float> &J, const SmallLayer<float> *layers, cudaStream_t s);
+cudaError_t launch_small(const SmallJob<double> &J, const SmallLayer<double> *layers, cudaStream_t s);
+
+// The layer data of angles (gamma, beta) for n qubits.
+template <typename Real>
+SmallLayer<Real> small_layer(double gamma, double beta, int n, int half) {
+  SmallLayer<Real> L;
+  const double c = std::cos(beta), s = std::sin(beta);
+  L.form = std::fabs(c) >= std::fabs(s) ? 0 : 1;
+  L.tau = (Real)(L.form ? c / s : s / c);
+  // the factor of one rotation by the rounded tau (unitary); the adjoint's is its negative in form 1
+  const double t = (double)L.tau, sigma = std::copysign(1.0 / std::sqrt(1.0 + t * t), L.form ? s : c);
+  double pw[2 * (kSmallMaxN + 1) + 1];  // powers of sigma
+  pw[0] = 1.0;
+  for (int i = 1; i <= 2 * (kSmallMaxN + 1); ++i) pw[i] = pw[i - 1] * sigma;
+  const double all = pw[n];
+  L.sig = (Real)all;
+  L.sig_adj = (Real)(L.form && (n & 1) ? -all : all);
+  L.wg = (Real)(all * all);
+  using T = SmallTile<Real>;
+  const int d = small_dims(n, half), R = T::rounds(d);
+  for (int up = 0; up < 2; ++up) {
+    int done = 0;
+    for (int i = 0; i < T::kMaxRounds; ++i) {
+      L.w[up][i] = (Real)pw[2 * done];
+      if (i < R) done += popc_c(T::mask(d, up ? i : R - 1 - i));
+      if (i == 0) {
+        L.w_comp[up] = (Real)pw[2 * done];
+        done += half;
+      }
+    }
+  }
+  const double g2 = gamma / 6.283185307179586476925286766559;
+  L.g2pi = g2;
+  L.g_hi = (float)g2;
+  L.g_lo = (float)(g2 - (double)L.g_hi);
+  return L;
+}
 
 }  // namespace qaoa

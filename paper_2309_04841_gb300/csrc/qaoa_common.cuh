@@ -221,15 +221,61 @@ struct BwdParams {
   PhaseData<Real> ph;     // un-phase data (exp(+i g f))
 };
 
-// Per-layer data of the single-CTA small-n kernels.
+// ---- single-CTA kernels (small_kernels.cu)
+constexpr int kSmallMaxN = 12;  // most index bits one CTA holds
+constexpr int kSmallMaxLayers = 128;  // most layers of a request that the server batches
+
+// A register tile of d index bits holds 2^eb amplitudes a thread: few where that
+// fills more of a warp, or more warps.  complex128 takes fewer than complex64:
+// its phases are long dependent chains, which only other warps overlap.  Its
+// rounds, the lowest register bit of round k, and (bit j: register bit j) the
+// index bits that round k rotates: eb k .. eb (k + 1) - 1.
+__host__ __device__ constexpr int small_dims(int n, int half) { return n - half; }
 template <typename Real>
-struct SmallLayer {
-  Real cb, sb;        // cos(beta), sin(beta)
-  float g_hi, g_lo;   // g / 2pi split (complex64)
-  double g2pi;        // g / 2pi (complex128)
+struct SmallTile {
+  static constexpr bool F64 = sizeof(Real) == 8;
+  static constexpr int kMaxRounds = F64 ? 7 : 6;
+  static constexpr int kMaxLayers = F64 ? 96 : 128;  // layers a launch
+  // exchange buffers: two save a barrier, where they fit
+  __host__ __device__ static constexpr int buffers(int d) { return F64 && d > 10 ? 1 : 2; }
+  static constexpr int kTermLayers = F64 ? 4 : 8;    // adjoint layers whose gradient terms are summed at once
+  __host__ __device__ static constexpr int eb(int d) {
+    return F64 ? (d <= 7 ? 1 : d <= 11 ? 2 : 3) : (d <= 6 ? 1 : d <= 9 ? 2 : 3);
+  }
+  __host__ __device__ static constexpr int threads(int d) { return d - eb(d) < 5 ? 32 : 1 << (d - eb(d)); }
+  __host__ __device__ static constexpr int rounds(int d) { return (d + eb(d) - 1) / eb(d); }
+  __host__ __device__ static constexpr int shift(int d, int k) {
+    return eb(d) * k < d - eb(d) ? eb(d) * k : d - eb(d);
+  }
+  __host__ __device__ static constexpr uint32_t mask(int d, int k) {
+    uint32_t m = 0;
+    for (int j = 0; j < eb(d); ++j)
+      if (shift(d, k) + j >= eb(d) * k) m |= 1u << j;
+    return m;
+  }
 };
 
-constexpr int kSmallMaxN = 12;
+// Phase tables: bytes, and layers whose tables are built at once.
+constexpr int kSmallTableBytes = 8192;
+template <typename Real>
+__host__ __device__ constexpr int small_table_layers(int entries) {
+  return kSmallTableBytes / (entries * 2 * (int)sizeof(Real));
+}
+
+// One layer.  Rotations are reduced (kernels.h): multiplier tau of form `form`,
+// sig / sig_adj the product of the dropped factors over the layer's rotations,
+// forward and adjoint.  An inner product taken part-way through an adjoint layer
+// is weighted by the square of the factors dropped so far in that layer: before
+// step i of the rounds upward / downward, w_comp at the complement rotation, wg
+// after the last rotation.
+template <typename Real>
+struct SmallLayer {
+  Real tau, sig, sig_adj, wg;
+  Real w[2][SmallTile<Real>::kMaxRounds], w_comp[2];  // [1] upward, [0] downward
+  int form;
+  float g_hi, g_lo;  // g / 2pi split (complex64)
+  double g2pi;       // g / 2pi (complex128)
+};
 
 // One request for the on-chip kernels (a launch of k_small runs one, a launch
 // of k_small_batch runs one per CTA from a device array of these).
@@ -241,29 +287,26 @@ struct SmallJob {
   int cost_kind;
   int n, nl;        // qubits; layers in this launch
   int mode;         // 0 forward, 1 forward + adjoint, 2 adjoint only
+  // integer costs of a small range, d = (f - fmin) >> shift: phases from a table
+  // by d (ndig 0), or from two, of 64 entries by its low digit and of ndig by the
+  // rest; entries of both.  by_x: a table by the amplitude, any costs.  entries 0:
+  // phases computed
+  int entries, ndig, shift, fmin, by_x;
+  int half;         // complement symmetry: n - 1 index bits are held
   int init_plus, init_lambda, reduce;
   Real amp;
   double fmin_d;
-  double *out;              // [E, O]
+  double *out;              // [E, O] (mode 2 with init_lambda reads E)
   double *out_dg, *out_db;  // per-layer gradient outputs
   const SmallLayer<Real> *L;
 };
-constexpr int kSmallMaxLayers = 128;
 
-template <typename Real>
+// Launch parameters with room for CAP layers (a launch copies all of it, so
+// short circuits take a small block).
+template <typename Real, int CAP>
 struct SmallParams {
-  using C2 = typename C2T<Real>::type;
-  C2 *psi, *lam;
-  const void *cost;
-  int cost_kind;
-  int n, nl;        // layers in this launch
-  int mode;         // 0 forward, 1 forward + backward (grad), 2 backward only
-  int init_plus, init_lambda, reduce;
-  Real amp;
-  double fmin_d;
-  double *out;      // forward: [E, O]; grad: also gamma/beta slots below
-  double *out_dg, *out_db;  // per-layer gradient outputs for this launch
-  SmallLayer<Real> L[kSmallMaxLayers];
+  SmallJob<Real> job;  // job.L unused
+  SmallLayer<Real> L[CAP];
 };
 
 }  // namespace qaoa

@@ -32,6 +32,7 @@
 
 namespace qaoa {
 void set_last_error(const char *msg);
+bool comp_symmetric_stats(int n, const qaoa_cost_stats *stats);  // api.cu
 }
 
 using namespace qaoa;
@@ -312,7 +313,6 @@ bool start_small_batch(qaoa_server *S, std::vector<Job *> &cand, int u) {
   Unit &U = S->units[u];
   std::vector<Job *> batch;
   size_t stage = 0, outs = 0;
-  int max_n = 1;
   for (Job *j : cand) {
     if ((int)batch.size() >= S->cfg.small_batch) break;
     const size_t need = sizeof(SmallJob<float>) + sizeof(SmallLayer<float>) * j->p;
@@ -320,7 +320,6 @@ bool start_small_batch(qaoa_server *S, std::vector<Job *> &cand, int u) {
     if (stage + need > U.h_stage_cap || outs + nd > U.h_out_cap) break;
     stage += need;
     outs += nd;
-    max_n = std::max(max_n, j->n);
     batch.push_back(j);
   }
   if (batch.empty()) return false;
@@ -365,7 +364,8 @@ bool start_small_batch(qaoa_server *S, std::vector<Job *> &cand, int u) {
   SmallLayer<float> *hl = reinterpret_cast<SmallLayer<float> *>(U.h_stage + sizeof(SmallJob<float>) * batch.size());
   const size_t layers_off = sizeof(SmallJob<float>) * batch.size();
   size_t lcur = 0, ocur = 0, scur = 0;
-  const double two_pi = 6.283185307179586476925286766559;
+  int max_nl = 1;
+  std::vector<SmallJob<float>> jobs(batch.size());
   for (size_t i = 0; i < batch.size(); ++i) {
     Job *j = batch[i];
     SmallJob<float> J;
@@ -376,12 +376,15 @@ bool start_small_batch(qaoa_server *S, std::vector<Job *> &cand, int u) {
     J.cost = S->d_arena + ce[i]->off;
     J.cost_kind = (int)ce[i]->ct;
     J.n = j->n;
+    J.half = comp_symmetric_stats(j->n, &ce[i]->stats);
+    max_nl = std::max(max_nl, j->p);
     J.nl = j->p;
     J.mode = j->want_grad ? 1 : 0;
     J.init_plus = 1;
     J.reduce = 1;
     J.amp = (float)(1.0 / std::sqrt(std::ldexp(1.0, j->n)));
     J.fmin_d = ce[i]->stats.f_min;
+    small_digits(J, ce[i]->stats.f_min, ce[i]->stats.f_max, ce[i]->stats.step_log2);
     double *d_o = reinterpret_cast<double *>(S->d_arena + o_out) + ocur;
     J.out = d_o;
     J.out_dg = d_o + 2;
@@ -389,27 +392,28 @@ bool start_small_batch(qaoa_server *S, std::vector<Job *> &cand, int u) {
     ocur += 2 + 2 * (size_t)j->p;
     J.L = reinterpret_cast<const SmallLayer<float> *>(S->d_arena + o_stage + layers_off) + lcur;
     for (int l = 0; l < j->p; ++l) {
-      SmallLayer<float> L;
-      L.cb = (float)std::cos(j->b[l]);
-      L.sb = (float)std::sin(j->b[l]);
-      const double g2 = j->g[l] / two_pi;
-      L.g2pi = g2;
-      L.g_hi = (float)g2;
-      L.g_lo = (float)(g2 - (double)L.g_hi);
-      hl[lcur + l] = L;
+      hl[lcur + l] = small_layer<float>(j->g[l], j->b[l], J.n, J.half);
     }
     lcur += j->p;
-    hj[i] = J;
+    jobs[i] = J;
     j->holds_cost = true;
     j->ckey = CostKey{j->problem, j->n, j->key};
     j->t_admit = now_s();
     j->state = kRunning;
     j->unit = u;
   }
+  // one launch for the jobs of each number of index bits
+  auto dims = [](const SmallJob<float> &J) { return small_dims(J.n, J.half); };
+  std::stable_sort(jobs.begin(), jobs.end(),
+                   [&](const SmallJob<float> &a, const SmallJob<float> &b) { return dims(a) < dims(b); });
+  std::copy(jobs.begin(), jobs.end(), hj);
   cudaError_t e = cudaMemcpyAsync(S->d_arena + o_stage, U.h_stage, stage, cudaMemcpyHostToDevice, U.stream);
-  if (e == cudaSuccess)
-    e = launch_small_batch(reinterpret_cast<const SmallJob<float> *>(S->d_arena + o_stage), (int)batch.size(),
-                           max_n, U.stream);
+  for (size_t i = 0, k; i < jobs.size() && e == cudaSuccess; i = k) {
+    for (k = i + 1; k < jobs.size() && dims(jobs[k]) == dims(jobs[i]); ++k) {
+    }
+    e = launch_small_batch(reinterpret_cast<const SmallJob<float> *>(S->d_arena + o_stage) + i, (int)(k - i),
+                           dims(jobs[i]), max_nl, U.stream);
+  }
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(U.h_out, S->d_arena + o_out, outs * sizeof(double), cudaMemcpyDeviceToHost, U.stream);
   if (e == cudaSuccess) e = cudaEventRecord(U.done, U.stream);

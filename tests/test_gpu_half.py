@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 
 from gpu_util import dev_np, torch
-from oracle import oracle
+import oracle
 from paper_2309_04841_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
@@ -30,7 +30,7 @@ def costs(Q, n, kind):
         return Q.labs_costs(n)
     if kind == "u16":
         return Q.labs_costs_u16(n)
-    e, w = I.maxcut_gnp(n, 0.4, graph_seed=n, weight_seed=n + 1)
+    e, w = I.maxcut_gnp(n, 0.4 if n >= 10 else 0.9, graph_seed=n, weight_seed=n + 1)
     return Q.maxcut_costs(n, e, w, Q.COST_F32 if kind == "f32" else Q.COST_F64)
 
 
@@ -38,10 +38,10 @@ def rel(a, b):
     return float(np.linalg.norm(a - b) / np.linalg.norm(b))
 
 
-# n: every count of groups (forward 13 + 9 rows + ..., adjoint 12 + 8 or 9), a group that takes only the complement,
+# n <= 13: on chip, every number of rounds and of bits in the last one.  n: every count of groups (forward 13 + 9 rows + ..., adjoint 12 + 8 or 9), a group that takes only the complement,
 # odd and even numbers of index bits, groups of exactly full rows
 @pytest.mark.parametrize("kind", ["i32", "u16", "f32", "f64"])
-@pytest.mark.parametrize("n", [14, 15, 16, 17, 19, 20, 21, 22, 23, 24])
+@pytest.mark.parametrize("n", [4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 19, 20, 21, 22, 23, 24])
 def test_half_vs_full(Q, n, kind):
     T = torch()
     p = 3
@@ -92,3 +92,25 @@ def test_mark(Q):
     a, _ = Q.simulate(fd, s, g, b)
     c, _ = Q.simulate(fd, full(Q, s), g, b)
     np.testing.assert_array_equal(dev_np(a), dev_np(c))
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 5, 7, 8, 9, 11, 12])
+@pytest.mark.parametrize("st", ["c64", "c128"])
+def test_on_chip_any_costs(Q, n, st):
+    # no symmetry: costs with linear terms, every register tile, against the oracle; p = 130 crosses a launch
+    terms = [(1, (q,)) for q in range(n)] + [(2, (0, n - 1))] * (n > 1) + [(-1, tuple(range(min(3, n))))]
+    f = oracle.costs_terms_int(n, terms).astype(float)
+    fd = Q.precompute_costs(n, terms)
+    s = Q.cost_stats_compute(fd)
+    assert s.reserved == 0 or n == 1  # (n = 1: the terms cancel)
+    for p in (1, 2, 130):
+        g, b = I.angles(p, n, 0, 0.3), I.angles(p, 50 + n)
+        tol = (5e-6 if st == "c64" else 1e-13) * max(1.0, p / 3)
+        psi = oracle.simulate(n, f, g, b)
+        x, _ = Q.simulate(fd, s, g, b, state_type=Q.C64 if st == "c64" else Q.C128)
+        assert np.linalg.norm(dev_np(x) - psi) < tol
+        E, dg, db = oracle.grad(n, f, g, b)
+        out = dev_np(Q.grad(fd, s, g, b, state_type=Q.C64 if st == "c64" else Q.C128))
+        ref = np.concatenate([dg, db])
+        assert np.linalg.norm(out[2:] - ref) <= 10 * tol * max(np.linalg.norm(ref), np.abs(f).max())
+        assert abs(out[0] - E) <= 10 * tol * np.abs(f).max()
