@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cmath>
 #include <complex>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -1158,6 +1159,24 @@ bool dyadic_scale(const double *w, size_t m, int *e_out) {
   return true;
 }
 
+// Terms for launch_walsh: weights in units of 2^-e, results times 2^-halve.
+WalshTerms walsh_terms(int n, qaoa_cost_type ct, void *out, int e, int halve) {
+  WalshTerms P;
+  memset(&P, 0, offsetof(WalshTerms, mask));
+  P.n = n;
+  P.out_kind = (int)ct;
+  P.shift = halve;
+  P.scale = ldexp(1.0, e + halve);
+  P.inv_scale = ldexp(1.0, -(e + halve));
+  P.out = out;
+  return P;
+}
+
+void walsh_add(WalshTerms &P, uint64_t mask, int64_t w) {
+  P.mask[P.nterms] = (uint32_t)mask;
+  P.w[P.nterms++] = w;
+}
+
 }  // namespace
 
 namespace qaoa {
@@ -1309,10 +1328,22 @@ qaoa_status qaoa_precompute_costs(int n, const qaoa_term *terms, size_t n_terms,
     if (ct == QAOA_COST_F32 && n_terms > (size_t)kTermChunk)
       return fail(QAOA_ERR_INVALID_ARG, "float32 costs take at most 1024 terms per call");
   }
+  const size_t nchunks = n_terms ? (n_terms + kTermChunk - 1) / kTermChunk : 1;
+  if (n >= kWalshBits && n <= 32 && mode != kTermF64) {  // sums in any order: by transform
+    for (size_t c = 0; c < nchunks; ++c) {
+      const size_t k0 = c * kTermChunk, k1 = std::min(k0 + (size_t)kTermChunk, n_terms);
+      WalshTerms P = walsh_terms(n, ct, d_costs, mode == kTermFixed ? e_fix : 0, 0);
+      P.accumulate = c > 0;
+      for (size_t k = k0; k < k1; ++k)
+        walsh_add(P, terms[k].mask, (int64_t)(mode == kTermFixed ? ldexp(w[k], e_fix) : w[k]));
+      LAUNCH("costs_terms", cost_bytes(ct) * (double)(1ull << n) * (c > 0 ? 2.0 : 1.0), s,
+             launch_walsh(P, mode == kTermFixed, s, nsm));
+    }
+    return QAOA_OK;
+  }
   static TermChunk P;  // large parameter block; calls are serialised below
   static std::mutex *mu = new std::mutex();
   std::lock_guard<std::mutex> lock(*mu);
-  const size_t nchunks = n_terms ? (n_terms + kTermChunk - 1) / kTermChunk : 1;
   for (size_t c = 0; c < nchunks; ++c) {
     memset(&P, 0, sizeof(P));
     P.n = n;
@@ -1380,6 +1411,30 @@ qaoa_status qaoa_maxcut_costs(int n, const int32_t *edges, const double *w, size
     if (i < 0 || j < 0 || i >= n || j >= n || i == j) return fail(QAOA_ERR_INVALID_ARG, "maxcut_costs: bad edge");
     wv[e] = w ? w[e] : 1.0;
     if (!std::isfinite(wv[e])) return fail(QAOA_ERR_INVALID_ARG, "maxcut_costs: non-finite weight");
+  }
+  // 2 f = sum w s_i s_j - sum w, by transform where the sums are exact (2 sum |w| in range)
+  if (n >= kWalshBits && n <= 32 && m < (size_t)kTermChunk) {
+    int e = 0;
+    double tot = 0.0;
+    bool whole = true;
+    for (size_t i = 0; i < m; ++i) {
+      tot += fabs(wv[i]);
+      whole = whole && wv[i] == nearbyint(wv[i]);
+    }
+    const bool wide = ct != QAOA_COST_I32;
+    if (wide ? dyadic_scale(wv.data(), m, &e) : (whole && tot < 1073741824.0)) {
+      WalshTerms P = walsh_terms(n, ct, d_costs, e, 1);
+      int64_t sum = 0;
+      for (size_t i = 0; i < m; ++i) {
+        const int64_t wi = (int64_t)ldexp(wv[i], e);
+        sum += wi;
+        walsh_add(P, (1ull << edges[2 * i]) ^ (1ull << edges[2 * i + 1]), wi);
+      }
+      walsh_add(P, 0, -sum);
+      cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+      LAUNCH("costs_maxcut", cost_bytes(ct) * (double)(1ull << n), s, launch_walsh(P, wide, s, num_sms()));
+      return QAOA_OK;
+    }
   }
   static EdgeChunk P;
   static std::mutex *mu = new std::mutex();

@@ -27,6 +27,17 @@ struct TermChunk {
   double wd[kTermChunk];
 };
 
+// Terms of exactly added weights for k_walsh: value(x) = (acc(x) >> shift), or
+// acc(x) * inv_scale for float outputs, acc the sum of +-w.
+struct WalshTerms {
+  int n, nterms, out_kind, accumulate, shift;
+  double scale, inv_scale;
+  void *out;
+  uint32_t mask[kTermChunk];
+  int64_t w[kTermChunk];
+};
+constexpr int kWalshBits = 13;  // index bits of a tile: the smallest n
+
 struct EdgeChunk {
   int n, m, mode, out_kind;
   double inv_scale;
@@ -37,6 +48,7 @@ struct EdgeChunk {
 };
 
 cudaError_t launch_terms(const TermChunk &P, cudaStream_t s, int nsm);
+cudaError_t launch_walsh(const WalshTerms &P, bool wide, cudaStream_t s, int nsm);
 cudaError_t launch_labs(int n, int32_t *out, cudaStream_t s, int nsm);
 cudaError_t launch_labs_u16(int n, uint16_t *out, cudaStream_t s, int nsm);
 cudaError_t launch_probs(int n, void *psi, bool c128, void *out, cudaStream_t s, int nsm);
