@@ -17,12 +17,14 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libqaoa.so")
 # (source, object, extra flags): the TMA kernels are compiled once per cost
 # element width (4 bytes: int32 / float32; 2 bytes: uint16) and the on-chip
-# kernels once per precision, in parallel.
+# and small-tile kernels once per precision, in parallel.
 UNITS = [("api.cu", "api.o", []), ("pass_kernels.cu", "pass_kernels.o", []),
          ("small_kernels.cu", "small_kernels.o", []),
          ("small_kernels.cu", "small_kernels_f64.o", ["-DQAOA_SMALL_F64"]), ("cost_kernels.cu", "cost_kernels.o", []),
          ("profile.cu", "profile.o", []), ("tma_kernels.cu", "tma_kernels.o", []),
          ("tma_kernels.cu", "tma_kernels_u16.o", ["-DQAOA_TMA_CW=2"]),
+         ("mid_kernels.cu", "mid_kernels.o", []),
+         ("mid_kernels.cu", "mid_kernels_f64.o", ["-DQAOA_MID_F64"]),
          ("noalloc.cu", "noalloc.o", []), ("serve.cu", "serve.o", []),
          ("xy_kernels.cu", "xy_kernels.o", [])]
 SOURCES = sorted({u[0] for u in UNITS})

@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "../../include/qaoa.h"
+#include "calls.h"
 #include "kernels.h"
 #include "qaoa_common.cuh"
 
@@ -150,33 +151,32 @@ qaoa_status check_angles(const double *g, const double *b, int p) {
 
 const double kTwoPi = 6.283185307179586476925286766559;
 
-// Phase data for multiplying by exp(-i g f) (times `scale` in table mode;
-// the computed mode leaves the scale to the kernel).
+// Phase data for multiplying by scale * exp(-i g f) (real scales only).
 template <typename Real>
-void make_phase(PhaseData<Real> &ph, double g, qaoa_cost_type ct, const qaoa_cost_stats *stats,
-                std::complex<double> scale = 1.0) {
-  using C2 = typename C2T<Real>::type;
+void make_phase(PhaseData<Real> &ph, double g, qaoa_cost_type ct, const qaoa_cost_stats *stats, double scale) {
   memset(&ph, 0, sizeof(ph));
-  const double range = stats ? stats->f_max - stats->f_min : 1e300;
-  if (integer_cost(ct) && stats && range >= 0 && range < 65536.0) {
-    ph.mode = 0;
-    ph.fmin = (int)stats->f_min;
-    ph.nhi = (int)(range / 256.0) + 1;
-    for (int j = 0; j < 256; ++j) {
-      const double a = g * (double)j;
-      ph.tab_lo[j] = C2{(Real)cos(a), (Real)-sin(a)};
-      const double b = g * ((double)stats->f_min + 256.0 * (double)j);
-      const std::complex<double> hv = std::complex<double>(cos(b), -sin(b)) * scale;
-      ph.tab_hi[j] = C2{(Real)hv.real(), (Real)hv.imag()};
-    }
+  ph.mode = 1;
+  ph.g2pi = g / kTwoPi;
+  ph.g_hi = (float)ph.g2pi;
+  ph.g_lo = (float)(ph.g2pi - (double)ph.g_hi);
+  ph.scl = (Real)scale;
+  if (!integer_cost(ct) || !stats) return;
+  const int shift = stats->step_log2 < 31 ? (int)stats->step_log2 : 0;
+  const double top = std::floor((stats->f_max - stats->f_min) / std::ldexp(1.0, shift));  // the largest d
+  if (!(top >= 0 && top < 262144.0) || !(stats->f_min >= -2147483648.0 && stats->f_max <= 2147483647.0)) return;
+  const int n1 = (int)top / 64 + 1;
+  ph.mode = 0;
+  ph.fmin = (int)stats->f_min;
+  ph.shift = shift;
+  if (64 + n1 <= kTileTable) {
+    ph.nd = 2;
+    ph.last = n1 - 1;
+    ph.entries = 64 + n1;
   } else {
-    ph.mode = 1;
-    const double g2 = g / kTwoPi;
-    ph.g2pi = g2;
-    ph.g_hi = (float)g2;
-    ph.g_lo = (float)(g2 - (double)ph.g_hi);
+    ph.nd = 3;
+    ph.last = (int)top / 4096;
+    ph.entries = 128 + ph.last + 1;
   }
-  ph.scl = (Real)(ph.mode == 1 ? scale.real() : 1.0);  // the tiled passes fold only real scales
 }
 
 // Digit tables of exp(-i g f) for the TMA passes (layout in PhaseDigits).
@@ -436,11 +436,6 @@ uint32_t comp_mark(int n, const qaoa_cost_stats *st) {
   return (uint32_t)(h >> 32) | 1u;
 }
 
-// The smallest n of the half-vector passes: from there the full vector has more
-// tiles than the GPU has SMs, so half of them take half the time.  Below, the
-// passes are as long as one tile takes, and the box pairs make that longer:
-// complex64 n = 18 p = 20 gradient 717 us on half vectors, 653 us on full ones.
-constexpr int kHalfMinN64 = 21, kHalfMinN128 = 20;
 // On chip (small_kernels.cu) from the smallest register tile on.
 constexpr int kHalfMinN = 4;
 
@@ -451,7 +446,19 @@ bool comp_symmetric(int n, const qaoa_cost_stats *stats, int init_plus) {
   return n >= kHalfMinN && init_plus && stats && stats->reserved != 0 && stats->reserved == comp_mark(n, stats);
 }
 
-bool half_tiled(int n, qaoa_state_type st) { return n >= (st == QAOA_C64 ? kHalfMinN64 : kHalfMinN128); }
+
+// The small-tile passes (mid_kernels.cu): up to n = 19, where they are ahead of the
+// larger tiles in every form (objective and gradient, p = 12: complex64 half vector
+// 403 -> 277 us, p = 4: complex128 half vector n = 18 655 -> 386 us); at n = 20
+// complex128 half vectors only (1928 -> 1027 us; the full vector 1928 against 2016
+// us, complex64 446 against 481 (half) and 653 us (full)).
+bool mid_path(int n, qaoa_state_type st, bool half) {
+  return n < kMidMaxN || (n == kMidMaxN && st == QAOA_C128 && half);
+}
+
+// Beyond, half vectors from n = 21 on in complex64: with fewer tiles than SMs a pass
+// is as long as one tile takes, and a box pair takes longer than a plain tile.
+bool half_path(int n, qaoa_state_type st) { return st == QAOA_C128 || n != kMidMaxN; }
 
 // The on-chip kernels: n <= 12, and complex64 n = 13 where half of it is 12 bits.
 bool small_path(int n, qaoa_state_type st, bool symmetric) {
@@ -461,12 +468,12 @@ bool small_path(int n, qaoa_state_type st, bool symmetric) {
 // Groups of a half vector of m index bits: the LOW group, then HIGH groups of
 // at most `cap` rotations (`wide`: up to as many groups of one more, on tiles
 // of 2^(TB+1) amplitudes, as save a group), the last of which also takes the
-// complement.  Segments of 2^c amplitudes, the widest that the rotations leave room
-// for (cmax at most).
-std::vector<Group> half_groups(int m, int TB, int cmax, bool wide) {
+// complement.  Segments of 2^c amplitudes, cmin <= c <= cmax, the widest that the
+// rotations leave room for.
+std::vector<Group> half_groups(int m, int TB, int cmin, int cmax, bool wide) {
   std::vector<Group> gs;
   gs.push_back(Group{false, TB, TB, (1u << TB) - 1u});
-  const int span = TB - 4;
+  const int span = TB - cmin;
   int left = m - TB + 1;  // rotations: the rows and the complement
   int k = (left + span - 1) / span, nwide = 0;
   if (wide && (left + span) / (span + 1) < k) {
@@ -478,7 +485,7 @@ std::vector<Group> half_groups(int m, int TB, int cmax, bool wide) {
     const bool last = g == k - 1, w = g >= k - nwide;
     const int tb = TB + (w ? 1 : 0);
     // as few as the others can take over, but a wide-segment group's fill where that holds them all
-    int cap = tb - 4;
+    int cap = tb - cmin;
     if (!w && nwide == 0 && left <= (k - g) * (TB - cmax)) cap = TB - cmax;
     const int take = std::min(cap, left);
     const int rows_new = take - (last ? 1 : 0);
@@ -487,7 +494,7 @@ std::vector<Group> half_groups(int m, int TB, int cmax, bool wide) {
     G.cl = w;
     G.comp = last;
     const int box = tb - (last ? 1 : 0);
-    int c = 4;
+    int c = cmin;
     while (!w && c < cmax && rows_new <= box - (c + 1)) ++c;
     G.c = c;
     const int rows = box - c;
@@ -712,6 +719,155 @@ int sweep_qubits(const Sweep &w) {
 
 int popc8(uint8_t m) { return __builtin_popcount((unsigned)m); }
 
+// ------------------------------------------------ small tiles (n <= 20)
+
+// The smallest tile that makes two groups: TB and TB - 2 rotations.
+int mid_tb(int n) { return n <= 14 ? 8 : n <= 16 ? 9 : n <= 18 ? 10 : 11; }
+
+std::vector<Group> mid_groups(int m, int TB, bool half) {
+  return half ? half_groups(m, TB, kMidC, kMidC, false) : plan_groups(m, TB, kMidC);
+}
+
+// Whether a pass may start beside the one before it.  complex128 passes past
+// n = 16 are bound by the FP64 pipe, which a waiting pass's tables then take from
+// the running one (n = 18 p = 20: 1660 us against 1409).
+bool mid_overlap(int n, bool half, bool f64) { return !f64 || n - (half ? 1 : 0) < 16; }
+
+template <typename Real>
+void mid_common(MidParams<Real> &P, int m, int TB, const Group &G, const void *cost, qaoa_cost_type ct, void *state,
+                const qaoa_cost_stats *stats) {
+  memset(&P, 0, sizeof(P));
+  P.psi = reinterpret_cast<typename C2T<Real>::type *>(state);
+  P.cost = cost;
+  P.cost_kind = cost_kind(ct);
+  P.g = make_geom(m, G, TB);
+  P.rot = G.rot;
+  P.post_scale = (Real)1;
+  P.fmin_d = stats ? stats->f_min : 0.0;
+}
+
+template <typename Real>
+qaoa_status mid_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats, const double *gam,
+                        const double *bet, int p, void *state, int init_plus, const Ws &ws, double *d_out, bool half,
+                        bool whole, bool overlap, cudaStream_t s) {
+  const int TB = mid_tb(n), m = half ? n - 1 : n;
+  const std::vector<Group> gs = mid_groups(m, TB, half);
+  if (gs.size() != 2) return fail(QAOA_ERR_INVALID_ARG, "internal: small tiles need two groups");
+  const std::vector<PassOp> ops = forward_schedule(2, p, init_plus != 0, d_out != nullptr);
+  if (d_out) CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
+  const double N = (double)(1ull << m);
+  MidParams<Real> P;
+  double sig = 1.0;  // as in tiled_forward_pl
+  for (const PassOp &op : ops) {
+    const Group &G = gs[op.group];
+    mid_common(P, m, TB, G, cost, ct, state, stats);
+    const int nrot = __builtin_popcount(G.rot);
+    if (op.l1 >= 0) {
+      const RedRot R = red_rot<Real>(bet[op.l1]);
+      P.t1 = (Real)R.t;
+      P.form1 = R.form;
+      sig *= ipow_d(R.sigma, nrot);
+    }
+    if (op.lp >= 0) {
+      make_phase<Real>(P.ph, gam[op.lp], ct, stats, sig);
+      sig = 1.0;
+    }
+    if (op.l2 >= 0) {
+      const RedRot R = red_rot<Real>(bet[op.l2]);
+      P.t2 = (Real)R.t;
+      P.form2 = R.form;
+      sig *= ipow_d(R.sigma, nrot);
+    }
+    P.kind = (op.l1 >= 0 ? 1 : 0) | (op.lp >= 0 ? 2 : 0) | (op.l2 >= 0 ? 4 : 0) | (op.reduce ? 8 : 0);
+    if (&op == &ops.back()) {
+      P.post_scale = (Real)sig;
+      if (half && whole) P.mirror = (1ull << n) - 1ull;
+    }
+    P.overlap = overlap && mid_overlap(n, half, sizeof(Real) == 8) && &op != &ops.front();
+    P.init_plus = op.init;
+    P.amp = (Real)(1.0 / sqrt(ldexp(1.0, n)));
+    P.partials = ws.partials;
+    P.counter = ws.counter;
+    P.out = d_out;
+    P.out_scale = half ? 2.0 : 1.0;
+    const double bytes = ((op.init ? 1.0 : 2.0) + (P.mirror ? 1.0 : 0.0)) * 2.0 * sizeof(Real) * N +
+                         (op.lp >= 0 || op.reduce ? cost_bytes(ct) * N : 0.0);
+    LAUNCH_N(G.high ? "fwd_mid_high" : "fwd_mid_low", bytes, s, launch_mid_fwd(P, G.high, TB, s));
+  }
+  return QAOA_OK;
+}
+
+// Partials of consecutive passes alternate between two places, so that the next
+// pass can add them while it writes its own.
+template <typename Real>
+qaoa_status mid_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats, const double *gam,
+                         const double *bet, int p, void *state, void *lam, const Ws &ws, const double *d_energy,
+                         double *d_grad_g, double *d_grad_b, bool half, bool overlap, cudaStream_t s) {
+  const int TB = mid_tb(n), m = half ? n - 1 : n, R = mid_rounds(TB);
+  const std::vector<Group> gs = mid_groups(m, TB, half);
+  if (gs.size() != 2) return fail(QAOA_ERR_INVALID_ARG, "internal: small tiles need two groups");
+  const std::vector<PassOp> ops = adjoint_schedule(2, p);
+  const double N = (double)(1ull << m);
+  MidParams<Real> P;
+  MidSums prev;
+  memset(&prev, 0, sizeof(prev));
+  double sig = 1.0;  // as in tiled_backward_pl
+  int flip = 0;
+  for (const PassOp &op : ops) {
+    const Group &G = gs[op.group];
+    mid_common(P, m, TB, G, cost, ct, state, stats);
+    P.lam = reinterpret_cast<typename C2T<Real>::type *>(lam);
+    MidSums sums;
+    memset(&sums, 0, sizeof(sums));
+    {
+      const RedRot Q = red_rot<Real>(-bet[op.l1]);
+      P.t1 = (Real)Q.t;
+      P.form1 = Q.form;
+      for (int k = 0; k < R; ++k) {
+        P.w1[k] = (Real)(sig * sig);
+        sig *= ipow_d(Q.sigma, __builtin_popcount(mid_mask(TB, G.rot, k)));
+      }
+      sums.out_b1 = d_grad_b + op.l1;
+    }
+    if (op.lp >= 0) {
+      P.wg = (Real)(sig * sig);
+      make_phase<Real>(P.ph, -gam[op.lp], ct, stats, sig);
+      sig = 1.0;
+      sums.out_g = d_grad_g + op.lp;
+    }
+    if (op.l2 >= 0) {
+      const RedRot Q = red_rot<Real>(-bet[op.l2]);
+      P.t2 = (Real)Q.t;
+      P.form2 = Q.form;
+      for (int i = 0; i < R; ++i) {
+        const int k = R - 1 - i;
+        P.w2[k] = (Real)(sig * sig);
+        sig *= ipow_d(Q.sigma, __builtin_popcount(mid_mask(TB, G.rot, k)));
+      }
+      sums.out_b2 = d_grad_b + op.l2;
+    }
+    P.kind = (op.lp >= 0 ? 2 : 0) | (op.l2 >= 0 ? 4 : 0) | (op.init ? 8 : 0);
+    if (&op == &ops.back()) {
+      P.post_scale = (Real)sig;
+      if (half) P.mirror = (1ull << n) - 1ull;
+    }
+    P.overlap = overlap && mid_overlap(n, half, sizeof(Real) == 8);  // (a forward pass is before the first)
+    P.energy = d_energy;
+    P.prev = prev;
+    P.partials = ws.partials + (flip ? 3 * P.g.ntiles : 0);
+    flip ^= 1;
+    const double bytes = ((op.init ? 3.0 : 4.0) + (P.mirror ? 1.0 : 0.0)) * 2.0 * sizeof(Real) * N +
+                         (op.lp >= 0 || op.init ? cost_bytes(ct) * N : 0.0);
+    LAUNCH_N(G.high ? "bwd_mid_high" : "bwd_mid_low", bytes, s, launch_mid_bwd(P, G.high, TB, s));
+    sums.partials = P.partials;
+    sums.ntiles = P.g.ntiles;
+    sums.scale = half ? 4.0 : 2.0;
+    prev = sums;
+  }
+  LAUNCH("bwd_mid_sum", 0.0, s, launch_mid_sum(prev, overlap, s));
+  return QAOA_OK;
+}
+
 template <typename Real, class Low, class High>
 qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                              const double *gam, const double *bet, int p, void *state, int init_plus,
@@ -719,7 +875,7 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
   using C2 = typename C2T<Real>::type;
   const int TB = Low::TB;
   const int m = half ? n - 1 : n;  // index bits of the vector that the passes hold
-  const std::vector<Group> gs = half ? half_groups(m, TB, kHighC, false) : plan_groups(n, TB, kHighC);
+  const std::vector<Group> gs = half ? half_groups(m, TB, kHighC, kHighC, false) : plan_groups(n, TB, kHighC);
   const std::vector<PassOp> ops = forward_schedule((int)gs.size(), p, init_plus != 0, d_out != nullptr);
   const int nsm = num_sms();
   if (d_out) CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
@@ -781,22 +937,13 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
   return QAOA_OK;
 }
 
-// complex128 at n <= 16: tiles small enough to spread the FP64-bound passes
-// over more SMs, with no more groups than the 4096-amplitude tiles (the
-// partial sums of the tiles fit the workspace: 2^(16-9) * 3 doubles)
 // half: a half vector (comp_symmetric); whole: the last pass writes both halves
 template <typename Real>
 qaoa_status tiled_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                           const double *gam, const double *bet, int p, void *state, int init_plus,
-                          const Ws &ws, double *d_out, bool half, bool whole, cudaStream_t s) {
-  if constexpr (sizeof(Real) == 8) {
-    if (n <= 14)
-      return tiled_forward_pl<Real, PlanT9Low, PlanT9High>(n, cost, ct, stats, gam, bet, p, state, init_plus,
-                                                           ws, d_out, half, whole, s);
-    if (n <= 16)
-      return tiled_forward_pl<Real, PlanT10Low, PlanT10High>(n, cost, ct, stats, gam, bet, p, state,
-                                                             init_plus, ws, d_out, half, whole, s);
-  }
+                          const Ws &ws, double *d_out, bool half, bool whole, bool overlap, cudaStream_t s) {
+  if (mid_path(n, sizeof(Real) == 8 ? QAOA_C128 : QAOA_C64, half))
+    return mid_forward<Real>(n, cost, ct, stats, gam, bet, p, state, init_plus, ws, d_out, half, whole, overlap, s);
   return tiled_forward_pl<Real, typename FwdTB<Real>::Low, typename FwdTB<Real>::High>(
       n, cost, ct, stats, gam, bet, p, state, init_plus, ws, d_out, half, whole, s);
 }
@@ -809,7 +956,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
   using C2 = typename C2T<Real>::type;
   const int TB = Low::TB;
   const int m = half ? n - 1 : n;
-  const std::vector<Group> gs = half ? half_groups(m, TB, kHighC, false) : plan_groups(n, TB, kHighC);
+  const std::vector<Group> gs = half ? half_groups(m, TB, kHighC, kHighC, false) : plan_groups(n, TB, kHighC);
   const std::vector<PassOp> ops = adjoint_schedule((int)gs.size(), p);
   const int nsm = num_sms();
   CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
@@ -883,15 +1030,10 @@ template <typename Real>
 qaoa_status tiled_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                            const double *gam, const double *bet, int p, void *state, void *lam,
                            const Ws &ws, const double *d_energy, double *d_grad_g, double *d_grad_b, bool half,
-                           cudaStream_t s) {
-  if constexpr (sizeof(Real) == 8) {
-    if (n <= 14)
-      return tiled_backward_pl<Real, PlanT9Low, PlanT9High>(n, cost, ct, stats, gam, bet, p, state, lam, ws,
-                                                            d_energy, d_grad_g, d_grad_b, half, s);
-    if (n <= 16)
-      return tiled_backward_pl<Real, PlanT10Low, PlanT10High>(n, cost, ct, stats, gam, bet, p, state, lam,
-                                                              ws, d_energy, d_grad_g, d_grad_b, half, s);
-  }
+                           bool overlap, cudaStream_t s) {
+  if (mid_path(n, sizeof(Real) == 8 ? QAOA_C128 : QAOA_C64, half))
+    return mid_backward<Real>(n, cost, ct, stats, gam, bet, p, state, lam, ws, d_energy, d_grad_g, d_grad_b, half,
+                              overlap, s);
   return tiled_backward_pl<Real, typename BwdTB<Real>::Low, typename BwdTB<Real>::High>(
       n, cost, ct, stats, gam, bet, p, state, lam, ws, d_energy, d_grad_g, d_grad_b, half, s);
 }
@@ -936,7 +1078,7 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
   using High = PlanTmaF13High;
   const int TB = Low::TB;
   const int m = half ? n - 1 : n;  // index bits of the vector that the passes hold
-  const std::vector<Group> gs = half ? half_groups(m, TB, kMaxSegBits, false) : tma_groups(n, TB);
+  const std::vector<Group> gs = half ? half_groups(m, TB, 4, kMaxSegBits, false) : tma_groups(n, TB);
   const std::vector<PassOp> ops = forward_schedule((int)gs.size(), p, init_plus != 0, d_out != nullptr);
   const int nsm = num_sms();
   if (d_out) CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
@@ -1018,7 +1160,7 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
   const int TB = Low::TB;
   const int m = half ? n - 1 : n;
   // HIGH groups of 9 new qubits where they save a group
-  const std::vector<Group> gs = half ? half_groups(m, TB, kMaxSegBits, true) : bwd_groups(n, TB);
+  const std::vector<Group> gs = half ? half_groups(m, TB, 4, kMaxSegBits, true) : bwd_groups(n, TB);
   const std::vector<PassOp> ops = adjoint_schedule((int)gs.size(), p);
   const int nsm = num_sms();
   CK(cudaMemsetAsync(ws.counter, 0, sizeof(unsigned), s), "memset counter");
@@ -1498,6 +1640,19 @@ qaoa_status qaoa_simulate(int n, const void *d_costs, qaoa_cost_type ct, const q
                           const double *gammas, const double *betas, int p, void *d_state,
                           qaoa_state_type st, int init_plus, void *d_work, size_t work_bytes,
                           double *d_out, qaoa_stream_t stream) {
+  return simulate_call(n, d_costs, ct, stats, gammas, betas, p, d_state, st, init_plus, d_work, work_bytes, d_out,
+                       true, stream);
+}
+
+}  // extern "C"
+
+namespace qaoa {
+// overlap: passes over small vectors may start before the one before them has
+// ended (launch_pdl in mid_kernels.cu)
+qaoa_status simulate_call(int n, const void *d_costs, qaoa_cost_type ct, const qaoa_cost_stats *stats,
+                          const double *gammas, const double *betas, int p, void *d_state, qaoa_state_type st,
+                          int init_plus, void *d_work, size_t work_bytes, double *d_out, bool overlap,
+                          qaoa_stream_t stream) {
   qaoa_status r = check_common(n, d_costs, ct, d_state, st);
   if (r != QAOA_OK) return r;
   if (!stats) return fail(QAOA_ERR_INVALID_ARG, "NULL stats");
@@ -1516,14 +1671,17 @@ qaoa_status qaoa_simulate(int n, const void *d_costs, qaoa_cost_type ct, const q
                                                   d_out, half, s);
   }
   CK(cudaMemsetAsync(ws.err, 0, sizeof(unsigned), s), "memset error word");
-  half = half && half_tiled(n, st);
-  if (st == QAOA_C64 && tma_ok(ct))
+  half = half && half_path(n, st);
+  if (st == QAOA_C64 && tma_ok(ct) && !mid_path(n, st, half))
     return tma_forward(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws, d_out, true, half, s);
   return st == QAOA_C64 ? tiled_forward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws,
-                                               d_out, half, true, s)
+                                               d_out, half, true, overlap, s)
                         : tiled_forward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, init_plus, ws,
-                                                d_out, half, true, s);
+                                                d_out, half, true, overlap, s);
 }
+}  // namespace qaoa
+
+extern "C" {
 
 // ------------------------------------------------------------- XY mixers
 
@@ -1824,6 +1982,17 @@ qaoa_status qaoa_grad(int n, const void *d_costs, qaoa_cost_type ct, const qaoa_
                       const double *gammas, const double *betas, int p, void *d_state, void *d_lambda,
                       qaoa_state_type st, void *d_work, size_t work_bytes, double *d_out,
                       qaoa_stream_t stream) {
+  return grad_call(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, st, d_work, work_bytes, d_out, true,
+                   stream);
+}
+
+}  // extern "C"
+
+namespace qaoa {
+qaoa_status grad_call(int n, const void *d_costs, qaoa_cost_type ct, const qaoa_cost_stats *stats,
+                      const double *gammas, const double *betas, int p, void *d_state, void *d_lambda,
+                      qaoa_state_type st, void *d_work, size_t work_bytes, double *d_out, bool overlap,
+                      qaoa_stream_t stream) {
   qaoa_status r = check_common(n, d_costs, ct, d_state, st);
   if (r != QAOA_OK) return r;
   if (!aligned16(d_lambda)) return fail(QAOA_ERR_INVALID_ARG, "lambda pointer NULL or not 16-byte aligned");
@@ -1841,25 +2010,25 @@ qaoa_status qaoa_grad(int n, const void *d_costs, qaoa_cost_type ct, const qaoa_
                ? small_grad<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, d_out, half, s)
                : small_grad<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, d_out, half, s);
   }
-  half = half && half_tiled(n, st);
   CK(cudaMemsetAsync(d_out + 2, 0, sizeof(double) * 2 * (size_t)p, s), "memset grad");
   CK(cudaMemsetAsync(ws.err, 0, sizeof(unsigned), s), "memset error word");
-  if (st == QAOA_C64 && tma_ok(ct)) {
+  half = half && half_path(n, st);
+  if (st == QAOA_C64 && tma_ok(ct) && (!mid_path(n, st, half) || adjoint_override())) {
     r = tma_forward(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, false, half, s);
     if (r != QAOA_OK) return r;
     return tma_backward(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws, d_out, d_out + 2,
                         d_out + 2 + p, half, s);
   }
   r = st == QAOA_C64 ? tiled_forward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, half,
-                                            false, s)
+                                            false, overlap, s)
                      : tiled_forward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, 1, ws, d_out, half,
-                                             false, s);
+                                             false, overlap, s);
   if (r != QAOA_OK) return r;
   return st == QAOA_C64
              ? tiled_backward<float>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws,
-                                     d_out, d_out + 2, d_out + 2 + p, half, s)
+                                     d_out, d_out + 2, d_out + 2 + p, half, overlap, s)
              : tiled_backward<double>(n, d_costs, ct, stats, gammas, betas, p, d_state, d_lambda, ws,
-                                      d_out, d_out + 2, d_out + 2 + p, half, s);
+                                      d_out, d_out + 2, d_out + 2 + p, half, overlap, s);
 }
 
-}  // extern "C"
+}  // namespace qaoa

@@ -62,8 +62,16 @@ cudaError_t launch_expect(int n, const void *psi, bool c128, const void *cost, i
                           double fmin, double *partials, unsigned *counter, double *out, int which,
                           cudaStream_t s, int nsm);
 
-// tb: log2 of the tile (float: 13 forward, 12 adjoint; double: 9, 10, 12
-// forward, 9, 10, 11 adjoint); other values fail with cudaErrorInvalidValue.
+// Small-tile passes (n <= 20), tb = 8 .. 11, one CTA a tile; k_mid_sum adds the
+// last adjoint pass's sums.
+cudaError_t launch_mid_fwd(const MidParams<float> &P, bool high, int tb, cudaStream_t s);
+cudaError_t launch_mid_fwd(const MidParams<double> &P, bool high, int tb, cudaStream_t s);
+cudaError_t launch_mid_bwd(const MidParams<float> &P, bool high, int tb, cudaStream_t s);
+cudaError_t launch_mid_bwd(const MidParams<double> &P, bool high, int tb, cudaStream_t s);
+cudaError_t launch_mid_sum(const MidSums &S, bool overlap, cudaStream_t s);
+
+// tb: log2 of the tile (float: 13 forward, 12 adjoint; double: 12 forward, 11
+// adjoint); other values fail with cudaErrorInvalidValue.
 cudaError_t launch_fwd(const FwdParams<float> &P, bool high, int tb, cudaStream_t s, int nsm);
 cudaError_t launch_fwd(const FwdParams<double> &P, bool high, int tb, cudaStream_t s, int nsm);
 cudaError_t launch_bwd(const BwdParams<float> &P, bool high, int tb, cudaStream_t s, int nsm);

@@ -166,6 +166,18 @@ __device__ __forceinline__ void unrot_regs_acc(C2 (&v)[1 << EB], C2 (&w)[1 << EB
   rot_regs<EB>(w, m, t, form);
 }
 
+// Cost value in the precision of the state.
+__device__ __forceinline__ void cost_r(const void *cost, int kind, uint64_t x, float &f) {
+  if (kind == kCostI32)
+    f = (float)__ldg(reinterpret_cast<const int *>(cost) + x);
+  else if (kind == kCostU16)
+    f = (float)__ldg(reinterpret_cast<const unsigned short *>(cost) + x);
+  else if (kind == kCostF32)
+    f = __ldg(reinterpret_cast<const float *>(cost) + x);
+  else
+    f = (float)__ldg(reinterpret_cast<const double *>(cost) + x);
+}
+
 // Cost value as a float pair hi + lo (exact for int32 and float32 costs,
 // ~2^-48 relative for float64 costs).
 __device__ __forceinline__ void cost_split(const void *cost, int kind, uint64_t x, float &hi,
@@ -194,45 +206,66 @@ __device__ __forceinline__ double cost_d(const void *cost, int kind, uint64_t x)
   return __ldg(reinterpret_cast<const double *>(cost) + x);
 }
 
-// exp(-i g f_x) for the layer described by ph (tables already in smem).
-__device__ __forceinline__ float2 phase_factor(const PhaseData<float> &ph, const float2 *tlo,
-                                               const float2 *thi, const void *cost, int kind,
-                                               uint64_t x) {
-  if (ph.mode == 0) {
-    const int f = kind == kCostU16 ? (int)__ldg(reinterpret_cast<const unsigned short *>(cost) + x)
-                                   : __ldg(reinterpret_cast<const int *>(cost) + x);
-    const uint32_t v = (uint32_t)(f - ph.fmin);
-    const uint32_t hi = min(v >> 8, 255u);
-    return cmul(thi[hi], tlo[v & 255u]);
-  }
-  // g f / 2pi as a float-float: p + e = g_hi * f_hi exactly (Dekker's
-  // two-product via fma), the small cross terms added once; only the
-  // fraction r in [-1/2, 1/2] reaches sincospi.
-  float fh, fl;
-  cost_split(cost, kind, x, fh, fl);
+__device__ __forceinline__ void cost_r(const void *cost, int kind, uint64_t x, double &f) {
+  f = cost_d(cost, kind, x);
+}
+
+// scl exp(-i g f), f = fh + fl: g f / 2pi as a float-float, p + e = g_hi * fh
+// exactly (Dekker's two-product via fma), the small cross terms added once; only
+// the fraction r in [-1/2, 1/2] reaches sincospi.
+__device__ __forceinline__ float2 phase_at(const PhaseData<float> &ph, float fh, float fl, float scl) {
   const float p = ph.g_hi * fh;
   const float e = fmaf(ph.g_hi, fh, -p);
   const float r = (p - rintf(p)) + (e + fmaf(ph.g_hi, fl, ph.g_lo * fh));
   float sn, cs;
   sincospif(2.0f * r, &sn, &cs);
-  return make_float2(cs * ph.scl, -sn * ph.scl);
+  return make_float2(cs * scl, -sn * scl);
 }
-
-__device__ __forceinline__ double2 phase_factor(const PhaseData<double> &ph, const double2 *tlo,
-                                                const double2 *thi, const void *cost, int kind,
-                                                uint64_t x) {
-  if (ph.mode == 0) {
-    const int f = kind == kCostU16 ? (int)__ldg(reinterpret_cast<const unsigned short *>(cost) + x)
-                                   : __ldg(reinterpret_cast<const int *>(cost) + x);
-    const uint32_t v = (uint32_t)(f - ph.fmin);
-    const uint32_t hi = min(v >> 8, 255u);
-    return cmul(thi[hi], tlo[v & 255u]);
-  }
-  const double t = ph.g2pi * cost_d(cost, kind, x);
+__device__ __forceinline__ double2 phase_at(const PhaseData<double> &ph, double f, double scl) {
+  const double t = ph.g2pi * f;
   const double r = t - rint(t);
   double sn, cs;
   sincospi(2.0 * r, &sn, &cs);
-  return make_double2(cs * ph.scl, -sn * ph.scl);
+  return make_double2(cs * scl, -sn * scl);
+}
+
+__device__ __forceinline__ float2 phase_int(const PhaseData<float> &ph, int f, float scl) {
+  const float fh = (float)f;
+  return phase_at(ph, fh, (float)((long long)f - (long long)fh), scl);
+}
+__device__ __forceinline__ double2 phase_int(const PhaseData<double> &ph, int f, double scl) {
+  return phase_at(ph, (double)f, scl);
+}
+
+// The phase tables in shared memory (mode 0).
+template <int NT, typename Real, typename C2>
+__device__ __forceinline__ void fill_phase(C2 *tab, const PhaseData<Real> &ph) {
+  const int lastbase = 64 * (ph.nd - 1);
+  for (int i = threadIdx.x; i < ph.entries; i += NT) {
+    const int digit = min(i >> 6, ph.nd - 1), j = (i - 64 * digit) << (6 * digit + ph.shift);
+    const bool last = i >= lastbase;
+    tab[i] = phase_int(ph, last ? ph.fmin + j : j, last ? ph.scl : (Real)1);
+  }
+}
+
+// exp(-i g f_x) for the layer described by ph (tables already in shared memory).
+template <typename Real, typename C2>
+__device__ __forceinline__ C2 phase_factor(const PhaseData<Real> &ph, const C2 *tab, const void *cost, int kind,
+                                           uint64_t x) {
+  if (ph.mode == 0) {
+    const int f = kind == kCostU16 ? (int)__ldg(reinterpret_cast<const unsigned short *>(cost) + x)
+                                   : __ldg(reinterpret_cast<const int *>(cost) + x);
+    const uint32_t d = (uint32_t)(f - ph.fmin) >> ph.shift;
+    if (ph.nd == 2) return cmul(tab[d & 63u], tab[64u + min(d >> 6, (uint32_t)ph.last)]);
+    return cmul(cmul(tab[d & 63u], tab[64u + ((d >> 6) & 63u)]), tab[128u + min(d >> 12, (uint32_t)ph.last)]);
+  }
+  if constexpr (sizeof(Real) == 4) {
+    float fh, fl;
+    cost_split(cost, kind, x, fh, fl);
+    return phase_at(ph, fh, fl, ph.scl);
+  } else {
+    return phase_at(ph, cost_d(cost, kind, x), ph.scl);
+  }
 }
 
 // Index of this thread's amplitude in register r of round R of the tile at
@@ -263,13 +296,13 @@ struct AmpIndex {
 
 template <class PL, int R, bool CP, typename Real, typename C2>
 __device__ __forceinline__ void apply_phase(C2 (&v)[PL::NREG], const PhaseData<Real> &ph,
-                                            const C2 *tlo, const C2 *thi, const void *cost,
-                                            int kind, const Geom &g, uint64_t base) {
+                                            const C2 *tab, const void *cost, int kind, const Geom &g,
+                                            uint64_t base) {
   const AmpIndex<PL, R, CP> ix(g, base);
 #pragma unroll
   for (int r = 0; r < PL::NREG; ++r) {
     const uint64_t x = ix.at(r);
-    v[r] = cmul(v[r], phase_factor(ph, tlo, thi, cost, kind, x));
+    v[r] = cmul(v[r], phase_factor(ph, tab, cost, kind, x));
   }
 }
 
@@ -304,10 +337,19 @@ __device__ __forceinline__ void accum_eo(const C2 (&v)[PL::NREG], const void *co
 #pragma unroll
   for (int r = 0; r < PL::NREG; ++r) {
     const uint64_t x = ix.at(r);
-    const double f = cost_d(cost, kind, x);
     const Real pr = v[r].x * v[r].x + v[r].y * v[r].y;
-    e += pr * (Real)f;
-    o += (f == fmin) ? pr : (Real)0;
+    Real f;
+    bool at_min;
+    cost_r(cost, kind, x, f);
+    if (sizeof(Real) == 8 || kind == kCostF64)
+      at_min = cost_d(cost, kind, x) == fmin;
+    else if (kind == kCostF32)
+      at_min = f == (Real)fmin;
+    else  // (no float64 conversion per amplitude)
+      at_min = (kind == kCostU16 ? (int)__ldg(reinterpret_cast<const unsigned short *>(cost) + x)
+                                 : __ldg(reinterpret_cast<const int *>(cost) + x)) == (int)fmin;
+    e += pr * f;
+    o += at_min ? pr : (Real)0;
   }
 }
 
@@ -374,16 +416,10 @@ __global__ void __launch_bounds__(PL::NT, 2) k_fwd(const __grid_constant__ FwdPa
   constexpr int NREG = PL::NREG, NR = PL::NR, EB = PL::EB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2 *tile = reinterpret_cast<C2 *>(smem_raw);
-  C2 *tlo = tile + (1 << PL::TB);
-  C2 *thi = tlo + 256;
-  double *red = reinterpret_cast<double *>(thi + 256);
+  C2 *tab = tile + (1 << PL::TB);
+  double *red = reinterpret_cast<double *>(tab + kTileTable);
 
-  if (P.has_phase && P.ph.mode == 0) {
-    for (int i = threadIdx.x; i < 256; i += PL::NT) {
-      tlo[i] = P.ph.tab_lo[i];
-      thi[i] = P.ph.tab_hi[i];
-    }
-  }
+  if (P.has_phase && P.ph.mode == 0) fill_phase<PL::NT>(tab, P.ph);
   const Geom g = P.g;
   const bool has1 = (P.s1.m[0] | P.s1.m[1] | P.s1.m[2]) != 0;
   const bool has2 = (P.s2.m[0] | P.s2.m[1] | P.s2.m[2]) != 0;
@@ -407,7 +443,7 @@ __global__ void __launch_bounds__(PL::NT, 2) k_fwd(const __grid_constant__ FwdPa
         xpose<PL, 1, 2>(v, tile);
         rot_regs<EB>(v, P.s1.m[2], P.t1, P.form1);
       }
-      if (P.has_phase) apply_phase<PL, NR - 1, CP>(v, P.ph, tlo, thi, P.cost, P.cost_kind, g, base);
+      if (P.has_phase) apply_phase<PL, NR - 1, CP>(v, P.ph, tab, P.cost, P.cost_kind, g, base);
       if (has2) {
         rot_regs<EB>(v, P.s2.m[NR - 1], P.t2, P.form2);
         if constexpr (NR == 3) {
@@ -421,7 +457,7 @@ __global__ void __launch_bounds__(PL::NT, 2) k_fwd(const __grid_constant__ FwdPa
         final0 = false;
       }
     } else {
-      if (P.has_phase) apply_phase<PL, 0, CP>(v, P.ph, tlo, thi, P.cost, P.cost_kind, g, base);
+      if (P.has_phase) apply_phase<PL, 0, CP>(v, P.ph, tab, P.cost, P.cost_kind, g, base);
       rot_regs<EB>(v, P.s2.m[0], P.t2, P.form2);
       xpose<PL, 0, 1>(v, tile);
       rot_regs<EB>(v, P.s2.m[1], P.t2, P.form2);
@@ -472,18 +508,12 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C2 *tv = reinterpret_cast<C2 *>(smem_raw);
   C2 *tw = tv + (1 << PL::TB);
-  C2 *tlo = tw + (1 << PL::TB);
-  C2 *thi = tlo + 256;
-  double *red = reinterpret_cast<double *>(thi + 256);
+  C2 *tab = tw + (1 << PL::TB);
+  double *red = reinterpret_cast<double *>(tab + kTileTable);
 
-  if (P.has_phase && P.ph.mode == 0) {
-    for (int i = threadIdx.x; i < 256; i += PL::NT) {
-      tlo[i] = P.ph.tab_lo[i];
-      thi[i] = P.ph.tab_hi[i];
-    }
-  }
+  if (P.has_phase && P.ph.mode == 0) fill_phase<PL::NT>(tab, P.ph);
   const Geom g = P.g;
-  const double fc = cost_shift(P.energy);
+  const Real fc = (Real)cost_shift(P.energy);
   const bool has1 = (P.s1.m[0] | P.s1.m[1] | P.s1.m[2]) != 0;
   const bool has2 = (P.s2.m[0] | P.s2.m[1] | P.s2.m[2]) != 0;
 
@@ -497,7 +527,9 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
       const AmpIndex<PL, 0, CP> ix(g, base);
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
-        const Real f = (Real)(cost_d(P.cost, P.cost_kind, ix.at(r)) - fc);
+        Real f;
+        cost_r(P.cost, P.cost_kind, ix.at(r), f);
+        f -= fc;
         w[r] = mk<C2>(f * v[r].x, f * v[r].y);
       }
     } else {
@@ -519,9 +551,11 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
         const uint64_t x = ix.at(r);
-        const Real f = (Real)(cost_d(P.cost, P.cost_kind, x) - fc);
+        Real f;
+        cost_r(P.cost, P.cost_kind, x, f);
+        f -= fc;
         raw += f * (w[r].x * v[r].y - w[r].y * v[r].x);
-        const C2 ph = phase_factor(P.ph, tlo, thi, P.cost, P.cost_kind, x);
+        const C2 ph = phase_factor(P.ph, tab, P.cost, P.cost_kind, x);
         v[r] = cmul(v[r], ph);
         w[r] = cmul(w[r], ph);
       }
@@ -582,7 +616,7 @@ static int blocks_per_sm(K kernel, int nt, size_t smem) {
 template <class PL, typename Real, bool CP = false>
 static cudaError_t launch_fwd_t(const FwdParams<Real> &P, cudaStream_t s, int nsm) {
   using C2 = typename C2T<Real>::type;
-  const size_t smem = ((size_t)(1 << PL::TB) + 512) * sizeof(C2) + (PL::NT / 32) * 3 * sizeof(double);
+  const size_t smem = ((size_t)(1 << PL::TB) + kTileTable) * sizeof(C2) + (PL::NT / 32) * 3 * sizeof(double);
   auto kern = k_fwd<PL, Real, CP>;
   static int nb = -1;  // per instantiation; the device is fixed per process
   if (nb < 0) {
@@ -599,7 +633,7 @@ static cudaError_t launch_fwd_t(const FwdParams<Real> &P, cudaStream_t s, int ns
 template <class PL, typename Real, bool CP = false>
 static cudaError_t launch_bwd_t(const BwdParams<Real> &P, cudaStream_t s, int nsm) {
   using C2 = typename C2T<Real>::type;
-  const size_t smem = ((size_t)(2 << PL::TB) + 512) * sizeof(C2) + (PL::NT / 32) * 3 * sizeof(double);
+  const size_t smem = ((size_t)(2 << PL::TB) + kTileTable) * sizeof(C2) + (PL::NT / 32) * 3 * sizeof(double);
   auto kern = k_bwd<PL, Real, CP>;
   static int nb = -1;
   if (nb < 0) {
@@ -630,24 +664,16 @@ cudaError_t launch_fwd(const FwdParams<float> &P, bool high, int tb, cudaStream_
   return dispatch_fwd<PlanF13Low, PlanF13High>(P, high, s, nsm);
 }
 cudaError_t launch_fwd(const FwdParams<double> &P, bool high, int tb, cudaStream_t s, int nsm) {
-  switch (tb) {
-    case 9: return dispatch_fwd<PlanT9Low, PlanT9High>(P, high, s, nsm);
-    case 10: return dispatch_fwd<PlanT10Low, PlanT10High>(P, high, s, nsm);
-    case 12: return dispatch_fwd<PlanT12Low, PlanT12High>(P, high, s, nsm);
-    default: return cudaErrorInvalidValue;
-  }
+  if (tb != PlanT12Low::TB) return cudaErrorInvalidValue;
+  return dispatch_fwd<PlanT12Low, PlanT12High>(P, high, s, nsm);
 }
 cudaError_t launch_bwd(const BwdParams<float> &P, bool high, int tb, cudaStream_t s, int nsm) {
   if (tb != PlanT12Low::TB) return cudaErrorInvalidValue;
   return dispatch_bwd<PlanT12Low, PlanT12High>(P, high, s, nsm);
 }
 cudaError_t launch_bwd(const BwdParams<double> &P, bool high, int tb, cudaStream_t s, int nsm) {
-  switch (tb) {
-    case 9: return dispatch_bwd<PlanT9Low, PlanT9High>(P, high, s, nsm);
-    case 10: return dispatch_bwd<PlanT10Low, PlanT10High>(P, high, s, nsm);
-    case 11: return dispatch_bwd<PlanT11Low, PlanT11High>(P, high, s, nsm);
-    default: return cudaErrorInvalidValue;
-  }
+  if (tb != PlanT11Low::TB) return cudaErrorInvalidValue;
+  return dispatch_bwd<PlanT11Low, PlanT11High>(P, high, s, nsm);
 }
 
 }  // namespace qaoa

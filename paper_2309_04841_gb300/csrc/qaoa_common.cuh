@@ -86,27 +86,14 @@ using PlanT11Low = Plan<11, 4, 128, 4, 3, 0x0780, 0x001F, 0x0060,
 using PlanT11High = Plan<11, 4, 128, 4, 2, 0x0780, 0x001F, 0x0060,
                          0x00F0, 0x010F, 0x0600>;
 
-// 1024- and 512-amplitude tiles for complex128 at n <= 16 / n <= 14: the
-// same number of groups as the 4096-amplitude tiles there, but 4-8 times as
-// many CTAs for the FP64-bound rotations.
-using PlanT10Low = Plan<10, 4, 64, 4, 3, 0x03C0, 0x001F, 0x0020,
-                        0x000F, 0x01F0, 0x0200, 0x00F0, 0x010F, 0x0200>;
-using PlanT10High = Plan<10, 4, 64, 4, 2, 0x03C0, 0x001F, 0x0020,
-                         0x00F0, 0x010F, 0x0200>;
-using PlanT9Low = Plan<9, 4, 32, 4, 3, 0x01E0, 0x001F, 0x0000,
-                       0x000F, 0x01F0, 0x0000, 0x00F0, 0x010F, 0x0000>;
-using PlanT9High = Plan<9, 4, 32, 4, 2, 0x01E0, 0x001F, 0x0000,
-                        0x00F0, 0x010F, 0x0000>;
-
 static_assert(PlanF13Low::valid() && PlanF13High::valid(), "bad F13 plan");
-static_assert(PlanT10Low::valid() && PlanT10High::valid(), "bad T10 plan");
-static_assert(PlanT9Low::valid() && PlanT9High::valid(), "bad T9 plan");
 static_assert(PlanT12Low::valid() && PlanT12High::valid(), "bad T12 plan");
 static_assert(PlanT11Low::valid() && PlanT11High::valid(), "bad T11 plan");
 
 // Passenger (low-segment) bits of a HIGH pass: 2^4 contiguous amplitudes
 // (128 B for complex64, 256 B for complex128) per global segment.
 constexpr int kHighC = 4;
+constexpr int kMidC = 2;  // of the small tiles (mid_kernels.cu)
 
 // The gradient is the same for f and f - c, any c: d/d beta and d/d gamma are
 // commutators' expectations.  With c = E the vector lambda = (f - c) psi is as
@@ -152,20 +139,21 @@ struct Sweep {
 };
 
 // ------------------------------------------------------------ parameters
-// Per-layer phase data.  Integer costs use a two-level table
-// exp(-i g (fmin + 256 hi + lo)) = T_hi[hi] * T_lo[lo] built on the host in
-// float64; other costs use a float-float reduction of g f / (2 pi).
+// Per-layer phase data.  Mode 0, integer costs of a small range, with
+// d = (f - fmin) >> shift: exp(-i g f) = T0[d & 63] T1[d >> 6] (nd 2), or three
+// digits, T0[d & 63] T1[(d >> 6) & 63] T2[d >> 12]; each CTA builds the `entries`
+// of its tables (fill_phase).  Mode 1: computed per amplitude.  Both reduce
+// g f / 2 pi, in complex64 as a float-float.
+constexpr int kTileTable = 192;  // most entries
 template <typename Real>
 struct PhaseData {
   using C2 = typename C2T<Real>::type;
-  int mode;     // 0: table (integer costs), 1: computed
-  int fmin;     // table origin
-  int nhi;      // entries of T_hi in use
-  float g_hi, g_lo;  // complex64 computed mode: g / 2pi = g_hi + g_lo
-  double g2pi;       // complex128 computed mode: g / 2pi
-  Real scl;          // computed mode: factor applied with the phase (tables carry it in T_hi)
-  C2 tab_lo[256];
-  C2 tab_hi[256];
+  int mode;
+  int fmin, shift;
+  int nd, last, entries;  // digits; entries of the last table - 1; of all
+  float g_hi, g_lo;  // complex64: g / 2pi = g_hi + g_lo
+  double g2pi;       // complex128: g / 2pi
+  Real scl;          // factor applied with the phase (the last table carries it)
 };
 
 template <typename Real>
@@ -219,6 +207,54 @@ struct BwdParams {
   double out_scale;       // inner products times this before they are added
   uint64_t mirror;        // nonzero (2^n - 1): psi[x] is also stored at its complement
   PhaseData<Real> ph;     // un-phase data (exp(+i g f))
+};
+
+// ---- small-tile passes, n <= 20 (mid_kernels.cu)
+constexpr int kMidMaxN = 20, kMidMaxRounds = 6;
+
+// Partial sums [ntiles][3] of an adjoint pass and the slots that scale times
+// their sums are added to; ntiles 0: none.
+struct MidSums {
+  const double *partials;
+  uint64_t ntiles;
+  double *out_b1, *out_g, *out_b2;
+  double scale;
+};
+
+// The register bits that round k of a tile of TB bits rotates: round k holds bits
+// 2k, 2k+1 (the last one TB-2, TB-1) and leaves what an earlier round has rotated.
+__host__ __device__ constexpr int mid_rounds(int TB) { return (TB + 1) / 2; }
+__host__ __device__ constexpr int mid_shift(int TB, int k) { return 2 * k < TB - 2 ? 2 * k : TB - 2; }
+__host__ __device__ constexpr uint32_t mid_mask(int TB, uint32_t rot, int k) {
+  const uint32_t fresh = mid_shift(TB, k) < 2 * k ? 2u : 3u;
+  return (rot >> mid_shift(TB, k)) & fresh;
+}
+
+template <typename Real>
+struct MidParams {
+  using C2 = typename C2T<Real>::type;
+  C2 *psi, *lam;
+  const void *cost;
+  int cost_kind;
+  Geom g;
+  int kind;             // as the TMA passes': kernels.h
+  uint32_t rot;         // tile bits rotated by each sweep
+  Real t1, t2;          // sweeps before and after the phase, reduced (FwdParams, BwdParams)
+  int form1, form2;
+  Real w1[kMidMaxRounds], w2[kMidMaxRounds], wg;
+  Real post_scale;
+  int init_plus;
+  int overlap;          // launched to overlap the pass before it, whose own costs were complete
+  Real amp;
+  double fmin_d;
+  const double *energy;
+  double *partials;
+  unsigned *counter;
+  double *out;
+  double out_scale;
+  uint64_t mirror;
+  MidSums prev;         // summed by an extra CTA
+  PhaseData<Real> ph;
 };
 
 // ---- single-CTA kernels (small_kernels.cu)

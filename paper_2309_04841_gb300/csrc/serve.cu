@@ -14,6 +14,8 @@
 // rejected at once.  Every request's arithmetic depends only on its own
 // inputs (fixed launch shapes, deterministic reductions), so its result is
 // the same alone and in any mix.
+#include <sys/prctl.h>
+
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -27,6 +29,7 @@
 #include <vector>
 
 #include "../../include/qaoa.h"
+#include "calls.h"
 #include "kernels.h"
 #include "qaoa_common.cuh"
 
@@ -287,11 +290,11 @@ bool start_large(qaoa_server *S, Job *j, int u) {
   double *d_out = reinterpret_cast<double *>(S->d_arena + o_out);
   qaoa_status r;
   if (j->want_grad)
-    r = qaoa_grad(j->n, S->d_arena + ce->off, ce->ct, &ce->stats, j->g.data(), j->b.data(), j->p,
-                  S->d_arena + o_state, S->d_arena + o_lam, QAOA_C64, S->d_arena + o_work, wsb, d_out, st);
+    r = grad_call(j->n, S->d_arena + ce->off, ce->ct, &ce->stats, j->g.data(), j->b.data(), j->p,
+                  S->d_arena + o_state, S->d_arena + o_lam, QAOA_C64, S->d_arena + o_work, wsb, d_out, false, st);
   else
-    r = qaoa_simulate(j->n, S->d_arena + ce->off, ce->ct, &ce->stats, j->g.data(), j->b.data(), j->p,
-                      S->d_arena + o_state, QAOA_C64, 1, S->d_arena + o_work, wsb, d_out, st);
+    r = simulate_call(j->n, S->d_arena + ce->off, ce->ct, &ce->stats, j->g.data(), j->b.data(), j->p,
+                      S->d_arena + o_state, QAOA_C64, 1, S->d_arena + o_work, wsb, d_out, false, st);
   const size_t nd = j->want_grad ? 2 + 2 * (size_t)j->p : 2;
   if (r == QAOA_OK && nd <= U.h_out_cap)
     r = cudaMemcpyAsync(U.h_out, d_out, nd * sizeof(double), cudaMemcpyDeviceToHost, U.stream) == cudaSuccess
@@ -457,8 +460,15 @@ void reap(qaoa_server *S) {
 
 constexpr int kMaxBypass = 8;
 
+bool any_busy(const qaoa_server *S) {
+  for (const Unit &U : S->units)
+    if (U.busy) return true;
+  return false;
+}
+
 void worker_main(qaoa_server *S) {
   cudaSetDevice(S->device);
+  prctl(PR_SET_TIMERSLACK, 1000ul, 0ul, 0ul, 0ul);  // ns, this thread only
   std::unique_lock<std::mutex> lk(S->mu);
   while (!S->stop) {
     reap(S);
@@ -498,7 +508,9 @@ void worker_main(qaoa_server *S) {
       }
     }
     S->cv_done.notify_all();
-    if (!progressed) S->cv_work.wait_for(lk, std::chrono::microseconds(50));
+    // Running units are polled; the thread's timer slack (50 us by default) is
+    // cut so that a short request is not reported a poll and a slack late.
+    if (!progressed) S->cv_work.wait_for(lk, std::chrono::microseconds(any_busy(S) ? 20 : 1000));
   }
 }
 

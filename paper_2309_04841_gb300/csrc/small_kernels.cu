@@ -17,122 +17,14 @@
 // a call, n = 12 586 -> 66 us; complex128 877 -> 254 and 3577 -> 953 us.
 #include <cstring>
 
-#include "qaoa_common.cuh"
 #include "kernels.h"
+#include "tile_ops.cuh"
 
 namespace qaoa {
 
 namespace {
 
-__device__ __forceinline__ double ld_cost(const void *cost, int kind, uint32_t x) {
-  if (kind == kCostI32) return (double)reinterpret_cast<const int *>(cost)[x];
-  if (kind == kCostU16) return (double)reinterpret_cast<const unsigned short *>(cost)[x];
-  if (kind == kCostF32) return (double)reinterpret_cast<const float *>(cost)[x];
-  return reinterpret_cast<const double *>(cost)[x];
-}
-
-// ---- per precision: vector arithmetic, costs, phases, sums
-template <typename Real> struct Ops;
-
-template <> struct Ops<float> {
-  using C2 = float2;
-  using F = float2;  // a cost value as float pair hi + lo
-  __device__ static __forceinline__ F integer(int f) {
-    const float h = (float)f;
-    return make_float2(h, (float)((long long)f - (long long)h));
-  }
-  __device__ static __forceinline__ C2 mk(float x, float y) { return make_float2(x, y); }
-  __device__ static __forceinline__ C2 axpy(float t, C2 a, C2 b) { return __ffma2_rn(make_float2(t, t), a, b); }
-  // exact for int32 and float32 costs, about 2^-48 relative for float64 ones
-  __device__ static __forceinline__ F cost(const void *c, int kind, uint32_t x) {
-    if (kind == kCostI32) return integer(reinterpret_cast<const int *>(c)[x]);
-    if (kind == kCostU16) return make_float2((float)reinterpret_cast<const unsigned short *>(c)[x], 0.f);
-    if (kind == kCostF32) return make_float2(reinterpret_cast<const float *>(c)[x], 0.f);
-    const double f = reinterpret_cast<const double *>(c)[x];
-    const float h = (float)f;
-    return make_float2(h, (float)(f - (double)h));
-  }
-  __device__ static __forceinline__ float value(F f) { return f.x; }
-  // scl exp(-i g f) with g / 2pi = g_hi + g_lo: Dekker's two-product by fma,
-  // only the fraction reaches sincospi
-  __device__ static __forceinline__ C2 phase(const SmallLayer<float> &L, F f, float scl) {
-    const float p = L.g_hi * f.x;
-    const float e = fmaf(L.g_hi, f.x, -p);
-    const float r = (p - rintf(p)) + (e + fmaf(L.g_hi, f.y, L.g_lo * f.x));
-    float sn, cs;
-    sincospif(2.0f * r, &sn, &cs);
-    return make_float2(cs * scl, -sn * scl);
-  }
-  // slot of index i: 16 lanes of a half-warp hit 16 bank pairs in every layout
-  __device__ static __forceinline__ uint32_t slot(uint32_t i) { return i ^ ((i >> 4) & 7u) ^ ((i >> 3) & 8u); }
-  // running sum as a float pair (Knuth's TwoSum)
-  struct Sum {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x) {
-      const float s = hi + x, bb = s - hi;
-      lo += (hi - (s - bb)) + (x - bb);
-      hi = s;
-    }
-    __device__ __forceinline__ float get() const { return hi + lo; }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-  };
-};
-
-template <> struct Ops<double> {
-  using C2 = double2;
-  using F = double;
-  __device__ static __forceinline__ F integer(int f) { return (double)f; }
-  __device__ static __forceinline__ C2 mk(double x, double y) { return make_double2(x, y); }
-  __device__ static __forceinline__ C2 axpy(double t, C2 a, C2 b) {
-    return make_double2(fma(t, a.x, b.x), fma(t, a.y, b.y));
-  }
-  __device__ static __forceinline__ F cost(const void *c, int kind, uint32_t x) { return ld_cost(c, kind, x); }
-  __device__ static __forceinline__ double value(F f) { return f; }
-  __device__ static __forceinline__ C2 phase(const SmallLayer<double> &L, F f, double scl) {
-    const double t = L.g2pi * f;
-    double sn, cs;
-    sincospi(2.0 * (t - rint(t)), &sn, &cs);
-    return make_double2(cs * scl, -sn * scl);
-  }
-  // 8 lanes of a quarter-warp hit 8 slots of 16 bytes
-  __device__ static __forceinline__ uint32_t slot(uint32_t i) { return i ^ ((i >> 3) & 7u); }
-  struct Sum {
-    double s = 0.0;
-    __device__ __forceinline__ void add(double x) { s += x; }
-    __device__ __forceinline__ double get() const { return s; }
-    __device__ __forceinline__ double value() const { return s; }
-  };
-};
-
-template <typename C2>
-__device__ __forceinline__ C2 cm(C2 a, C2 b) {
-  C2 r;
-  r.x = a.x * b.x - a.y * b.y;
-  r.y = a.x * b.y + a.y * b.x;
-  return r;
-}
-
-// z * i^k
-template <typename C2>
-__device__ __forceinline__ C2 ipow(C2 z, int k) {
-  C2 r = z;
-  if (k & 1) {
-    r.x = -z.y;
-    r.y = z.x;
-  }
-  if (k & 2) {
-    r.x = -r.x;
-    r.y = -r.y;
-  }
-  return r;
-}
-
-template <typename C2>
-__device__ __forceinline__ C2 neg(C2 a) {
-  a.x = -a.x;
-  a.y = -a.y;
-  return a;
-}
+using namespace tile;
 
 // Deterministic block sum (fixed tree); thread 0 gets the result.
 template <int K>
@@ -209,17 +101,6 @@ __device__ __forceinline__ Real inner(const typename Ops<Real>::C2 (&v)[1 << EB]
   return ((p[0].x + p[1].x) + (p[0].y + p[1].y)) - ((q[0].x + q[1].x) + (q[0].y + q[1].y));
 }
 
-template <int I> struct Int { static constexpr int value = I; };
-
-// f(Int<0>()), ..., f(Int<N - 1>())
-template <int N, int I = 0, class F>
-__device__ __forceinline__ void unroll(F f) {
-  if constexpr (I < N) {
-    f(Int<I>());
-    unroll<N, I + 1>(f);
-  }
-}
-
 }  // namespace
 
 // mode 0: forward layers [0, nl) (+ optional E/O reduction)
@@ -268,10 +149,10 @@ __device__ __forceinline__ void small_run(const SmallJob<Real> &P) {
   };
   auto index = [&](auto K, int r) { return base_of(K) | ((uint32_t)r << T::shift(D, K.value)); };
   uint32_t sb[R];
-  unroll<R>([&](auto K) { sb[K.value] = O::slot(base_of(K)); });
-  auto slot = [&](auto K, int r) { return sb[K.value] ^ O::slot((uint32_t)r << T::shift(D, K.value)); };
+  unroll<R>([&](auto K) { sb[K.value] = O::template slot<EB>(base_of(K)); });
+  auto slot = [&](auto K, int r) { return sb[K.value] ^ O::template slot<EB>((uint32_t)r << T::shift(D, K.value)); };
 
-  for (uint32_t x = tid; x < N; x += blockDim.x) fs[O::slot(x)] = O::cost(P.cost, P.cost_kind, x);
+  for (uint32_t x = tid; x < N; x += blockDim.x) fs[O::template slot<EB>(x)] = O::cost(P.cost, P.cost_kind, x);
   {  // a copy of the layers: every layer starts with them, and from shared memory they take one latency
     static_assert(sizeof(SmallLayer<Real>) % 8 == 0, "copied in 8-byte words");
     const uint64_t *src = reinterpret_cast<const uint64_t *>(P.L);
@@ -335,7 +216,7 @@ __device__ __forceinline__ void small_run(const SmallJob<Real> &P) {
       const Real eb = (((D - 1) >> 1) + __popc(base_of(K2))) & 1 ? (Real)-1 : (Real)1;
 #pragma unroll
       for (int r = 0; r < REGS; ++r) {
-        const uint32_t j = slot(K2, r) ^ O::slot(all);
+        const uint32_t j = slot(K2, r) ^ O::template slot<EB>(all);
         const Real ep = (popc_c(r) & 1) ? -eb : eb;
         const C2 b = bv[j];
         if (two.value) {
@@ -365,7 +246,7 @@ __device__ __forceinline__ void small_run(const SmallJob<Real> &P) {
       const bool low = P.ndig && e < 64;  // the low digit of two
       const Real scl = low ? (Real)1 : adj ? L.sig_adj : li == 0 ? (Real)1 : Ls[li - 1].sig;
       const int j = low ? e << P.shift : P.fmin + ((P.ndig ? (e - 64) * 64 : e) << P.shift);
-      const F f = P.by_x ? fs[O::slot((uint32_t)e)] : O::integer(j);
+      const F f = P.by_x ? fs[O::template slot<EB>((uint32_t)e)] : O::integer(j);
       C2 z = O::phase(L, f, scl);
       if (adj) z.y = -z.y;
       tab[i] = z;
@@ -511,7 +392,7 @@ __device__ __forceinline__ void small_run(const SmallJob<Real> &P) {
 #pragma unroll
     for (int r = 0; r < REGS; ++r) {
       if (P.mode == 1 || P.init_lambda) {
-        const Real f = O::value(fs[O::slot(at(r))]) - fc;
+        const Real f = O::value(fs[O::template slot<EB>(at(r))]) - fc;
         w[r] = O::mk(f * v[r].x, f * v[r].y);
       } else {
         w[r] = ipow(P.lam[at(r)], -__popc(at(r)));

@@ -1,0 +1,166 @@
+// tile_ops.cuh -- what the on-chip and the small-tile kernels share: arithmetic per
+// precision, costs and phases, and slots of tile offsets in shared memory that are
+// linear over XOR and free of bank conflicts in every round of a tile.
+#pragma once
+
+#include "qaoa_common.cuh"
+
+namespace qaoa {
+namespace tile {
+
+__device__ __forceinline__ double ld_cost(const void *cost, int kind, uint32_t x) {
+  if (kind == kCostI32) return (double)reinterpret_cast<const int *>(cost)[x];
+  if (kind == kCostU16) return (double)reinterpret_cast<const unsigned short *>(cost)[x];
+  if (kind == kCostF32) return (double)reinterpret_cast<const float *>(cost)[x];
+  return reinterpret_cast<const double *>(cost)[x];
+}
+
+// ---- per precision: vector arithmetic, costs, phases, sums
+template <typename Real> struct Ops;
+
+template <> struct Ops<float> {
+  using C2 = float2;
+  using F = float2;  // a cost value as float pair hi + lo
+  __device__ static __forceinline__ F integer(int f) {
+    const float h = (float)f;
+    return make_float2(h, (float)((long long)f - (long long)h));
+  }
+  __device__ static __forceinline__ C2 mk(float x, float y) { return make_float2(x, y); }
+  __device__ static __forceinline__ C2 axpy(float t, C2 a, C2 b) { return __ffma2_rn(make_float2(t, t), a, b); }
+  // exact for int32 and float32 costs, about 2^-48 relative for float64 ones
+  __device__ static __forceinline__ F cost(const void *c, int kind, uint32_t x) {
+    if (kind == kCostI32) return integer(reinterpret_cast<const int *>(c)[x]);
+    if (kind == kCostU16) return make_float2((float)reinterpret_cast<const unsigned short *>(c)[x], 0.f);
+    if (kind == kCostF32) return make_float2(reinterpret_cast<const float *>(c)[x], 0.f);
+    const double f = reinterpret_cast<const double *>(c)[x];
+    const float h = (float)f;
+    return make_float2(h, (float)(f - (double)h));
+  }
+  __device__ static __forceinline__ float value(F f) { return f.x; }
+  // scl exp(-i g f) with g / 2pi = g_hi + g_lo: Dekker's two-product by fma,
+  // only the fraction reaches sincospi
+  template <class L>
+  __device__ static __forceinline__ C2 phase(const L &l, F f, float scl) {
+    const float p = l.g_hi * f.x;
+    const float e = fmaf(l.g_hi, f.x, -p);
+    const float r = (p - rintf(p)) + (e + fmaf(l.g_hi, f.y, l.g_lo * f.x));
+    float sn, cs;
+    sincospif(2.0f * r, &sn, &cs);
+    return make_float2(cs * scl, -sn * scl);
+  }
+  // a float32 or float64 cost
+  __device__ static __forceinline__ F real(const void *c, int kind, uint64_t x) {
+    if (kind == kCostF32) return make_float2(__ldg(reinterpret_cast<const float *>(c) + x), 0.f);
+    const double f = __ldg(reinterpret_cast<const double *>(c) + x);
+    const float h = (float)f;
+    return make_float2(h, (float)(f - (double)h));
+  }
+  // Slot of tile offset i with EB register bits (rounds over consecutive bits):
+  // 16 lanes of a half-warp hit 16 bank pairs in the layouts of EB 2 and 3 (and
+  // all but a two-way conflict for EB 1).
+  template <int EB>
+  __host__ __device__ static constexpr uint32_t slot(uint32_t i) {
+    return EB == 3 ? i ^ ((i >> 4) & 7u) ^ ((i >> 3) & 8u) : i ^ ((i >> 4) & 3u) ^ ((i >> 2) & 12u);
+  }
+  // running sum as a float pair (Knuth's TwoSum)
+  struct Sum {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x) {
+      const float s = hi + x, bb = s - hi;
+      lo += (hi - (s - bb)) + (x - bb);
+      hi = s;
+    }
+    __device__ __forceinline__ void warp() {  // lane 0 gets the warp's sum
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float h = __shfl_down_sync(0xffffffffu, hi, o), l = __shfl_down_sync(0xffffffffu, lo, o);
+        add(h);
+        lo += l;
+      }
+    }
+    __device__ __forceinline__ float get() const { return hi + lo; }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  };
+};
+
+template <> struct Ops<double> {
+  using C2 = double2;
+  using F = double;
+  __device__ static __forceinline__ F integer(int f) { return (double)f; }
+  __device__ static __forceinline__ C2 mk(double x, double y) { return make_double2(x, y); }
+  __device__ static __forceinline__ C2 axpy(double t, C2 a, C2 b) {
+    return make_double2(fma(t, a.x, b.x), fma(t, a.y, b.y));
+  }
+  __device__ static __forceinline__ F cost(const void *c, int kind, uint32_t x) { return ld_cost(c, kind, x); }
+  __device__ static __forceinline__ double value(F f) { return f; }
+  template <class L>
+  __device__ static __forceinline__ C2 phase(const L &l, F f, double scl) {
+    const double t = l.g2pi * f;
+    double sn, cs;
+    sincospi(2.0 * (t - rint(t)), &sn, &cs);
+    return make_double2(cs * scl, -sn * scl);
+  }
+  __device__ static __forceinline__ F real(const void *c, int kind, uint64_t x) {
+    return kind == kCostF32 ? (double)__ldg(reinterpret_cast<const float *>(c) + x)
+                            : __ldg(reinterpret_cast<const double *>(c) + x);
+  }
+  // 8 lanes of a quarter-warp hit 8 slots of 16 bytes
+  template <int EB>
+  __host__ __device__ static constexpr uint32_t slot(uint32_t i) {
+    return EB == 3 ? i ^ ((i >> 3) & 7u) : i ^ ((i >> 3) & 3u) ^ ((i >> 2) & 4u);
+  }
+  struct Sum {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void warp() {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    }
+    __device__ __forceinline__ double get() const { return s; }
+    __device__ __forceinline__ double value() const { return s; }
+  };
+};
+
+template <typename C2>
+__device__ __forceinline__ C2 cm(C2 a, C2 b) {
+  C2 r;
+  r.x = a.x * b.x - a.y * b.y;
+  r.y = a.x * b.y + a.y * b.x;
+  return r;
+}
+
+// z * i^k
+template <typename C2>
+__device__ __forceinline__ C2 ipow(C2 z, int k) {
+  C2 r = z;
+  if (k & 1) {
+    r.x = -z.y;
+    r.y = z.x;
+  }
+  if (k & 2) {
+    r.x = -r.x;
+    r.y = -r.y;
+  }
+  return r;
+}
+
+template <typename C2>
+__device__ __forceinline__ C2 neg(C2 a) {
+  a.x = -a.x;
+  a.y = -a.y;
+  return a;
+}
+
+template <int I> struct Int { static constexpr int value = I; };
+
+// f(Int<0>()), ..., f(Int<N - 1>())
+template <int N, int I = 0, class F>
+__device__ __forceinline__ void unroll(F f) {
+  if constexpr (I < N) {
+    f(Int<I>());
+    unroll<N, I + 1>(f);
+  }
+}
+
+}  // namespace tile
+}  // namespace qaoa

@@ -41,7 +41,7 @@ def rel(a, b):
 # n <= 13: on chip, every number of rounds and of bits in the last one.  n: every count of groups (forward 13 + 9 rows + ..., adjoint 12 + 8 or 9), a group that takes only the complement,
 # odd and even numbers of index bits, groups of exactly full rows
 @pytest.mark.parametrize("kind", ["i32", "u16", "f32", "f64"])
-@pytest.mark.parametrize("n", [4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 19, 20, 21, 22, 23, 24])
+@pytest.mark.parametrize("n", [4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 17, 18, 19, 20, 21, 22, 23, 24])
 def test_half_vs_full(Q, n, kind):
     T = torch()
     p = 3
