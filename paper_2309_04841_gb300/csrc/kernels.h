@@ -258,15 +258,15 @@ struct alignas(64) XyTmaParams {
 cudaError_t launch_xy_tma(const XyTmaParams &P, bool low, cudaStream_t s, int nsm);
 cudaError_t launch_xy_tma_u16(const XyTmaParams &P, bool low, cudaStream_t s, int nsm);
 
-// One XY-mixer pass over tiles of 2^tb amplitudes: qubits 0..c-1 (contiguous)
-// and h..h+tb-c-1; the gates act on tile bits (ga[g], gb[g]) in order.
+// One XY-mixer pass over tiles of 2^tb amplitudes: qubits 0..c-1 (contiguous),
+// h1..h1+w1-1 and h2..h2+w2-1; the gates act on tile bits (ga[g], gb[g]) in order.
 constexpr int kXyMaxTb = 12;
 constexpr int kXyMaxGates = 64;
 struct XyPass {
   void *psi;
   const void *cost;
   uint64_t ntiles;
-  int tb, c, h;
+  int tb, c, h1, w1, h2, w2;
   int cost_kind, has_phase;  // phase exp(-i g f) applied while loading
   float g_hi, g_lo;          // complex64: g / 2pi = g_hi + g_lo
   double g2pi;               // complex128: g / 2pi
@@ -278,8 +278,6 @@ struct XyPass {
 };
 
 cudaError_t launch_xy_tile(const XyPass &P, bool c128, cudaStream_t s, int nsm);
-cudaError_t launch_xy_gate(void *psi, bool c128, int n, int i, int j, double tb2, double sb, int neg,
-                           cudaStream_t s, int nsm);
 cudaError_t launch_dicke(void *psi, bool c128, int n, int k, double amp, cudaStream_t s, int nsm);
 
 // The phase tables of a job (entries, ndig, shift, fmin) from its cost type and

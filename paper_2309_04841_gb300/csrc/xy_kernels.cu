@@ -6,10 +6,9 @@
 // [[cos b, -i sin b], [-i sin b, cos b]] (as three shears, see xy_pair).  A
 // layer's mixer is the ordered product of its edge gates, so consecutive
 // gates share qubits and must run in order.  k_xy_tile stages a tile of 2^tb amplitudes in shared memory
-// (2^c contiguous "passenger" qubits 0..c-1 times rows at qubits h..) and
-// applies a run of gates whose qubits all lie in the tile, one after the
-// other, with the layer's phase fused into the load of its first pass;
-// k_xy_gate applies one gate over the whole state for pairs no tile holds.
+// (2^c contiguous "passenger" qubits 0..c-1 times rows of two windows of qubits)
+// and applies a run of gates whose qubits all lie in the tile, one after the
+// other, with the layer's phase fused into the load of its first pass.
 #include "qaoa_common.cuh"
 #include "kernels.h"
 
@@ -79,12 +78,6 @@ __device__ __forceinline__ uint32_t insert2_32(uint32_t k, int lo, int hi) {
   return ((k >> hi) << (hi + 1)) | (k & ((1u << hi) - 1u));
 }
 
-// The same for global indices.
-__device__ __forceinline__ uint64_t insert2(uint64_t k, int lo, int hi) {
-  k = ((k >> lo) << (lo + 1)) | (k & ((1ull << lo) - 1ull));
-  return ((k >> hi) << (hi + 1)) | (k & ((1ull << hi) - 1ull));
-}
-
 __device__ __forceinline__ double xy_cost(const void *cost, int kind, uint64_t x) {
   if (kind == kCostI32) return (double)__ldg(reinterpret_cast<const int *>(cost) + x);
   if (kind == kCostU16) return (double)__ldg(reinterpret_cast<const unsigned short *>(cost) + x);
@@ -137,13 +130,14 @@ __device__ __forceinline__ double2 xy_phase_tab(const XyPass &P, const float2 *,
   return xy_phase(P, double2(), x);  // complex128 always computes
 }
 
-// Global index of tile offset t in tile T (bits of t below c are qubits
-// 0..c-1, the others qubits h..; T fills the remaining bits in order).
+// Global index of tile offset t in tile T: t's bits are qubits 0..c-1, h1.. and
+// h2.., T fills the gaps between and above them in order.
 __device__ __forceinline__ uint64_t xy_index(const XyPass &P, uint64_t T, uint32_t t) {
-  const int mid = P.h - P.c;
-  const uint64_t lo = T & ((1ull << mid) - 1ull), top = T >> mid;
-  return (uint64_t)(t & ((1u << P.c) - 1u)) | (lo << P.c) | ((uint64_t)(t >> P.c) << P.h) |
-         (top << (P.h + P.tb - P.c));
+  const int g1 = P.h1 - P.c, top1 = P.h1 + P.w1, g2 = P.h2 - top1;
+  const uint64_t lo = T & ((1ull << g1) - 1ull), mid = (T >> g1) & ((1ull << g2) - 1ull), top = T >> (g1 + g2);
+  const uint32_t r1 = (t >> P.c) & ((1u << P.w1) - 1u), r2 = t >> (P.c + P.w1);
+  return (uint64_t)(t & ((1u << P.c) - 1u)) | (lo << P.c) | ((uint64_t)r1 << P.h1) | (mid << top1) |
+         ((uint64_t)r2 << P.h2) | (top << (P.h2 + P.w2));
 }
 
 // Registers per thread for the next tile's amplitudes (complex64; tiles of
@@ -234,18 +228,6 @@ __global__ void __launch_bounds__(256, PF ? 3 : 1) k_xy_tile(const __grid_consta
   }
 }
 
-template <typename C2>
-__global__ void __launch_bounds__(256) k_xy_gate(C2 *psi, int n, int i, int j, double tb2, double sb,
-                                                int neg) {
-  using R = typename XyR<C2>::R;
-  const uint64_t K = 1ull << (n - 2);
-  const int lo = i < j ? i : j, hi = i < j ? j : i;
-  for (uint64_t k = blockIdx.x * 256ull + threadIdx.x; k < K; k += (uint64_t)gridDim.x * 256ull) {
-    const uint64_t x0 = insert2(k, lo, hi);
-    xy_pair<C2, R>(psi[x0 | (1ull << i)], psi[x0 | (1ull << j)], (R)tb2, (R)sb, neg != 0);
-  }
-}
-
 // |D^n_k>: amplitude C(n, k)^{-1/2} on every x of Hamming weight k, else 0.
 template <typename C2>
 __global__ void __launch_bounds__(256) k_dicke(C2 *psi, int n, int k, double amp) {
@@ -289,16 +271,6 @@ cudaError_t launch_xy_tile(const XyPass &P, bool c128, cudaStream_t s, int nsm) 
     k_xy_tile<double2, false><<<grid, 256, smem, s>>>(P);
   else
     k_xy_tile<float2, true><<<grid, 256, smem, s>>>(P);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_xy_gate(void *psi, bool c128, int n, int i, int j, double tb2, double sb, int neg,
-                           cudaStream_t s, int nsm) {
-  const unsigned grid = grid_n(1ull << (n - 2), nsm);
-  if (c128)
-    k_xy_gate<double2><<<grid, 256, 0, s>>>(reinterpret_cast<double2 *>(psi), n, i, j, tb2, sb, neg);
-  else
-    k_xy_gate<float2><<<grid, 256, 0, s>>>(reinterpret_cast<float2 *>(psi), n, i, j, tb2, sb, neg);
   return cudaGetLastError();
 }
 

@@ -113,3 +113,17 @@ def test_simulate_xy_ring_deeper(Q):
     assert np.linalg.norm(got - ref) <= 2e-5 * np.linalg.norm(ref)
     E = oracle.energy(n, ref, f)
     assert abs(dev_np(out)[0] - E) <= 1e-5 * max(1.0, abs(E))
+
+
+@pytest.mark.parametrize("n,st", [(15, "c128"), (17, "c64"), (20, "c64"), (23, "c64")])
+def test_complete_graph_blocks(Q, n, st):
+    # the block schedule of the complete graph: last blocks of fewer rows, windows that touch, 4- and 16-amplitude
+    # segments, against the oracle's lexicographic order (tolerances as above: the same gates)
+    stype = Q.C64 if st == "c64" else Q.C128
+    f = oracle.labs_costs(n).astype(float)
+    fd = Q.labs_costs(n)
+    stats = Q.cost_stats_compute(fd)
+    g, b = I.angles(1, 70 + n, 0, 0.3), I.angles(1, 71 + n)
+    state, _ = Q.simulate_xy(fd, stats, g, b, Q.dicke_state(n, n // 2, stype), Q.XY_COMPLETE)
+    ref = oracle.simulate_xy(n, f, g, b, oracle.dicke(n, n // 2), Q.XY_COMPLETE)
+    assert np.linalg.norm(dev_np(state).astype(np.complex128) - ref) <= TOL[st][0] * np.linalg.norm(ref)
