@@ -218,9 +218,12 @@ void make_phase(PhaseDigits &ph, double g, qaoa_cost_type ct, const qaoa_cost_st
     }
   } else {
     ph.mode = 1;
+    ph.nd = integer_cost(ct) ? 0 : 1;
     const double g2 = g / kTwoPi;
     ph.g_hi = (float)g2;
     ph.g_lo = (float)(g2 - (double)ph.g_hi);
+    ph.nent = 64;
+    for (int j = 0; j < 64; ++j) put(j, kTwoPi / 64.0 * j, true);
   }
 }
 
@@ -1114,7 +1117,6 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
     if (P.has_phase) {
       // the pending scale rides on the phase multiply
       make_phase(P.ph, gam[op.lp], ct, stats, sig);
-      P.scl_phase = f2c(sig);
       sig = 1.0;
     }
     if (op.l2 >= 0) {
@@ -1153,8 +1155,7 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
 
 qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_cost_stats *stats,
                          const double *gam, const double *bet, int p, void *state, void *lam,
-                         const Ws &ws, const double *d_energy, double *d_grad_g, double *d_grad_b, bool half,
-                           cudaStream_t s) {
+                         const Ws &ws, const double *d_energy, double *d_grad_g, double *d_grad_b, bool half, cudaStream_t s) {
   using Low = PlanTmaB12Low;
   using High = PlanTmaB12High;
   const int TB = Low::TB;
@@ -1228,7 +1229,6 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
       P.wg = (float)std::norm(sig);
       // the un-phase multiply also pays the pending scale
       make_phase(P.ph, -gam[op.lp], ct, stats, sig);
-      P.scl_phase = f2c(sig);
       sig = 1.0;
       P.out_g = d_grad_g + op.lp;
     }

@@ -16,6 +16,7 @@
 // p = 12 LABS n = 14 391 -> 111 us, n = 18 393 -> 187 us, without symmetry n = 18
 // 394 -> 231 us; complex128 p = 2 n = 14 253 -> 77 us, p = 4 n = 18 655 -> 386 us.
 #include "kernels.h"
+#include "overlap.cuh"
 #include "tile_ops.cuh"
 
 namespace qaoa {
@@ -35,9 +36,6 @@ using F = O::F;
 
 constexpr int kH1 = 1, kPH = 2, kH2 = 4, kRED = 8, kINIT = 8;
 constexpr int EB = 2, REGS = 4;
-
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // exp(-i b X) in reduced form (pass_kernels.cu) on the register bits in mask.
 __device__ __forceinline__ void rot_std(C2 (&v)[REGS], uint32_t mask, Real t, int form) {
@@ -450,22 +448,6 @@ __global__ void __launch_bounds__(TL::NT) k_mid_bwd(const __grid_constant__ MidP
 }
 
 // ---------------------------------------------------------------- launchers
-
-template <class Kernel, class Params>
-cudaError_t launch_pdl(Kernel kern, unsigned grid, int threads, size_t smem, const Params &P, bool overlap,
-                       cudaStream_t s) {
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid, 1, 1);
-  cfg.blockDim = dim3((unsigned)threads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = at;
-  cfg.numAttrs = overlap ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, P);
-}
 
 template <class TL, int K>
 cudaError_t launch_fwd_k(const MidParams<Real> &P, cudaStream_t s) {

@@ -624,13 +624,11 @@ struct NoHook {
   __device__ __forceinline__ void operator()() const {}
 };
 
-// exp(-i g f) from the raw 32-bit cost word (int32 or float32).
-// exp(-i g f) from the raw 32-bit cost word; M = 2 / 3: digit tables with M
-// digits (integer costs), M = 1: computed (int32 or float32 costs).  Callers
+// scale * exp(-i g f) from the raw 32-bit cost word; M = 2 / 3: digit tables with M
+// digits (integer costs), M = 1 / 0: computed (float32 / integer costs).  Callers
 // branch on the mode once per round, outside their register loops.
 template <int M>
-__device__ __forceinline__ float2 phase_of(const PhaseDigits &ph, int kind, const float2 *tab,
-                                           uint32_t word) {
+__device__ __forceinline__ float2 phase_of(const PhaseDigits &ph, const float2 *tab, uint32_t word) {
   if constexpr (M == 2 || M == 3) {
     // conflict-free lookups: this lane's copy of each digit table
     const uint32_t d = (uint32_t)((int)word - ph.fmin) >> ph.shift;
@@ -646,28 +644,30 @@ __device__ __forceinline__ float2 phase_of(const PhaseDigits &ph, int kind, cons
       return cmulf(cmulf(a, b), c);
     }
   } else {
-    float fh, fl;
-    if (kind != kCostF32) {  // int32 or uint16
-      const int f = (int)word;
-      fh = (float)f;
-      fl = (float)((long long)f - (long long)fh);
-    } else {
-      fh = __uint_as_float(word);
-      fl = 0.f;
-    }
     // g f / 2pi as a float-float: Dekker's two-product p + e = g_hi * fh via fma
-    const float p = ph.g_hi * fh;
-    const float e = fmaf(ph.g_hi, fh, -p);
-    const float r = (p - rintf(p)) + (e + fmaf(ph.g_hi, fl, ph.g_lo * fh));
-    float sn, cs;
-    sincospif(2.0f * r, &sn, &cs);
-    return f2(cs, -sn);
+    float r;
+    if constexpr (M == 1) {  // float32
+      const float f = __uint_as_float(word);
+      const float p = ph.g_hi * f;
+      r = (p - rintf(p)) + fmaf(ph.g_lo, f, fmaf(ph.g_hi, f, -p));
+    } else {  // int32 or uint16 of a range beyond the tables
+      const int f = (int)word;
+      const float fh = (float)f, fl = (float)((long long)f - (long long)fh);
+      const float p = ph.g_hi * fh;
+      const float e = fmaf(ph.g_hi, fh, -p);
+      r = (p - rintf(p)) + (e + fmaf(ph.g_hi, fl, ph.g_lo * fh));
+    }
+    const float m = fmaf(r, 64.f, 12582912.f);  // 1.5 2^23: the low bits are k = rint(64 r)
+    const float2 t = tab[((__float_as_uint(m) & 63u) << 4) | (threadIdx.x & (kPhaseCopies - 1))];
+    const float th = 6.28318531f * fmaf(m - 12582912.f, -0.015625f, r), q = th * th;
+    const float c = fmaf(q, fmaf(q, 1.f / 24.f, -0.5f), 1.f), sn = fmaf(th * q, -1.f / 6.f, th);
+    return f2(fmaf(t.x, c, t.y * sn), fmaf(t.y, c, -t.x * sn));  // t exp(-i th)
   }
 }
 
 // Phase mode of a pass as the template argument of phase_of.
 __device__ __forceinline__ int phase_m(const PhaseDigits &ph) {
-  return ph.mode != 0 ? 1 : ph.nd == 2 ? 2 : 3;
+  return ph.mode != 0 ? (ph.nd == 1 ? 1 : 0) : ph.nd == 2 ? 2 : 3;
 }
 
 // Shared-memory copy of the digit tables: entry e (of the concatenated
@@ -682,7 +682,7 @@ __device__ __forceinline__ float cost_val(int kind, uint32_t word) {
   return kind == kCostF32 ? __uint_as_float(word) : (float)(int)word;
 }
 
-// v <- v * exp(-i g f) (* scl in computed mode; table mode has it folded in).
+// v <- v * exp(-i g f) (* the scale that the tables carry).
 // Cost-tile slot of register r's amplitude in round R (tt = thr_tile).
 template <class PL, int R, bool CP>
 __device__ __forceinline__ uint32_t cost_slot(uint32_t tt, int r) {
@@ -694,27 +694,24 @@ __device__ __forceinline__ uint32_t cost_slot(uint32_t tt, int r) {
 
 template <class PL, int R, bool CP, int M>
 __device__ __forceinline__ void phase_round_m(float2 (&v)[PL::NREG], const CostWord *cb,
-                                              const PhaseDigits &ph, int kind, const float2 *tab,
-                                              float2 scl) {
+                                              const PhaseDigits &ph, const float2 *tab) {
   const uint32_t tt = thr_tile<PL, R>();
 #pragma unroll
-  for (int r = 0; r < PL::NREG; ++r) {
-    const float2 z = phase_of<M>(ph, kind, tab, cb[cost_slot<PL, R, CP>(tt, r)]);
-    v[r] = cmulf(v[r], M == 1 ? cmulf(scl, z) : z);
-  }
+  for (int r = 0; r < PL::NREG; ++r)
+    v[r] = cmulf(v[r], phase_of<M>(ph, tab, cb[cost_slot<PL, R, CP>(tt, r)]));
 }
 
 template <class PL, int R, bool CP = false>
-__device__ __forceinline__ void phase_round(float2 (&v)[PL::NREG], const CostWord *cb,
-                                            const PhaseDigits &ph, int kind, const float2 *tab,
-                                            float2 scl) {
-  const int m = phase_m(ph);
-  if (m == 2)
-    phase_round_m<PL, R, CP, 2>(v, cb, ph, kind, tab, scl);
-  else if (m == 3)
-    phase_round_m<PL, R, CP, 3>(v, cb, ph, kind, tab, scl);
-  else
-    phase_round_m<PL, R, CP, 1>(v, cb, ph, kind, tab, scl);
+__device__ __forceinline__ void phase_round(float2 (&v)[PL::NREG], const CostWord *cb, const PhaseDigits &ph,
+                                            const float2 *tab) {
+  switch (phase_m(ph)) {
+    case 2: phase_round_m<PL, R, CP, 2>(v, cb, ph, tab); break;
+    case 3: phase_round_m<PL, R, CP, 3>(v, cb, ph, tab); break;
+    case 1:
+      if constexpr (kCW == 4) phase_round_m<PL, R, CP, 1>(v, cb, ph, tab);
+      break;
+    default: phase_round_m<PL, R, CP, 0>(v, cb, ph, tab);
+  }
 }
 
 // Float-float running sum (Knuth's TwoSum adds each term exactly into hi + lo):
@@ -942,7 +939,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
   const int midbits = P.h - P.c;
   __shared__ int s_abort;
 
-  if (PH && P.ph.mode == 0) fill_phase_tab<kThreads>(tab, P.ph);
+  if (PH) fill_phase_tab<kThreads>(tab, P.ph);
   if (tid == 0) {
     s_abort = 0;
     mbar_init(full, 1);
@@ -1037,7 +1034,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
         if constexpr (!H2 && !RED) release(T);
         rot_round<PL, 2, CP>(v, P.s1.m[2], P.tau1, P.form1, cx);
       }
-      if constexpr (PH) phase_round<PL, NR - 1, CP>(v, cb, P.ph, P.cost_kind, tab, P.scl_phase);
+      if constexpr (PH) phase_round<PL, NR - 1, CP>(v, cb, P.ph, tab);
       if constexpr (H2) {
         rot_round<PL, NR - 1, CP>(v, P.s2.m[NR - 1], P.tau2, P.form2, cx);
         if constexpr (NR == 3) {
@@ -1058,7 +1055,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
         rot_round<PL, 0, CP>(v, P.s2.m[0], P.tau2, P.form2, cx);
       }
     } else {
-      if constexpr (PH) phase_round<PL, 0, CP>(v, cb, P.ph, P.cost_kind, tab, P.scl_phase);
+      if constexpr (PH) phase_round<PL, 0, CP>(v, cb, P.ph, tab);
       rot_round<PL, 0, CP>(v, P.s2.m[0], P.tau2, P.form2, cx);
       if constexpr (early_cost)
         xp_hook<PL, 0, 1, SW, CP>(v, buf, [&] { read_abort(); cost_next(T); });
@@ -1131,8 +1128,7 @@ __device__ __forceinline__ void unphase_round(float2 (&v)[PL::NREG], float2 (&w)
     const uint32_t word = cb[ci(cost_slot<PL, R, CP>(tt, r))];
     const float f = cost_val(P.cost_kind, word) - fc;
     ag += P.wg * f * (w[r].x * v[r].y - w[r].y * v[r].x);
-    float2 ph = phase_of<M>(P.ph, P.cost_kind, tab, word);
-    if constexpr (M == 1) ph = cmulf(ph, P.scl_phase);
+    const float2 ph = phase_of<M>(P.ph, tab, word);
     v[r] = cmulf(v[r], ph);
     w[r] = cmulf(w[r], ph);
   }
@@ -1142,13 +1138,14 @@ template <class PL, int R, bool CP = false, class CI = CostIdx>
 __device__ __forceinline__ void unphase_any(float2 (&v)[PL::NREG], float2 (&w)[PL::NREG],
                                             const CostWord *cb, const TmaBwdParams &P,
                                             const float2 *tab, float fc, float &ag, CI ci = CI()) {
-  const int m = phase_m(P.ph);
-  if (m == 2)
-    unphase_round<PL, R, CP, 2>(v, w, cb, P, tab, fc, ag, ci);
-  else if (m == 3)
-    unphase_round<PL, R, CP, 3>(v, w, cb, P, tab, fc, ag, ci);
-  else
-    unphase_round<PL, R, CP, 1>(v, w, cb, P, tab, fc, ag, ci);
+  switch (phase_m(P.ph)) {
+    case 2: unphase_round<PL, R, CP, 2>(v, w, cb, P, tab, fc, ag, ci); break;
+    case 3: unphase_round<PL, R, CP, 3>(v, w, cb, P, tab, fc, ag, ci); break;
+    case 1:
+      if constexpr (kCW == 4) unphase_round<PL, R, CP, 1>(v, w, cb, P, tab, fc, ag, ci);
+      break;
+    default: unphase_round<PL, R, CP, 0>(v, w, cb, P, tab, fc, ag, ci);
+  }
 }
 
 // The state tiles use the TMA 128-byte swizzle (16- to 64-amplitude segments).
@@ -1174,7 +1171,7 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
   const int midbits = P.h - P.c;
   __shared__ int s_abort;
 
-  if (PH && P.ph.mode == 0) fill_phase_tab<PL::NT>(tab, P.ph);
+  if (PH) fill_phase_tab<PL::NT>(tab, P.ph);
   if (tid == 0) {
     s_abort = 0;
     mbar_init(full, 1);
@@ -1477,7 +1474,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_pair(const __grid_constant_
     return lo | ((uint64_t)rank << midbits) | ((U >> midbits) << (midbits + 1));
   };
 
-  if (PH && P.ph.mode == 0) fill_phase_tab<kThreads>(tab, P.ph);
+  if (PH) fill_phase_tab<kThreads>(tab, P.ph);
   if (tid == 0) {
     s_abort = 0;
     mbar_init(full, 1);
@@ -1738,7 +1735,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_xy_tma(const __grid_constant__ 
   const bool neg = P.neg != 0;
   __shared__ int s_abort;
 
-  if (PH && P.ph.mode == 0) fill_phase_tab<kThreads>(tab, P.ph);
+  if (PH) fill_phase_tab<kThreads>(tab, P.ph);
   if (tid == 0) {
     s_abort = 0;
     mbar_init(full, 1);
@@ -1788,7 +1785,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_xy_tma(const __grid_constant__ 
     }
     float2 v[NREG];
     lds_round<PL, 0, SW>(v, buf);
-    if constexpr (PH) phase_round<PL, 0>(v, cb, P.ph, P.cost_kind, tab, f2(1.f, 0.f));
+    if constexpr (PH) phase_round<PL, 0>(v, cb, P.ph, tab);
     xy_round<EB>(v, P.em[0], t, s, neg);
     if constexpr (PH)
       xp_hook<PL, 0, 1, SW>(v, buf, [&] { read_abort(); cost_next(T); });
