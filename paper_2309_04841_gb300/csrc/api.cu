@@ -1713,8 +1713,7 @@ std::vector<XyOp> xy_ring_schedule(int n) {
   std::vector<XyOp> ops;
   auto fits = [](const XyOp &o, int q) { return q < o.c || (q >= o.h1 && q < o.h1 + o.w1); };
   for (const auto &e : xy_edges(n, QAOA_XY_RING)) {
-    if (!ops.empty() && (int)ops.back().gates.size() < kXyMaxGates && fits(ops.back(), e.first) &&
-        fits(ops.back(), e.second)) {
+    if (!ops.empty() && fits(ops.back(), e.first) && fits(ops.back(), e.second)) {
       ops.back().gates.push_back(e);
       continue;
     }
@@ -1738,17 +1737,28 @@ std::vector<XyOp> xy_ring_schedule(int n) {
 // layer takes K (K - 1) / 2 passes of up to 60 gates instead of one pass per few
 // gates (n = 19: 6 instead of 51; p = 2 from a Dicke state 610 -> 248 us).  Segments of 2^c amplitudes: 32 bytes while the
 // state stays in L2, 128 beyond.
+//
+// The same split again, into blocks of two qubits, orders the gates inside a tile
+// so that xy_rounds finds rounds of up to six of them on four qubits.
+void xy_cross(std::vector<std::pair<int, int>> &g, int i0, int i1, int j0, int j1) {
+  for (int i = i0; i < i1; i += 2)
+    for (int j = j0; j < j1; j += 2)
+      for (int a = i; a < std::min(i + 2, i1); ++a)
+        for (int b = j; b < std::min(j + 2, j1); ++b) g.push_back({a, b});
+}
+
+void xy_inside(std::vector<std::pair<int, int>> &g, int q0, int q1) {
+  for (int i = q0; i < q1; i += 2) {
+    if (i + 1 < q1) g.push_back({i, i + 1});
+    xy_cross(g, i, std::min(i + 2, q1), i + 2, q1);
+  }
+}
+
 std::vector<XyOp> xy_complete_schedule(int n, bool c128) {
   std::vector<XyOp> ops;
   if (n <= kXyMaxTb) {
     XyOp o{n, n, 0, n, 0, {}};
-    for (const auto &e : xy_edges(n, QAOA_XY_COMPLETE)) {
-      if ((int)o.gates.size() == kXyMaxGates) {
-        ops.push_back(o);
-        o.gates.clear();
-      }
-      o.gates.push_back(e);
-    }
+    xy_inside(o.gates, 0, n);
     ops.push_back(o);
     return ops;
   }
@@ -1762,30 +1772,62 @@ std::vector<XyOp> xy_complete_schedule(int n, bool c128) {
       // a tile has kXyMaxTb bits: a last block of fewer rows starts lower
       const int hJ = std::min(start[J], n - rest);
       XyOp o = I == 0 ? XyOp{start[1], hJ, rest, n, 0, {}} : XyOp{c, start[I], rest, hJ, rest, {}};
-      if (I > 0 && start[I] + rest > hJ) {  // the rows of the two touch: one window
-        o.h1 = n - 2 * rest;
-        o.w1 = 2 * rest;
-        o.h2 = n;
-        o.w2 = 0;
-      }
-      auto add = [&](int i, int j) {
-        if ((int)o.gates.size() == kXyMaxGates) {
-          ops.push_back(o);
-          o.gates.clear();
-        }
-        o.gates.push_back({i, j});
-      };
-      auto inside = [&](int B) {
-        for (int i = start[B]; i < start[B + 1]; ++i)
-          for (int j = i + 1; j < start[B + 1]; ++j) add(i, j);
-      };
-      if (J == I + 1) inside(I);
-      for (int i = start[I]; i < start[I + 1]; ++i)
-        for (int j = start[J]; j < start[J + 1]; ++j) add(i, j);
-      if (I == K - 2) inside(K - 1);
+      if (I > 0 && start[I] + rest > hJ) o = XyOp{c, n - 2 * rest, 2 * rest, n, 0, {}};  // the two touch: one window
+      if (J == I + 1) xy_inside(o.gates, start[I], start[I + 1]);
+      xy_cross(o.gates, start[I], start[I + 1], start[J], start[J + 1]);
+      if (I == K - 2) xy_inside(o.gates, start[K - 1], n);
       ops.push_back(o);
     }
   return ops;
+}
+
+// A pass's gates in rounds (XyRound): a gate joins the last round while that has
+// at most four tile bits and every gate of it that shares a bit comes before this one
+// in the round's lexicographic order.
+std::vector<XyRound> xy_rounds(const XyOp &o) {
+  struct Open {
+    std::vector<int> bits;                   // ascending
+    std::vector<std::pair<int, int>> gates;  // tile bits, ascending pairs
+  };
+  std::vector<Open> rounds;
+  for (const auto &e : o.gates) {
+    std::pair<int, int> g{o.tbit(e.first), o.tbit(e.second)};
+    if (g.first > g.second) std::swap(g.first, g.second);
+    bool join = !rounds.empty();
+    std::vector<int> bits;
+    if (join) {
+      bits = rounds.back().bits;
+      for (int b : {g.first, g.second})
+        if (std::find(bits.begin(), bits.end(), b) == bits.end()) bits.push_back(b);
+      join = bits.size() <= 4;
+      for (const auto &h : rounds.back().gates)
+        if (h.first == g.first || h.first == g.second || h.second == g.first || h.second == g.second)
+          join = join && h < g;
+    }
+    if (!join) {
+      rounds.push_back(Open());
+      bits = {g.first, g.second};
+    }
+    std::sort(bits.begin(), bits.end());
+    rounds.back().bits = bits;
+    rounds.back().gates.push_back(g);
+  }
+  const int tb = o.c + o.w1 + o.w2;
+  std::vector<XyRound> out;
+  for (Open &r : rounds) {
+    for (int b = 0; (int)r.bits.size() < std::min(4, tb); ++b)  // fill up with any other bits
+      if (std::find(r.bits.begin(), r.bits.end(), b) == r.bits.end()) r.bits.push_back(b);
+    std::sort(r.bits.begin(), r.bits.end());
+    XyRound x;
+    memset(&x, 0, sizeof(x));
+    for (size_t i = 0; i < r.bits.size(); ++i) x.bit[i] = (uint8_t)r.bits[i];
+    for (int k = 0; k < 6; ++k)
+      for (const auto &g : r.gates)
+        if (xy_gate_b(k) < r.bits.size() && g.first == r.bits[xy_gate_a(k)] && g.second == r.bits[xy_gate_b(k)])
+          x.mask |= (uint8_t)(1u << k);
+    out.push_back(x);
+  }
+  return out;
 }
 
 // The pair rotation by beta as three shears: beta reduced to [-pi/2, pi/2]
@@ -1908,6 +1950,8 @@ qaoa_status qaoa_simulate_xy(int n, const void *d_costs, qaoa_cost_type ct, cons
     return QAOA_OK;
   }
   const std::vector<XyOp> ops = graph == QAOA_XY_RING ? xy_ring_schedule(n) : xy_complete_schedule(n, c128);
+  std::vector<std::vector<XyRound>> rounds;
+  for (const XyOp &o : ops) rounds.push_back(xy_rounds(o));
   static XyPass P;
   static std::mutex *mu = new std::mutex();
   std::lock_guard<std::mutex> lock(*mu);
@@ -1940,11 +1984,9 @@ qaoa_status qaoa_simulate_xy(int n, const void *d_costs, qaoa_cost_type ct, cons
       P.tb2 = tb2;
       P.sb = sb;
       P.neg = neg;
-      P.ngates = (int)o.gates.size();
-      for (int g = 0; g < P.ngates; ++g) {
-        P.ga[g] = (uint8_t)o.tbit(o.gates[g].first);
-        P.gb[g] = (uint8_t)o.tbit(o.gates[g].second);
-      }
+      P.nrounds = (int)rounds[k].size();
+      if (P.nrounds > kXyMaxRounds) return fail(QAOA_ERR_INVALID_ARG, "internal: too many XY rounds");
+      std::copy(rounds[k].begin(), rounds[k].end(), P.rounds);
       LAUNCH("xy_tile", 2.0 * es * N + (P.has_phase ? cost_bytes(ct) * N : 0.0), s,
              launch_xy_tile(P, c128, s, nsm));
     }

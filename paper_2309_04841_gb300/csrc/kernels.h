@@ -263,9 +263,18 @@ cudaError_t launch_xy_tma(const XyTmaParams &P, bool low, cudaStream_t s, int ns
 cudaError_t launch_xy_tma_u16(const XyTmaParams &P, bool low, cudaStream_t s, int nsm);
 
 // One XY-mixer pass over tiles of 2^tb amplitudes: qubits 0..c-1 (contiguous),
-// h1..h1+w1-1 and h2..h2+w2-1; the gates act on tile bits (ga[g], gb[g]) in order.
+// h1..h1+w1-1 and h2..h2+w2-1, in rounds: round k holds the four tile bits of
+// rounds[k].bit (ascending) in registers and applies, for each set bit of its mask,
+// the gate on register bits xy_gate_a, xy_gate_b, in that (lexicographic) order.
 constexpr int kXyMaxTb = 12;
-constexpr int kXyMaxGates = 64;
+constexpr int kXyMaxRounds = 32;
+// register bits of gate g: (0,1) (0,2) (0,3) (1,2) (1,3) (2,3)
+__host__ __device__ constexpr int xy_gate_a(int g) { return g < 3 ? 0 : g < 5 ? 1 : 2; }
+__host__ __device__ constexpr int xy_gate_b(int g) { return g < 3 ? g + 1 : g < 5 ? g - 1 : 3; }
+struct XyRound {
+  uint8_t bit[4];
+  uint8_t mask;
+};
 struct XyPass {
   void *psi;
   const void *cost;
@@ -276,8 +285,8 @@ struct XyPass {
   double g2pi;               // complex128: g / 2pi
   double tb2, sb;            // tan(b/2), sin(b) of the layer's beta reduced to |b| <= pi/2
   int neg;                   // the reduction took out a factor -1
-  int ngates;
-  uint8_t ga[kXyMaxGates], gb[kXyMaxGates];
+  int nrounds;
+  XyRound rounds[kXyMaxRounds];
   PhaseDigits ph;  // complex64 integer costs: digit tables (mode 0), else computed
 };
 
