@@ -697,7 +697,7 @@ std::vector<PassOp> adjoint_schedule(int k, int p) {
 struct RedRot {
   double t;
   int form;
-  double sigma;
+  SigmaPair sigma;
 };
 
 template <typename Real>
@@ -705,13 +705,7 @@ RedRot red_rot(double b) {
   const double c = cos(b), s = sin(b);
   const int form = fabs(c) >= fabs(s) ? 0 : 1;
   const double t = (double)(Real)(form ? c / s : s / c);
-  return RedRot{t, form, copysign(1.0 / sqrt(1.0 + t * t), form ? s : c)};
-}
-
-double ipow_d(double x, int k) {
-  double r = 1.0;
-  for (int i = 0; i < k; ++i) r *= x;
-  return r;
+  return RedRot{t, form, sigma_pair(t, form ? s : c)};
 }
 
 int sweep_qubits(const Sweep &w) {
@@ -769,7 +763,7 @@ qaoa_status mid_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
       const RedRot R = red_rot<Real>(bet[op.l1]);
       P.t1 = (Real)R.t;
       P.form1 = R.form;
-      sig *= ipow_d(R.sigma, nrot);
+      sig *= sigma_pow(R.sigma, nrot);
     }
     if (op.lp >= 0) {
       make_phase<Real>(P.ph, gam[op.lp], ct, stats, sig);
@@ -779,7 +773,7 @@ qaoa_status mid_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
       const RedRot R = red_rot<Real>(bet[op.l2]);
       P.t2 = (Real)R.t;
       P.form2 = R.form;
-      sig *= ipow_d(R.sigma, nrot);
+      sig *= sigma_pow(R.sigma, nrot);
     }
     P.kind = (op.l1 >= 0 ? 1 : 0) | (op.lp >= 0 ? 2 : 0) | (op.l2 >= 0 ? 4 : 0) | (op.reduce ? 8 : 0);
     if (&op == &ops.back()) {
@@ -828,7 +822,7 @@ qaoa_status mid_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
       P.form1 = Q.form;
       for (int k = 0; k < R; ++k) {
         P.w1[k] = (Real)(sig * sig);
-        sig *= ipow_d(Q.sigma, __builtin_popcount(mid_mask(TB, G.rot, k)));
+        sig *= sigma_pow(Q.sigma, __builtin_popcount(mid_mask(TB, G.rot, k)));
       }
       sums.out_b1 = d_grad_b + op.l1;
     }
@@ -845,7 +839,7 @@ qaoa_status mid_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
       for (int i = 0; i < R; ++i) {
         const int k = R - 1 - i;
         P.w2[k] = (Real)(sig * sig);
-        sig *= ipow_d(Q.sigma, __builtin_popcount(mid_mask(TB, G.rot, k)));
+        sig *= sigma_pow(Q.sigma, __builtin_popcount(mid_mask(TB, G.rot, k)));
       }
       sums.out_b2 = d_grad_b + op.l2;
     }
@@ -902,7 +896,7 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
       const RedRot R = red_rot<Real>(bet[op.l1]);
       P.t1 = (Real)R.t;
       P.form1 = R.form;
-      sig *= ipow_d(R.sigma, sweep_qubits(P.s1));
+      sig *= sigma_pow(R.sigma, sweep_qubits(P.s1));
     }
     if (op.l2 >= 0) {
       P.s2 = G.high ? make_sweep<High>(G.rot, !two) : make_sweep<Low>(G.rot, !two);
@@ -916,7 +910,7 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
       make_phase<Real>(P.ph, gam[op.lp], ct, stats, sig);
       sig = 1.0;
     }
-    if (op.l2 >= 0) sig *= ipow_d(red_rot<Real>(bet[op.l2]).sigma, sweep_qubits(P.s2));
+    if (op.l2 >= 0) sig *= sigma_pow(red_rot<Real>(bet[op.l2]).sigma, sweep_qubits(P.s2));
     P.post_scale = (Real)1;
     if (&op == &ops.back()) {
       P.post_scale = (Real)sig;
@@ -984,7 +978,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
       P.form1 = R.form;
       for (int r = 0; r < Low::NR; ++r) {  // the kernel walks s1 upward
         P.w1[r] = (Real)(sig * sig);
-        sig *= ipow_d(R.sigma, popc8(P.s1.m[r]));
+        sig *= sigma_pow(R.sigma, popc8(P.s1.m[r]));
       }
     }
     P.out_b1 = d_grad_b + op.l1;
@@ -1003,7 +997,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
       for (int k = 0; k < Low::NR; ++k) {  // and s2 downward
         const int r = Low::NR - 1 - k;
         P.w2[r] = (Real)(sig * sig);
-        sig *= ipow_d(R.sigma, popc8(P.s2.m[r]));
+        sig *= sigma_pow(R.sigma, popc8(P.s2.m[r]));
       }
       P.out_b2 = d_grad_b + op.l2;
     }
@@ -1060,7 +1054,7 @@ uint32_t fmin_word(qaoa_cost_type ct, const qaoa_cost_stats *stats) {
 struct TanRot {
   float tau;
   int form;
-  std::complex<double> sigma;
+  SigmaPair sigma;
 };
 
 // Reduced form of exp(-i b X) in the twisted basis (b = -beta for the
@@ -1111,7 +1105,7 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
       const TanRot R = tan_rot(bet[op.l1], false);
       P.tau1 = R.tau;
       P.form1 = R.form;
-      sig *= std::pow(R.sigma, nrot);
+      sig *= sigma_pow(R.sigma, nrot);
     }
     P.has_phase = op.lp >= 0;
     if (P.has_phase) {
@@ -1124,7 +1118,7 @@ qaoa_status tma_forward(int n, const void *cost, qaoa_cost_type ct, const qaoa_c
       const TanRot R = tan_rot(bet[op.l2], false);
       P.tau2 = R.tau;
       P.form2 = R.form;
-      sig *= std::pow(R.sigma, nrot);
+      sig *= sigma_pow(R.sigma, nrot);
     }
     if (&op == &ops.back()) {
       P.end_scale = 1;
@@ -1220,7 +1214,7 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
       // product is the true one divided by |sig|^2
       for (int r = 0; r < Low::NR; ++r) {  // the kernel walks s1 upward
         P.w1[r] = (float)std::norm(sig);
-        sig *= std::pow(R.sigma, popc8(P.s1.m[r]) + popc8(P.s1.lm[r]));
+        sig *= sigma_pow(R.sigma, popc8(P.s1.m[r]) + popc8(P.s1.lm[r]));
       }
     }
     P.out_b1 = d_grad_b + op.l1;
@@ -1240,7 +1234,7 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
       for (int k = 0; k < Low::NR; ++k) {  // and s2 downward
         const int r = Low::NR - 1 - k;
         P.w2[r] = (float)std::norm(sig);
-        sig *= std::pow(R.sigma, popc8(P.s2.m[r]) + popc8(P.s2.lm[r]));
+        sig *= sigma_pow(R.sigma, popc8(P.s2.m[r]) + popc8(P.s2.lm[r]));
       }
       P.out_b2 = d_grad_b + op.l2;
     }
