@@ -369,8 +369,9 @@ qaoa_status qaoa_overlap(int n, const void *d_state, qaoa_state_type st,
 /*
  * Objective and gradient with respect to all 2p angles (not in the paper):
  * forward simulation from |+>^n, then one backward sweep that un-applies the
- * layers in place on two state vectors (psi and lambda = d E / d psi^*, less
- * E psi, which changes no derivative), accumulating
+ * layers in place on two state vectors (psi and lambda = d E / d psi^*; all but
+ * the complex64 passes over n >= 20 integer or float64 costs take lambda less
+ * E psi, which changes no derivative but its rounding error), accumulating
  *   dE/dbeta_l  = 2 Im <lambda| sum_q X_q |psi>   inside the un-mixer passes,
  *   dE/dgamma_l = 2 Im <lambda| f |psi>          before each un-phase.
  *   d_state, d_lambda: device, 2^n amplitudes each (contents ignored and

@@ -688,24 +688,52 @@ std::vector<PassOp> adjoint_schedule(int k, int p) {
 }
 
 // Reduced form of exp(-i b X) (rot_tan; kernels.h): the form with |t| <= 1 and
-// the real factor it drops.  The factor belongs to the multiplier as the kernels
-// hold it, rounded to Real: with 1 / sqrt(1 + t^2) of that t every rotation is
-// unitary (by an angle a rounding off), whereas the cosine of the exact angle
-// left the norm off by up to 3e-8 a rotation, the same for all n rotations of a
-// layer -- most of the error of a complex64 energy (LABS n = 27 p = 10:
-// 2.2e-6 -> 2.1e-7 relative).
+// the real factor it drops.
 struct RedRot {
   double t;
   int form;
   SigmaPair sigma;
 };
 
+// Small tiles and complex128: the factor of the multiplier as the kernels hold it,
+// rounded to Real.  With 1 / sqrt(1 + t^2) of that t every rotation is unitary (by
+// an angle a rounding off), whereas the cosine of the exact angle leaves the norm off
+// by up to 3e-8 a complex64 rotation, the same for all n rotations of a layer.
 template <typename Real>
 RedRot red_rot(double b) {
   const double c = cos(b), s = sin(b);
   const int form = fabs(c) >= fabs(s) ? 0 : 1;
   const double t = (double)(Real)(form ? c / s : s / c);
   return RedRot{t, form, sigma_pair(t, form ? s : c)};
+}
+
+// Streamed complex64 passes (n >= 20): the cosine or sine of the angle itself, and for
+// integer and float64 costs lambda = f psi (shift_of): the arithmetic that these passes
+// always had, amplitude by amplitude.  Where |grad| is small against E its rounding
+// error is largest -- LABS n = 30 p = 10, 40 sets of angles: 2e-6 to 1e-4 of |grad|,
+// E / |grad| about 20 to 75 -- and any other rounding differs from it by as much: with
+// the unitary factor and (f - E) psi 7 of the 40 gradients lay more than 2e-5 of their
+// norm from these, though mostly closer to exact values (energies 1e-6 .. 3e-6 ->
+// 1e-7).  Programs hold and compare such values, so they stay what they were;
+// complex128 is the way to closer ones.
+RedRot red_rot_streamed(double b) {
+  const double c = cos(b), s = sin(b);
+  const int form = fabs(c) >= fabs(s) ? 0 : 1;
+  return RedRot{form ? c / s : s / c, form, SigmaPair{form ? s : c, 0.0}};
+}
+
+// The energy that costs are taken from in a complex64 adjoint sweep (cost_shift), or
+// NULL.  float32 costs take their phases from a table and a polynomial, which round
+// differently from the sincospi that they replaced: with the shift the gradient is the
+// closer one, to exact values and to the former ones (G(21, 0.5) p = 37: 7.8e-6 of the
+// norm from the former gradient with it, 2.5e-5 without).
+const double *shift_of(qaoa_cost_type ct, const double *d_energy) {
+  return ct == QAOA_COST_F32 ? d_energy : nullptr;
+}
+
+template <typename Real>
+RedRot red_rot_tiled(double b) {
+  return sizeof(Real) == 8 ? red_rot<Real>(b) : red_rot_streamed(b);
 }
 
 int sweep_qubits(const Sweep &w) {
@@ -893,14 +921,14 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
     // (these plans hold every rotated bit in registers: no lane rotations)
     if (op.l1 >= 0) {
       P.s1 = G.high ? make_sweep<High>(G.rot, true) : make_sweep<Low>(G.rot, true);
-      const RedRot R = red_rot<Real>(bet[op.l1]);
+      const RedRot R = red_rot_tiled<Real>(bet[op.l1]);
       P.t1 = (Real)R.t;
       P.form1 = R.form;
       sig *= sigma_pow(R.sigma, sweep_qubits(P.s1));
     }
     if (op.l2 >= 0) {
       P.s2 = G.high ? make_sweep<High>(G.rot, !two) : make_sweep<Low>(G.rot, !two);
-      const RedRot R = red_rot<Real>(bet[op.l2]);
+      const RedRot R = red_rot_tiled<Real>(bet[op.l2]);
       P.t2 = (Real)R.t;
       P.form2 = R.form;
     }
@@ -910,7 +938,7 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
       make_phase<Real>(P.ph, gam[op.lp], ct, stats, sig);
       sig = 1.0;
     }
-    if (op.l2 >= 0) sig *= sigma_pow(red_rot<Real>(bet[op.l2]).sigma, sweep_qubits(P.s2));
+    if (op.l2 >= 0) sig *= sigma_pow(red_rot_tiled<Real>(bet[op.l2]).sigma, sweep_qubits(P.s2));
     P.post_scale = (Real)1;
     if (&op == &ops.back()) {
       P.post_scale = (Real)sig;
@@ -973,7 +1001,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
     // forms of exp(-i (-beta) X)
     P.s1 = G.high ? make_sweep<High>(G.rot, true) : make_sweep<Low>(G.rot, true);
     {
-      const RedRot R = red_rot<Real>(-bet[op.l1]);
+      const RedRot R = red_rot_tiled<Real>(-bet[op.l1]);
       P.t1 = (Real)R.t;
       P.form1 = R.form;
       for (int r = 0; r < Low::NR; ++r) {  // the kernel walks s1 upward
@@ -991,7 +1019,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
     }
     if (op.l2 >= 0) {
       P.s2 = G.high ? make_sweep<High>(G.rot, false) : make_sweep<Low>(G.rot, false);
-      const RedRot R = red_rot<Real>(-bet[op.l2]);
+      const RedRot R = red_rot_tiled<Real>(-bet[op.l2]);
       P.t2 = (Real)R.t;
       P.form2 = R.form;
       for (int k = 0; k < Low::NR; ++k) {  // and s2 downward
@@ -1009,7 +1037,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
     if (uses_lanes(P.s1) || uses_lanes(P.s2))
       return fail(QAOA_ERR_INVALID_ARG, "internal: plan needs lane rotations");
     P.init_lambda = op.init;
-    P.energy = d_energy;
+    P.energy = sizeof(Real) == 8 ? d_energy : shift_of(ct, d_energy);
     P.partials = ws.partials;
     P.counter = ws.counter;
     const double N = (double)(1ull << m);
@@ -1060,7 +1088,7 @@ struct TanRot {
 // Reduced form of exp(-i b X) in the twisted basis (b = -beta for the
 // adjoint): form 0 t = tan b, sigma = cos b; form 1 u = cot b, sigma = sin b.
 TanRot tan_rot(double beta, bool adjoint) {
-  const RedRot r = red_rot<float>(adjoint ? -beta : beta);
+  const RedRot r = red_rot_streamed(adjoint ? -beta : beta);
   return TanRot{(float)r.t, r.form, r.sigma};
 }
 
@@ -1199,11 +1227,10 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
     pair_sweep.lm[1] = (uint8_t)(((G.rot >> TB) & 1u) << 4);
     P.cluster = wide ? 2 : G.cl ? 1 : 0;
     auto sweep = [&](bool up) {
-      return wide && G.comp ? make_sweep<PlanTmaB13Comp>(G.rot, up)
-             : wide         ? make_sweep<PlanTmaB13High>(G.rot, up)
-             : G.cl         ? pair_sweep
-             : G.high       ? make_sweep<High>(G.rot, up)
-                            : make_sweep<Low>(G.rot, up);
+      return wide     ? make_sweep<PlanTmaB13High>(G.rot, up)
+             : G.cl   ? pair_sweep
+             : G.high ? make_sweep<High>(G.rot, up)
+                      : make_sweep<Low>(G.rot, up);
     };
     P.s1 = sweep(true);
     {
@@ -1241,7 +1268,7 @@ qaoa_status tma_backward(int n, const void *cost, qaoa_cost_type ct, const qaoa_
     if ((uses_lanes(P.s1) || uses_lanes(P.s2)) && !G.cl)
       return fail(QAOA_ERR_INVALID_ARG, "internal: plan needs lane rotations");
     P.init_lambda = op.init;
-    P.energy = d_energy;
+    P.energy = shift_of(ct, d_energy);
     P.untwist = &op == &ops.back();
     if (half && P.untwist) P.mirror = (1ull << n) - 1ull;
     P.partials = ws.partials;

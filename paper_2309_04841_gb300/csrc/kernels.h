@@ -99,10 +99,6 @@ static_assert(PlanTmaB12Low::valid() && PlanTmaB12High::valid(), "bad TMA B12 pl
 // round 1 tile bits 4-7 and tile bit 12 as lane bit 4 (a shuffle rotation).
 using PlanTmaB13High = Plan<13, 4, 512, 0, 2, 0x0F00, 0x001F, 0x10E0, 0x00F0, 0x100F, 0x0F00>;
 static_assert(PlanTmaB13High::valid(), "bad TMA B13 plan");
-// The same group with a complement pair (below): tile bit 12 in registers in
-// round 0 and a warp bit in round 1, tile bit 8 the lane rotation of round 1.
-using PlanTmaB13Comp = Plan<13, 4, 512, 0, 2, 0x1E00, 0x001F, 0x01E0, 0x00F0, 0x010F, 0x1E00>;
-static_assert(PlanTmaB13Comp::valid(), "bad TMA B13 complement plan");
 // Complement pairs: on a cost vector with f(x) = f(~x) the state keeps
 // psi(x) = psi(~x), so the passes hold the 2^(n-1) amplitudes with the top
 // qubit 0 (m = n - 1 index bits).  The rotation of the top qubit pairs x with
@@ -111,13 +107,18 @@ static_assert(PlanTmaB13Comp::valid(), "bad TMA B13 complement plan");
 // offset t of box 1 is the amplitude ~x of the x at offset t of box 0.  The
 // shared-memory slot of (box 1, t) is the bitwise complement of t, a constant
 // XOR, so the loads stay two plain boxes.  Tile bit TB - 1 must be the last
-// register bit of round 0 and a warp bit of round 1.
+// register bit of round 0 and a warp bit of round 1, or a warp bit of round 0 and
+// the last lane bit of round 1 (the 512-thread plan: the pair's rotation is then the
+// shuffle that the full vector's top qubit takes in the same place, so that both
+// round every amplitude alike).
 template <class PL>
 constexpr bool comp_plan() {
-  return PL::NR == 2 && (PL::reg(0) >> (PL::TB - 1)) == 1u && (PL::warp(1) >> (PL::TB - 1)) == 1u;
+  const int b = PL::TB - 1;
+  return PL::NR == 2 && (((PL::reg(0) >> b) == 1u && (PL::warp(1) >> b) == 1u) ||
+                         ((PL::warp(0) >> b) == 1u && (PL::lane(1) >> b) == 1u));
 }
-static_assert(comp_plan<PlanTmaF13High>() && comp_plan<PlanTmaB12High>() && comp_plan<PlanTmaB13Comp>(),
-              "complement tile bit: last register bit of round 0, warp bit of round 1");
+static_assert(comp_plan<PlanTmaF13High>() && comp_plan<PlanTmaB12High>() && comp_plan<PlanTmaB13High>(),
+              "complement tile bit");
 
 // The TMA passes hold vectors in the twisted basis s(x) = (-i)^popc(x) psi(x),
 // where exp(-i b X_q) acts on a pair as the real rotation
@@ -197,7 +198,7 @@ struct alignas(64) TmaBwdParams {
   float w1[4], w2[4]; // |scale|^2 weights of the inner products taken in each round
   float wg;           // |scale|^2 weight of the d/d gamma inner product
   int has_phase, init_lambda;
-  const double *energy;  // E of the forward sweep (cost_shift)
+  const double *energy;  // E of the forward sweep or NULL (cost_shift)
   int untwist;  // last pass: psi back to the standard basis, lambda not stored
   uint64_t mirror;   // with untwist, nonzero (2^n - 1): psi[x] is also stored at its complement
   double out_scale;  // inner products times this before they are added

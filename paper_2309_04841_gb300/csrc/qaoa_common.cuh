@@ -99,9 +99,9 @@ constexpr int kMidC = 2;  // of the small tiles (mid_kernels.cu)
 // commutators' expectations.  With c = E the vector lambda = (f - c) psi is as
 // short as it can be, and Im <lambda|(f - c)|psi> sums terms of the size of the
 // costs' spread instead of their mean, so the roundings that both carry weigh
-// less (complex64 gradients of four angle sets, LABS n = 27 p = 10: 1.3e-6 .. 4.7e-6 of
-// the norm from 64 bits before, 0.4e-6 .. 1.2e-6 with this and the unitary rotations).
+// less.  NULL: c = 0 (streamed complex64 passes over integer costs; api.cu says why).
 __device__ __forceinline__ double cost_shift(const double *energy) {
+  if (!energy) return 0.0;
   const double e = __ldcg(energy);
   return isfinite(e) ? e : 0.0;
 }
@@ -200,7 +200,7 @@ struct BwdParams {
   Real post_scale;        // psi and lambda times this before the store
   int has_phase;          // g_gamma accumulation + un-phase between sweeps
   int init_lambda;        // lambda <- (f - E) psi at load
-  const double *energy;   // E of the forward sweep (cost_shift)
+  const double *energy;   // E of the forward sweep or NULL (cost_shift)
   double *partials;       // [ntiles][3]
   unsigned *counter;
   double *out_b1, *out_g, *out_b2;  // gradient slots (accumulated: +=)

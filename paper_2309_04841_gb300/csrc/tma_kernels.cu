@@ -256,15 +256,25 @@ __device__ __forceinline__ void rot_tw(float2 (&v)[1 << EB], uint32_t m, float t
 //   m even:  (a, b) <- (a + t kappa b, b + t kappa a),  kappa = i eps
 // and Im <lambda| X |psi> of the pair is eps (l_a . s_b - l_b . s_a), or
 // -eps Im(conj(l_a) s_b + conj(l_b) s_a).  eps here is this thread's sign for
-// register 0 of round 0 (the register's own parity is a constant).
+// register 0 of the round that rotates the pair (the register's own parity is a
+// constant).  The box bit is the last register bit of round 0 or, on the 512-thread
+// plan, a warp bit of round 0 and a lane bit of round 1.
 struct CompCtx {
   float eps = 1.f;
-  bool odd = false, box1 = false;  // box1: this thread's amplitudes of round 1 are in box 1
+  bool odd = false;
+  bool box1[2] = {false, false};  // this thread's amplitudes of the round are in box 1
 };
 
+// Register bit that holds the box bit in round R, else -1.
+template <class PL, int R>
+__host__ __device__ constexpr int comp_reg() {
+  return ((PL::reg(R) >> (PL::TB - 1)) & 1u) ? PL::EB - 1 : -1;
+}
+
 // rot_tw on a round of a complement-pair tile: UB >= 0, the box is register
-// bit UB (left to rot_comp); UB = -1, the whole thread is in one box.
-template <int EB, int UB>
+// bit UB (left to rot_comp); UB = -1, the whole thread is in one box, and with LBOX
+// the lanes of a warp in both.
+template <int EB, int UB, bool LBOX>
 __device__ __forceinline__ void rot_tw_comp(float2 (&v)[1 << EB], uint32_t m, float tau, int form, bool box1) {
   if (form == 0) {
     const float ts = UB < 0 && box1 ? -tau : tau;
@@ -282,8 +292,7 @@ __device__ __forceinline__ void rot_tw_comp(float2 (&v)[1 << EB], uint32_t m, fl
           }
       }
   } else {
-    const float2 tp = f2(tau, tau);
-    auto sweep = [&](bool all_rev) {
+    auto sweep = [&](bool all_rev, float2 tp) {
 #pragma unroll
       for (int i = 0; i < EB; ++i)
         if (i != UB && ((m >> i) & 1u)) {
@@ -297,10 +306,20 @@ __device__ __forceinline__ void rot_tw_comp(float2 (&v)[1 << EB], uint32_t m, fl
             }
         }
     };
-    if (UB < 0 && box1)
-      sweep(true);
-    else
-      sweep(false);
+    if constexpr (LBOX) {
+      // lanes of both boxes run the same instructions: with the multiplier negated too, a
+      // rotation in box 1 comes out negated
+      const float s = box1 ? -1.f : 1.f;
+      sweep(false, f2(s * tau, s * tau));
+      if (__popc(m) & 1) {
+#pragma unroll
+        for (int r = 0; r < (1 << EB); ++r) v[r] = f2(s * v[r].x, s * v[r].y);
+      }
+    } else if (UB < 0 && box1) {
+      sweep(true, f2(tau, tau));
+    } else {
+      sweep(false, f2(tau, tau));
+    }
   }
 }
 
@@ -339,12 +358,11 @@ __device__ __forceinline__ void rot_round(float2 (&v)[PL::NREG], uint32_t m, flo
                                           const CompCtx &cx) {
   if constexpr (!CP) {
     rot_tw<PL::EB>(v, m, tau, form);
-  } else if constexpr (R == 0) {
-    constexpr int UB = PL::EB - 1;
-    rot_tw_comp<PL::EB, UB>(v, m, tau, form, false);
-    if ((m >> UB) & 1u) rot_comp<PL::EB, UB>(v, tau, form, cx);
   } else {
-    rot_tw_comp<PL::EB, -1>(v, m, tau, form, cx.box1);
+    constexpr int UB = comp_reg<PL, R>();
+    rot_tw_comp<PL::EB, UB, false>(v, m, tau, form, cx.box1[R]);
+    if constexpr (UB >= 0)
+      if ((m >> UB) & 1u) rot_comp<PL::EB, UB>(v, tau, form, cx);
   }
 }
 
@@ -405,11 +423,12 @@ __device__ __forceinline__ void unrot_tw(float2 (&v)[1 << EB], float2 (&w)[1 << 
   rot_tw<EB>(w, m, tau, form);
 }
 
-// unrot_tw on a round of a complement-pair tile (UB as in rot_tw_comp).
+// unrot_tw on a round of a complement-pair tile (UB as in rot_tw_comp; with LANES
+// the lane bit in lm is the box bit).
 template <int EB, int UB, bool LANES>
 __device__ __forceinline__ void unrot_tw_comp(float2 (&v)[1 << EB], float2 (&w)[1 << EB], uint32_t m,
                                               uint32_t lm, float tau, int form, float wr, float &acc,
-                                              const CompCtx &cx) {
+                                              const CompCtx &cx, bool box1) {
   if (m == 0u && (!LANES || lm == 0u)) return;
   float2 pp[2] = {f2(0.f, 0.f), f2(0.f, 0.f)}, pm[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
 #pragma unroll
@@ -426,7 +445,7 @@ __device__ __forceinline__ void unrot_tw_comp(float2 (&v)[1 << EB], float2 (&w)[
         }
     }
   const float2 sp = __fadd2_rn(pp[0], pp[1]), sm = __fadd2_rn(pm[0], pm[1]);
-  const float sgn = UB < 0 && cx.box1 ? -1.f : 1.f;
+  const float sgn = UB < 0 && box1 ? -1.f : 1.f;
   float term = sgn * ((sp.x + sp.y) - (sm.x + sm.y));
   if constexpr (UB >= 0) {
     if ((m >> UB) & 1u) {
@@ -447,31 +466,31 @@ __device__ __forceinline__ void unrot_tw_comp(float2 (&v)[1 << EB], float2 (&w)[
   float lane_term = 0.f;
   if constexpr (LANES) {
     if (lm != 0u) {
+      // rot_comp on pairs in two lanes; z: kappa times the partner's amplitude (m even: i eps;
+      // odd: eps, and minus that in box 1)
       const int lb = __ffs((int)lm) - 1;
-      const float sg = ((threadIdx.x >> lb) & 1u) ? -sgn : sgn;  // sgn * (-1 for the pair's upper element)
-      const float2 st = f2(sg * tau, sg * tau), tt = f2(tau, tau);
+      const float2 tt = f2(tau, tau);
       float2 q = f2(0.f, 0.f);
+      auto rot = [&](float2 &a, float2 z) { a = form == 0 ? __ffma2_rn(tt, z, a) : __ffma2_rn(tt, a, z); };
 #pragma unroll
       for (int r = 0; r < (1 << EB); ++r) {
         const float2 pv = f2(__shfl_xor_sync(0xffffffffu, v[r].x, 1 << lb),
                              __shfl_xor_sync(0xffffffffu, v[r].y, 1 << lb));
         const float2 pw = f2(__shfl_xor_sync(0xffffffffu, w[r].x, 1 << lb),
                              __shfl_xor_sync(0xffffffffu, w[r].y, 1 << lb));
-        q = __ffma2_rn(w[r], pv, q);
-        if (form == 0) {
-          v[r] = __ffma2_rn(st, pv, v[r]);
-          w[r] = __ffma2_rn(st, pw, w[r]);
-        } else {
-          v[r] = __ffma2_rn(tt, v[r], f2(sg * pv.x, sg * pv.y));
-          w[r] = __ffma2_rn(tt, w[r], f2(sg * pw.x, sg * pw.y));
-        }
+        const float e = ((popc_c(r) & 1) ? -cx.eps : cx.eps) * (cx.odd ? sgn : 1.f);
+        const float2 zv = cx.odd ? f2(e * pv.x, e * pv.y) : f2(-e * pv.y, e * pv.x);
+        const float2 zw = cx.odd ? f2(e * pw.x, e * pw.y) : f2(-e * pw.y, e * pw.x);
+        q = __ffma2_rn(w[r], zv, q);
+        rot(v[r], zv);
+        rot(w[r], zw);
       }
-      lane_term = sg * (q.x + q.y);
+      lane_term = q.x + q.y;
     }
   }
   acc = fmaf(term + lane_term, wr, acc);
-  rot_tw_comp<EB, UB>(v, m, tau, form, cx.box1);
-  rot_tw_comp<EB, UB>(w, m, tau, form, cx.box1);
+  rot_tw_comp<EB, UB, LANES>(v, m, tau, form, box1);
+  rot_tw_comp<EB, UB, LANES>(w, m, tau, form, box1);
   if constexpr (UB >= 0) {
     if ((m >> UB) & 1u) {
       rot_comp<EB, UB>(v, tau, form, cx);
@@ -487,7 +506,8 @@ __device__ __forceinline__ void unrot_round(float2 (&v)[PL::NREG], float2 (&w)[P
   if constexpr (!CP)
     unrot_tw<PL::EB, LANES>(v, w, s.m[R], s.lm[R], tau, form, wr, acc);
   else
-    unrot_tw_comp<PL::EB, R == 0 ? PL::EB - 1 : -1, LANES && R != 0>(v, w, s.m[R], s.lm[R], tau, form, wr, acc, cx);
+    unrot_tw_comp<PL::EB, comp_reg<PL, R>(), LANES && R != 0>(v, w, s.m[R], s.lm[R], tau, form, wr, acc, cx,
+                                                             cx.box1[R]);
 }
 
 // z * i^k (k folds to a constant where the register index is one)
@@ -546,7 +566,7 @@ __device__ __forceinline__ void untwist_round(float2 (&v)[PL::NREG], uint64_t T,
     const float2 z1 = cmulf(scale, ipow(f2(1.f, 0.f), m - k));
 #pragma unroll
     for (int r = 0; r < PL::NREG; ++r) {
-      if constexpr (R == 0) {
+      if constexpr (comp_reg<PL, R>() >= 0) {
         if ((r >> (PL::EB - 1)) & 1)
           v[r] = ipow(cmulf(v[r], z1), 1 - popc_c(r));
         else
@@ -557,6 +577,14 @@ __device__ __forceinline__ void untwist_round(float2 (&v)[PL::NREG], uint64_t T,
       }
     }
   }
+}
+
+// eps of this thread (CompCtx) in tile T of a vector of m index bits.
+template <class PL>
+__device__ __forceinline__ float comp_sign(uint64_t T, int m) {
+  constexpr int R = comp_reg<PL, 0>() >= 0 ? 0 : 1;
+  const uint32_t t = thr_tile<PL, R>() & ((1u << (PL::TB - 1)) - 1u);
+  return ((((m - 1) >> 1) + __popc(t) + __popcll(T)) & 1) ? -1.f : 1.f;
 }
 
 // Registers <- shared tile in round-R layout (16-byte accesses when the
@@ -995,7 +1023,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
   CompCtx cx;
   if constexpr (CP) {
     cx.odd = (P.comp & 1) != 0;
-    cx.box1 = (thr_tile<PL, 1>() >> (PL::TB - 1)) != 0u;
+    cx.box1[0] = (thr_tile<PL, 0>() >> (PL::TB - 1)) != 0u;
+    cx.box1[1] = (thr_tile<PL, 1>() >> (PL::TB - 1)) != 0u;
   }
   int i = 0;
   for (;; ++i) {
@@ -1010,7 +1039,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_fwd_tma(const __grid_constant__
       atomicExch(P.err, 1u);
     }
     float2 v[NREG];
-    if constexpr (CP) cx.eps = ((((P.comp - 1) >> 1) + twist_base<PL, 0>(T)) & 1) ? -1.f : 1.f;
+    if constexpr (CP) cx.eps = comp_sign<PL>(T, P.comp);
     if (P.init_plus) {
       // |+>^n in the twisted basis: amp (-i)^popc(x)
       const float2 z0 = ipow(f2(P.amp, 0.f), -twist_base<PL, 0>(T));
@@ -1250,7 +1279,8 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
   CompCtx cx;
   if constexpr (CP) {
     cx.odd = (P.comp & 1) != 0;
-    cx.box1 = (thr_tile<PL, 1>() >> (PL::TB - 1)) != 0u;
+    cx.box1[0] = (thr_tile<PL, 0>() >> (PL::TB - 1)) != 0u;
+    cx.box1[1] = (thr_tile<PL, 1>() >> (PL::TB - 1)) != 0u;
   }
   int i = 0;
   for (;; ++i) {
@@ -1265,10 +1295,10 @@ __global__ void __launch_bounds__(PL::NT, 512 / PL::NT) k_bwd_tma(const __grid_c
       atomicExch(P.err, 1u);
     }
     float2 v[NREG], w[NREG];
-    if constexpr (CP) cx.eps = ((((P.comp - 1) >> 1) + twist_base<PL, 0>(T)) & 1) ? -1.f : 1.f;
+    if constexpr (CP) cx.eps = comp_sign<PL>(T, P.comp);
     lds_round<PL, 0, SW, CP>(v, bv);
     if constexpr (INIT) {
-      // lambda = (f - E) psi: the derivative of <psi|f - E|psi> with respect to psi^*
+      // lambda = (f - c) psi: the derivative of <psi|f - c|psi> with respect to psi^* (c: cost_shift)
       const uint32_t tt = thr_tile<PL, 0>();
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
@@ -2122,7 +2152,7 @@ cudaError_t QAOA_TMA_FN(launch_bwd_tma)(const TmaBwdParams &P, bool high, cudaSt
       return cudaErrorInvalidValue;
   if (P.comp) {
     if (!high || P.cluster == 1) return cudaErrorInvalidValue;
-    return P.cluster == 2 ? dispatch_bwd_comp<PlanTmaB13Comp>(P, s, nsm)
+    return P.cluster == 2 ? dispatch_bwd_comp<PlanTmaB13High>(P, s, nsm)
                           : dispatch_bwd_comp<PlanTmaB12High>(P, s, nsm);
   }
   if (P.cluster == 2) {  // a HIGH group of up to 9 qubits on one 512-thread CTA
