@@ -164,6 +164,8 @@ void make_phase(PhaseData<Real> &ph, double g, qaoa_cost_type ct, const qaoa_cos
   const int shift = stats->step_log2 < 31 ? (int)stats->step_log2 : 0;
   const double top = std::floor((stats->f_max - stats->f_min) / std::ldexp(1.0, shift));  // the largest d
   if (!(top >= 0 && top < 262144.0) || !(stats->f_min >= -2147483648.0 && stats->f_max <= 2147483647.0)) return;
+  // (the tables' own offsets, digit << shift, are int32: a range of 2^31 and more is computed)
+  if (stats->f_max - stats->f_min >= 2147483648.0) return;
   const int n1 = (int)top / 64 + 1;
   ph.mode = 0;
   ph.fmin = (int)stats->f_min;

@@ -1,0 +1,48 @@
+"""Every way to a phase exp(-i gamma f) of integer costs -- tables of two and three digits, computed -- against the
+oracle, on chip, on the small tiles and on the streamed passes of both precisions.
+
+Tolerances as in test_gpu_half.py: 5e-6 of the norm for complex64 states of p = 2 layers and n <= 21, 1e-13 for
+complex128, ten times that for gradients.  Phases of |gamma f| <= 100 are reduced from a float pair (2^-48) or a
+double pair, below both."""
+import numpy as np
+import pytest
+
+from gpu_util import dev_np
+import oracle
+from paper_2309_04841_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def Q():
+    from paper_2309_04841_gb300 import qaoa
+    return qaoa
+
+
+def check(Q, n, terms, scale, st, symmetric=False):
+    """Simulation and gradient of an integer polynomial at p = 2, gammas up to `scale`."""
+    f = oracle.costs_terms_int(n, terms).astype(float)
+    fd = Q.precompute_costs(n, terms)
+    s = Q.cost_stats_compute(fd)
+    assert (s.f_min, s.f_max) == (f.min(), f.max()) and (s.reserved != 0) == symmetric
+    g, b = I.angles(2, 5 + n, 0.2 * scale, scale), I.angles(2, 70 + n)
+    tol = 5e-6 if st == Q.C64 else 1e-13
+    x, e = Q.simulate(fd, s, g, b, state_type=st)
+    assert np.linalg.norm(dev_np(x) - oracle.simulate(n, f, g, b)) < tol
+    E, dg, db = oracle.grad(n, f, g, b)
+    out = dev_np(Q.grad(fd, s, g, b, state_type=st))
+    spread = np.abs(f).max()
+    assert abs(out[0] - E) <= 10 * tol * spread and abs(dev_np(e)[0] - E) <= 10 * tol * spread
+    for got, ref in ((out[2:4], dg), (out[4:], db)):  # d/d gamma is a factor 1 / scale the larger
+        assert np.linalg.norm(got - ref) <= 10 * tol * max(np.linalg.norm(ref), spread)
+    return s
+
+
+# values +-2^30 +-2^29: steps of 2^30, a range of 3 2^30, so digit << shift leaves int32
+@pytest.mark.parametrize("n,st", [(4, 0), (12, 0), (12, 1), (13, 0), (14, 0), (14, 1), (16, 1), (19, 0), (21, 0), (21, 1)])
+@pytest.mark.parametrize("odd", [False, True])
+def test_range_over_int32(Q, n, st, odd):
+    terms = [(2 ** 30, (0, n - 1)), (2 ** 29, (1,) if odd else (1, 2))]
+    s = check(Q, n, terms, 4e-9, st, symmetric=not odd)
+    assert s.step_log2 == 30 and s.f_max - s.f_min == 3 * 2 ** 30
