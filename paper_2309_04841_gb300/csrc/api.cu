@@ -156,9 +156,7 @@ template <typename Real>
 void make_phase(PhaseData<Real> &ph, double g, qaoa_cost_type ct, const qaoa_cost_stats *stats, double scale) {
   memset(&ph, 0, sizeof(ph));
   ph.mode = 1;
-  ph.g2pi = g / kTwoPi;
-  ph.g_hi = (float)ph.g2pi;
-  ph.g_lo = (float)(ph.g2pi - (double)ph.g_hi);
+  turns_pair(g, ph.g_hi, ph.g_lo);
   ph.scl = (Real)scale;
   if (!integer_cost(ct) || !stats) return;
   const int shift = stats->step_log2 < 31 ? (int)stats->step_log2 : 0;

@@ -222,8 +222,8 @@ __device__ __forceinline__ float2 phase_at(const PhaseData<float> &ph, float fh,
   return make_float2(cs * scl, -sn * scl);
 }
 __device__ __forceinline__ double2 phase_at(const PhaseData<double> &ph, double f, double scl) {
-  const double t = ph.g2pi * f;
-  const double r = t - rint(t);
+  const double p = ph.g_hi * f;
+  const double r = (p - rint(p)) + fma(ph.g_lo, f, fma(ph.g_hi, f, -p));
   double sn, cs;
   sincospi(2.0 * r, &sn, &cs);
   return make_double2(cs * scl, -sn * scl);

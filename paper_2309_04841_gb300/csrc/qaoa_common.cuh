@@ -143,7 +143,8 @@ struct Sweep {
 // d = (f - fmin) >> shift: exp(-i g f) = T0[d & 63] T1[d >> 6] (nd 2), or three
 // digits, T0[d & 63] T1[(d >> 6) & 63] T2[d >> 12]; each CTA builds the `entries`
 // of its tables (fill_phase).  Mode 1: computed per amplitude.  Both reduce
-// g f / 2 pi, in complex64 as a float-float.
+// g f / 2 pi from g / 2 pi as a pair of Reals: rounded to one it would be off by a
+// relative error that all amplitudes share.
 constexpr int kTileTable = 192;  // most entries
 template <typename Real>
 struct PhaseData {
@@ -151,8 +152,7 @@ struct PhaseData {
   int mode;
   int fmin, shift;
   int nd, last, entries;  // digits; entries of the last table - 1; of all
-  float g_hi, g_lo;  // complex64: g / 2pi = g_hi + g_lo
-  double g2pi;       // complex128: g / 2pi
+  Real g_hi, g_lo;   // g / 2pi = g_hi + g_lo
   Real scl;          // factor applied with the phase (the last table carries it)
 };
 
@@ -308,9 +308,9 @@ template <typename Real>
 struct SmallLayer {
   Real tau, sig, sig_adj, wg;
   Real w[2][SmallTile<Real>::kMaxRounds], w_comp[2];  // [1] upward, [0] downward
+  Real g_hi, g_lo;  // g / 2pi = g_hi + g_lo
   int form;
-  float g_hi, g_lo;  // g / 2pi split (complex64)
-  double g2pi;       // g / 2pi (complex128)
+  int pad;  // to 8-byte words (copied as such)
 };
 
 // One request for the on-chip kernels (a launch of k_small runs one, a launch

@@ -95,9 +95,9 @@ template <> struct Ops<double> {
   __device__ static __forceinline__ double value(F f) { return f; }
   template <class L>
   __device__ static __forceinline__ C2 phase(const L &l, F f, double scl) {
-    const double t = l.g2pi * f;
+    const double p = l.g_hi * f;
     double sn, cs;
-    sincospi(2.0 * (t - rint(t)), &sn, &cs);
+    sincospi(2.0 * ((p - rint(p)) + fma(l.g_lo, f, fma(l.g_hi, f, -p))), &sn, &cs);
     return make_double2(cs * scl, -sn * scl);
   }
   __device__ static __forceinline__ F real(const void *c, int kind, uint64_t x) {

@@ -46,3 +46,24 @@ def test_range_over_int32(Q, n, st, odd):
     terms = [(2 ** 30, (0, n - 1)), (2 ** 29, (1,) if odd else (1, 2))]
     s = check(Q, n, terms, 4e-9, st, symmetric=not odd)
     assert s.step_log2 == 30 and s.f_max - s.f_min == 3 * 2 ** 30
+
+
+# complex128: at beta = 0 a layer is the phase alone, exp(-i gamma f) 2^(-n/2), here with |gamma f| up to about 430.
+# The fraction of gamma f / 2 pi is known to 2^-54 of a turn (3.5e-16 in the angle), sincospi adds 2.2e-16, a table's
+# product as much again for each of up to three factors: 2e-15 in all.  (With gamma / 2 pi in one double the angle is
+# off by |gamma f| 2^-53 and more: 5e-14.)
+@pytest.mark.parametrize("kind", ["i32", "f64"])
+@pytest.mark.parametrize("n", [5, 8, 12, 14, 18, 21])
+@pytest.mark.parametrize("half", [False, True])
+def test_double_phase(Q, n, kind, half):
+    f = oracle.labs_costs(n)
+    fd = Q.labs_costs(n) if kind == "i32" else Q.labs_costs(n).double()
+    s = Q.cost_stats_compute(fd)
+    if not half:
+        s.reserved = 0
+    gamma = 430.1 / f.max()
+    x, _ = Q.simulate(fd, s, [gamma], [0.0], state_type=Q.C128)
+    v, at = np.unique(f, return_inverse=True)
+    a = np.longdouble(gamma) * v.astype(np.longdouble)
+    ref = (np.cos(a).astype(float) - 1j * np.sin(a).astype(float))[at.reshape(-1)]
+    assert np.abs(dev_np(x) * 2.0 ** (n / 2) - ref).max() < 2e-15
