@@ -172,26 +172,27 @@ def state_dtype(st):
     return {C64: torch.complex64, C128: torch.complex128}[st]
 
 
-_dtype_codes = {}  # torch dtype -> cost type, state type
+_dtype_codes = None  # (torch dtype -> cost type, torch dtype -> state type)
 
 
 def _codes():
-    if not _dtype_codes:
+    global _dtype_codes
+    if _dtype_codes is None:
         torch = _torch()
-        _dtype_codes["cost"] = {torch.int32: COST_I32, torch.float32: COST_F32, torch.float64: COST_F64,
-                                torch.int16: COST_U16}
+        cost = {torch.int32: COST_I32, torch.float32: COST_F32, torch.float64: COST_F64, torch.int16: COST_U16}
         if hasattr(torch, "uint16"):
-            _dtype_codes["cost"][torch.uint16] = COST_U16
-        _dtype_codes["state"] = {torch.complex64: C64, torch.complex128: C128}
+            cost[torch.uint16] = COST_U16
+        # one assignment of the finished tables: other threads see both or neither
+        _dtype_codes = cost, {torch.complex64: C64, torch.complex128: C128}
     return _dtype_codes
 
 
 def cost_type_of(costs):
-    return _codes()["cost"][costs.dtype]
+    return _codes()[0][costs.dtype]
 
 
 def state_type_of(state):
-    return _codes()["state"][state.dtype]
+    return _codes()[1][state.dtype]
 
 
 def _n_of(t):
