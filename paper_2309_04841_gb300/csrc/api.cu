@@ -217,9 +217,10 @@ void make_phase(PhaseDigits &ph, double g, qaoa_cost_type ct, const qaoa_cost_st
       put(64 + j, g * fmin + unit * 1024.0 * j, true);
     }
   } else {
-    ph.mode = 1;
-    ph.nd = integer_cost(ct) ? 0 : 1;
     const double g2 = g / kTwoPi;
+    ph.mode = 1;
+    ph.real = !integer_cost(ct);
+    ph.nd = ph.real && stats && std::max(fabs(stats->f_min), fabs(stats->f_max)) * fabs(g2) < 6.9e10 ? 1 : 0;
     ph.g_hi = (float)g2;
     ph.g_lo = (float)(g2 - (double)ph.g_hi);
     ph.nent = 64;

@@ -141,7 +141,11 @@ static_assert(comp_plan<PlanTmaF13High>() && comp_plan<PlanTmaB12High>() && comp
 // g / 2pi = g_hi + g_lo (float-float): the fraction r of g f / 2pi splits into
 // k / 64, looked up in d[] = scale * exp(-2 pi i k / 64), and a rest of at most
 // 1 / 128, whose sine and cosine are their Taylor polynomials (to the third and
-// fourth power; the next terms are 2e-9).  It is the pivots' arithmetic that costs
+// fourth power; the next terms are 2e-9).  64 r has to be a small number for that: its
+// integer part must fit the mantissa beside the rounding constant.  The low part of
+// g f / 2pi, up to 2^-25 of it, is part of r, so from |g f / 2pi| = 2^36 on (penalties of
+// 1e12, say) nd = 0 takes the form that reduces r once more; nd = 1 (float32 costs below)
+// does without, 0.8% of a weighted MaxCut n = 28 gradient.  It is the pivots' arithmetic that costs
 // there: weighted MaxCut n = 28 pivots 658 -> 556 us forward and 1339 -> 1152 us
 // adjoint against sincospi and a scale multiply per amplitude.
 constexpr int kPhaseCopies = 16;
@@ -152,7 +156,8 @@ struct PhaseDigits {
   int mode;
   int fmin;
   int shift;
-  int nd;     // 2 or 3 digits
+  int nd;     // 2 or 3 digits; mode 1: float32 costs of ordinary size (1) or any (0)
+  int real;   // mode 1: float32 costs
   int last;   // entries of the last table - 1 (its index is clamped to this)
   int nent;   // entries in use
   float g_hi, g_lo;

@@ -653,7 +653,7 @@ struct NoHook {
 };
 
 // scale * exp(-i g f) from the raw 32-bit cost word; M = 2 / 3: digit tables with M
-// digits (integer costs), M = 1 / 0: computed (float32 / integer costs).  Callers
+// digits (integer costs), M = 1 / 0: computed (float32 / any costs).  Callers
 // branch on the mode once per round, outside their register loops.
 template <int M>
 __device__ __forceinline__ float2 phase_of(const PhaseDigits &ph, const float2 *tab, uint32_t word) {
@@ -678,12 +678,14 @@ __device__ __forceinline__ float2 phase_of(const PhaseDigits &ph, const float2 *
       const float f = __uint_as_float(word);
       const float p = ph.g_hi * f;
       r = (p - rintf(p)) + fmaf(ph.g_lo, f, fmaf(ph.g_hi, f, -p));
-    } else {  // int32 or uint16 of a range beyond the tables
+    } else {  // integers of a range beyond the tables; float32 of any size
       const int f = (int)word;
-      const float fh = (float)f, fl = (float)((long long)f - (long long)fh);
+      const float fh = ph.real ? __uint_as_float(word) : (float)f;
+      const float fl = ph.real ? 0.f : (float)((long long)f - (long long)fh);
       const float p = ph.g_hi * fh;
       const float e = fmaf(ph.g_hi, fh, -p);
       r = (p - rintf(p)) + (e + fmaf(ph.g_hi, fl, ph.g_lo * fh));
+      r -= rintf(r);  // e alone is many turns from |p| = 2^24 on
     }
     const float m = fmaf(r, 64.f, 12582912.f);  // 1.5 2^23: the low bits are k = rint(64 r)
     const float2 t = tab[((__float_as_uint(m) & 63u) << 4) | (threadIdx.x & (kPhaseCopies - 1))];

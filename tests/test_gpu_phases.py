@@ -67,3 +67,25 @@ def test_double_phase(Q, n, kind, half):
     a = np.longdouble(gamma) * v.astype(np.longdouble)
     ref = (np.cos(a).astype(float) - 1j * np.sin(a).astype(float))[at.reshape(-1)]
     assert np.abs(dev_np(x) * 2.0 ** (n / 2) - ref).max() < 2e-15
+
+
+# Costs so large that even the low part of gamma f / 2 pi, a float pair, is many turns: the phase carries no
+# information then, but every factor still has modulus one, and the amplitudes of the costs beside them are exact.
+@pytest.mark.parametrize("n", [12, 14, 21, 22])
+@pytest.mark.parametrize("half", [False, True])
+def test_penalty_costs(Q, n, half):
+    import torch
+    f = Q.labs_costs(n).float()
+    big = torch.logspace(10, 35, f[5::64].numel(), dtype=torch.float64).float()
+    f[5::64] = big.to(f.device)
+    if half:
+        f = torch.maximum(f, f.flip(0))
+    s = Q.cost_stats_compute(f)
+    assert (s.reserved != 0) == half
+    x, _ = Q.simulate(f, s, [0.31], [0.0], state_type=Q.C64)
+    x = dev_np(x) * 2.0 ** (n / 2)
+    f0 = dev_np(f).astype(float)
+    assert np.abs(np.abs(x) - 1.0).max() < 2e-6  # the phase's and the scale's roundings
+    assert np.abs(x - np.exp(-1j * 0.31 * f0))[f0 < 1e6].max() < 2e-6
+    x, _ = Q.simulate(f, s, [0.31, 0.23], [0.4, 0.2], state_type=Q.C64)
+    assert abs(float(torch.linalg.vector_norm(x)) - 1.0) < 5e-6
