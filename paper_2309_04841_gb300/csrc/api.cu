@@ -158,6 +158,7 @@ void make_phase(PhaseData<Real> &ph, double g, qaoa_cost_type ct, const qaoa_cos
   ph.mode = 1;
   turns_pair(g, ph.g_hi, ph.g_lo);
   ph.scl = (Real)scale;
+  ph.scl_lo = (Real)(scale - (double)ph.scl);
   if (!integer_cost(ct) || !stats) return;
   const int shift = stats->step_log2 < 31 ? (int)stats->step_log2 : 0;
   const double top = std::floor((stats->f_max - stats->f_min) / std::ldexp(1.0, shift));  // the largest d

@@ -147,7 +147,7 @@ __device__ __forceinline__ void fill_tables(C2 *tab, const PhaseData<Real> &ph) 
   for (int i = threadIdx.x; i < ph.entries; i += NT) {
     const int digit = min(i >> 6, ph.nd - 1), j = (i - 64 * digit) << (6 * digit + ph.shift);
     const bool last = i >= 64 * (ph.nd - 1);
-    tab[i] = O::phase(ph, O::integer(last ? ph.fmin + j : j), last ? ph.scl : (Real)1);
+    tab[i] = O::entry(ph, O::integer(last ? ph.fmin + j : j), last ? ph.scl : (Real)1, last ? ph.scl_lo : (Real)0);
   }
 }
 

@@ -153,7 +153,7 @@ struct PhaseData {
   int fmin, shift;
   int nd, last, entries;  // digits; entries of the last table - 1; of all
   Real g_hi, g_lo;   // g / 2pi = g_hi + g_lo
-  Real scl;          // factor applied with the phase (the last table carries it)
+  Real scl, scl_lo;  // factor applied with the phase (the last table carries it), as a pair
 };
 
 template <typename Real>

@@ -89,3 +89,22 @@ def test_penalty_costs(Q, n, half):
     assert np.abs(x - np.exp(-1j * 0.31 * f0))[f0 < 1e6].max() < 2e-6
     x, _ = Q.simulate(f, s, [0.31, 0.23], [0.4, 0.2], state_type=Q.C64)
     assert abs(float(torch.linalg.vector_norm(x)) - 1.0) < 5e-6
+
+
+# complex64 tables: with beta = 0 a layer multiplies every amplitude by the same table product, so 32 equal layers add an
+# entry's error up 32 times.  Entries within 0.55 ulp (2.4e-8 rms a complex entry below one) and one product of two
+# (3.4e-8): 32 sqrt(2 * 2.4^2 + 3.4^2) e-8 = 1.5e-6 rms; with the angle rounded to float before its sine and cosine an
+# entry has 4e-8 more and the sum is above 2e-6 for some gammas.  1.6e-6 allowed on the mean of four gammas.
+@pytest.mark.parametrize("n", [13, 14, 16, 18, 19])
+@pytest.mark.parametrize("half", [False, True])
+def test_single_table_entries(Q, n, half):
+    f, fd, p = oracle.labs_costs(n), Q.labs_costs(n), 32
+    s = Q.cost_stats_compute(fd)
+    if not half:
+        s.reserved = 0
+    rms = []
+    for gamma in (0.013, 0.0371, 0.077, 0.1):
+        x, _ = Q.simulate(fd, s, [gamma] * p, [0.0] * p, state_type=Q.C64)
+        d = dev_np(x) * 2.0 ** (n / 2) - np.exp(-1j * gamma * p * f)
+        rms.append(np.sqrt(np.mean(np.abs(d) ** 2)))
+    assert np.mean(rms) < 1.6e-6
