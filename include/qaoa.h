@@ -95,7 +95,15 @@ typedef struct {
                            vector then evolve only the amplitudes whose top
                            qubit is 0, with the same results.  The mark covers
                            n and the fields above: changing any of them, or
-                           setting it to 0, takes the path of any vector. */
+                           setting it to 0, takes the path of any vector.
+                           It says nothing of the vector's contents: statistics
+                           with a mark hold only for the vector as it was
+                           scanned.  After any write to it (one element, a
+                           field added, another instance of the same range)
+                           scan again, or set this to 0 if the fields above
+                           still hold; a call with a stale mark evolves half of
+                           a vector that is not symmetric, and gives wrong
+                           results without an error. */
 } qaoa_cost_stats;
 
 /* Human-readable name of a status code (static string, never NULL). */

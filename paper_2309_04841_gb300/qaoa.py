@@ -318,6 +318,9 @@ def maxcut_costs(n, edges, weights=None, cost_type=COST_I32, out=None):
 
 
 def cost_stats_compute(costs, work=None):
+    """Statistics of a cost vector, for simulate, grad and overlap.  They hold for the vector as it is now: scan again
+    after any write to it.  (Where f(x) = f(~x) they carry a mark, `reserved`, by which those calls evolve half of the
+    amplitudes; with a vector changed since, that gives wrong results without an error.  reserved = 0 drops the mark.)"""
     n = _n_of(costs)
     if work is None:
         work = workspace(n)
@@ -345,7 +348,8 @@ def _angles(gammas, betas):
 def simulate(costs, stats, gammas, betas, state=None, state_type=C64, init_plus=True,
              work=None, out=None, reduce=True):
     """Algorithm 3 on the device.  Returns (state, out) where out holds
-    [E, O] (device float64) when reduce is True, else None."""
+    [E, O] (device float64) when reduce is True, else None.  stats: of costs as
+    they are (scan again after any write, see cost_stats_compute)."""
     torch = _torch()
     n = _n_of(costs)
     g, b = _angles(gammas, betas)
@@ -491,7 +495,8 @@ def overlap(state, costs, stats, work=None, out=None):
 
 def grad(costs, stats, gammas, betas, state=None, lam=None, state_type=C64, work=None, out=None):
     """Objective and adjoint gradient.  Returns the device float64 tensor
-    [E, O, dE/dgamma_1..p, dE/dbeta_1..p]."""
+    [E, O, dE/dgamma_1..p, dE/dbeta_1..p].  stats: of costs as they are (scan
+    again after any write, see cost_stats_compute)."""
     torch = _torch()
     n = _n_of(costs)
     g, b = _angles(gammas, betas)

@@ -114,3 +114,21 @@ def test_on_chip_any_costs(Q, n, st):
         ref = np.concatenate([dg, db])
         assert np.linalg.norm(out[2:] - ref) <= 10 * tol * max(np.linalg.norm(ref), np.abs(f).max())
         assert abs(out[0] - E) <= 10 * tol * np.abs(f).max()
+
+
+@pytest.mark.parametrize("n", [8, 14, 21])
+def test_vector_changed_after_the_scan(Q, n):
+    # what the header asks for after a write: a new scan finds the asymmetry, reserved = 0 keeps the other fields' use
+    fd = Q.labs_costs(n)
+    s = Q.cost_stats_compute(fd)
+    fd[5] += 4  # within the range and the step of the statistics
+    assert s.f_min <= float(fd[5]) <= s.f_max
+    g, b = [0.05, 0.02], [0.3, 0.7]
+    f = dev_np(fd).astype(float)
+    ref = oracle.simulate(n, f, g, b)
+    new = Q.cost_stats_compute(fd)
+    assert new.reserved == 0
+    s.reserved = 0
+    for st in (s, new):
+        x, e = Q.simulate(fd, st, g, b, state_type=Q.C128)
+        assert np.linalg.norm(dev_np(x) - ref) < 1e-13
