@@ -121,7 +121,7 @@ def test_vector_changed_after_the_scan(Q, n):
     # what the header asks for after a write: a new scan finds the asymmetry, reserved = 0 keeps the other fields' use
     fd = Q.labs_costs(n)
     s = Q.cost_stats_compute(fd)
-    fd[5] += 4  # within the range and the step of the statistics
+    fd[5] += 4  # within the range of the statistics, and but for n = 14 (steps of 8) within their step
     assert s.f_min <= float(fd[5]) <= s.f_max
     g, b = [0.05, 0.02], [0.3, 0.7]
     f = dev_np(fd).astype(float)
@@ -129,6 +129,6 @@ def test_vector_changed_after_the_scan(Q, n):
     new = Q.cost_stats_compute(fd)
     assert new.reserved == 0
     s.reserved = 0
-    for st in (s, new):
+    for st in (s, new) if 4 % (1 << s.step_log2) == 0 else (new,):
         x, e = Q.simulate(fd, st, g, b, state_type=Q.C128)
         assert np.linalg.norm(dev_np(x) - ref) < 1e-13

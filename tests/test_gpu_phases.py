@@ -20,12 +20,16 @@ def Q():
     return qaoa
 
 
-def check(Q, n, terms, scale, st, symmetric=False):
+def check(Q, n, terms, scale, st, symmetric=False, u16=False, step=None):
     """Simulation and gradient of an integer polynomial at p = 2, gammas up to `scale`."""
     f = oracle.costs_terms_int(n, terms).astype(float)
     fd = Q.precompute_costs(n, terms)
     s = Q.cost_stats_compute(fd)
     assert (s.f_min, s.f_max) == (f.min(), f.max()) and (s.reserved != 0) == symmetric
+    if u16:
+        fd = Q.convert_costs(fd, s, Q.COST_U16)
+    if step is not None:  # a struct filled by hand: 0 is always valid
+        s = Q.CostStats(s.f_min, s.f_max, s.n_min, step, 0)
     g, b = I.angles(2, 5 + n, 0.2 * scale, scale), I.angles(2, 70 + n)
     tol = 5e-6 if st == Q.C64 else 1e-13
     x, e = Q.simulate(fd, s, g, b, state_type=st)
@@ -108,3 +112,28 @@ def test_single_table_entries(Q, n, half):
         d = dev_np(x) * 2.0 ** (n / 2) - np.exp(-1j * gamma * p * f)
         rms.append(np.sqrt(np.mean(np.abs(d) ** 2)))
     assert np.mean(rms) < 1.6e-6
+
+
+# weights, and the number of steps of the cost's range: tables of two digits take up to 3071 (streamed complex64) or
+# 8191 steps, of three up to 32767 or 262143, larger ranges are computed (n <= 12: tables up to 8191, then computed)
+WAYS = {"two": ((400, 148, 12), 140), "three": ((4001, 1503, 7), 5511), "three_wide": ((15001, 12503, 7), 27511),
+        "three_most": ((120001, 110003, 7), 230011), "computed": ((300001, 250003, 7), 550011)}
+
+
+@pytest.mark.parametrize("n,st", [(12, 0), (12, 1), (13, 0), (16, 0), (16, 1), (21, 0), (21, 1), (22, 0)])
+@pytest.mark.parametrize("way", list(WAYS))
+@pytest.mark.parametrize("half", [False, True])
+def test_every_way(Q, n, st, way, half):
+    (a, b, c), steps = WAYS[way]
+    terms = [(a, (0, n - 1)), (b, (2, 5) if half else (2,)), (c, (3, 4))] + [(c, (3, 4, 6))] * (not half)
+    s = check(Q, n, terms, 100.0 / (a + b + 2 * c), st, symmetric=half)
+    assert abs((s.f_max - s.f_min) / 2 ** s.step_log2 - steps) <= 14
+
+
+# uint16 costs: differences are even, so 32767 steps are the most; step_log2 = 0 by hand leaves tables of three digits
+@pytest.mark.parametrize("n,st", [(13, 0), (16, 1), (21, 0), (21, 1)])
+@pytest.mark.parametrize("step", [None, 0])
+def test_uint16_ways(Q, n, st, step):
+    for (a, b, c) in ((400, 148, 12), (4001, 1503, 7), (15001, 12503, 7)):
+        terms = [(a, (0, n - 1)), (b, (2,)), (c, (3, 4)), (a + b + c, ())]
+        check(Q, n, terms, 100.0 / (2 * (a + b + c)), st, u16=True, step=step)
