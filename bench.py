@@ -17,7 +17,8 @@ path), the time is the max over ranks and `value` counts all ranks' steps.
 
 Besides the headline line's required keys it reports: the roofline of the
 adjoint sweep and of the forward sweep on algorithmic bytes (20 B per
-amplitude per forward layer, 36 B per adjoint layer), the per-pass DRAM rates
+amplitude held per forward layer, 36 B per adjoint layer; half of the vector
+where the costs have f(x) = f(~x)), the per-pass DRAM rates
 (`kernel_efficiency`), the error of every result against the stored
 complex128 oracle values (`result_error`), the other named workloads
 (`variants`), the serving loop against the plain per-request path on a
@@ -207,6 +208,12 @@ def traffic_record(n, p):
     return rec.get("kernels")
 
 
+def held(stats, N):
+    """Amplitudes that an evaluation from |+> has to hold and move: half of the
+    vector where the cost vector has f(x) = f(~x) (the mark of its statistics)."""
+    return N // 2 if stats.reserved else N
+
+
 def cost_build_line(n, N, ms):
     """The LABS cost-vector build against the popcount rate: n - 1 popcounts
     per element (one per shift k), at 16 per clock per SM (the CUDA
@@ -354,14 +361,15 @@ def run_ours(a, ws, rank, local):
     e2e_s = max_over_ranks(time.perf_counter() - t, ws)
     barrier(ws)
 
-    # ---- rooflines on algorithmic bytes (N amplitudes, complex64 8 B, int32
-    # cost 4 B): a forward layer reads psi and f and writes psi (20 B N), an
-    # adjoint layer reads psi, lambda, f and writes psi, lambda (36 B N)
+    # ---- rooflines on algorithmic bytes (H amplitudes held, complex64 8 B,
+    # int32 cost 4 B): a forward layer reads psi and f and writes psi (20 B H),
+    # an adjoint layer reads psi, lambda, f and writes psi, lambda (36 B H)
+    H = held(stats, N)
     peak, peak_src = measured_peaks()
     kinds = {k: v for k, v in prof.items() if v["launches"] > 0}
     sp = sweep_split(kinds, a.steps)
-    alg_adj = 36.0 * N * p
-    alg_fwd = 20.0 * N * p
+    alg_adj = 36.0 * H * p
+    alg_fwd = 20.0 * H * p
     ach_adj = alg_adj / (sp["adjoint"]["ms"] * 1e-3) / 1e9
     ach_fwd = alg_fwd / (sp["forward"]["ms"] * 1e-3) / 1e9
     traffic = traffic_record(n, p)
@@ -393,7 +401,7 @@ def run_ours(a, ws, rank, local):
             "achieved": ach_adj, "peak": peak, "unit": "GB/s", "frac": ach_adj / peak,
             "traffic": dram_adj,
             "algorithmic_bytes_per_launch": alg_adj,
-            "launch": f"one adjoint sweep = p={p} layers x 36 B x 2^{n} amplitudes, "
+            "launch": f"one adjoint sweep = p={p} layers x 36 B x 2^{H.bit_length() - 1} amplitudes, "
                       f"{sp['adjoint']['launches']} kernel launches",
             "ms_per_launch": sp["adjoint"]["ms"],
             "pass_structure_bytes_per_launch": sp["adjoint"]["pass_bytes"],
@@ -477,7 +485,7 @@ def variants(a, ws, costs, stats, state, work, out, g, b, w, stream):
          "value": 1000.0 / ms128, "unit": UNIT, "ms_per_eval": ms128,
          # complex128: a forward layer moves 16 + 4 + 16 B per amplitude, an
          # adjoint layer 2 * 32 + 4 B
-         "step_alg_frac": (36.0 + 68.0) * N * p / (ms128 * 1e-3) / 1e9 / peak,
+         "step_alg_frac": (36.0 + 68.0) * held(stats, N) * p / (ms128 * 1e-3) / 1e9 / peak,
          "energy": float(o128[0])}
     if G and G["recipe"]["n"] == n and G["recipe"]["p"] == p:
         e["energy_rel_err"] = rel_err(float(o128[0]), G["energy"])
@@ -553,7 +561,7 @@ def forward_variant(name, st, reps, stream, peak):
     r = o.cpu().numpy()
     es = 16.0 if st == Q.C128 else 8.0
     cb = float(fd.element_size())
-    alg = (2 * es + cb) * N * p  # read psi and f, write psi, per layer
+    alg = (2 * es + cb) * held(stats, N) * p  # read psi and f, write psi, per layer
     v = {"workload": f"{name}: n={n} p={p}, {'complex128' if st == Q.C128 else 'complex64'} state, "
                      f"{w['cost']} costs, forward + energy/overlap",
          "us_per_eval": ms * 1e3, "evals_per_s": 1000.0 / ms, "layers_per_s": p * 1000.0 / ms,
@@ -593,8 +601,8 @@ def grad_variant(name, reps, stream, peak):
     Q.profile_enable(False)
     sp = sweep_split({k: v for k, v in Q.profile_read(reset=True).items() if v["launches"] > 0}, reps)
     cb = float(fd.element_size())
-    a_adj = (32.0 + cb) * N * p
-    a_fwd = (16.0 + cb) * N * p
+    a_adj = (32.0 + cb) * held(stats, N) * p
+    a_fwd = (16.0 + cb) * held(stats, N) * p
     del s, lam, fd
     torch.cuda.empty_cache()
     return {"workload": f"{name}: n={n} p={p}, complex64, {w['cost']} costs, objective + all "
