@@ -387,10 +387,13 @@ qaoa_status qaoa_overlap(int n, const void *d_state, qaoa_state_type st,
  *   d_out: device, 2 + 2p doubles: [E, O, dE/dgamma_1..p, dE/dbeta_1..p],
  *     E and O of the forward final state.
  * Asynchronous.
- * Plan (complex64, n >= 13): the backward passes rotate the qubits in
+ * Plan: n <= 12 (complex64 with the mark of qaoa_cost_stats.reserved: n <= 13)
+ * runs on chip in one launch per 128 layers (complex128: 96), n <= 19 in passes
+ * over small tiles.  Beyond, the complex64 backward passes rotate the qubits in
  * groups; a group of up to 9 qubits on a 2^13-amplitude tile is taken where
  * it saves a group (n = 21, 29, 30).  Its passes run on one 512-thread CTA
- * per tile, the last pass on a pair of CTAs that exchange halves of the tile.
+ * per tile; without the mark the last pass runs on a pair of CTAs that exchange
+ * halves of the tile.
  * Environment variables, read at each call: QAOA_ADJOINT_PAIRS = "never" (no
  * such groups) or "always" (every group above the lowest 12 qubits is one);
  * QAOA_ADJOINT_WIDE = "pair" (every pass of those groups on CTA pairs) or
@@ -412,8 +415,9 @@ qaoa_status qaoa_grad(int n, const void *d_costs, qaoa_cost_type ct,
  * (qaoa_server_submit returns at once).  A scheduler thread admits them as
  * GPU slots and device memory free up and runs admitted work concurrently:
  * requests with n <= 12 and p <= 128 are packed many per kernel launch (one
- * CTA each, state on chip); larger ones run on their own CUDA streams, up to
- * max_inflight units at a time.  All device memory comes from one
+ * CTA each, state on chip), two such batches at a time, more when 64 requests
+ * wait; larger ones run on their own CUDA streams, up to max_inflight units at
+ * a time in all.  All device memory comes from one
  * caller-owned arena (d_arena, arena_bytes), sub-allocated by the server:
  * a running request holds its state (8 B x 2^n, complex64), lambda (the same,
  * gradient requests only), workspace and outputs; cost vectors are cached per
@@ -429,7 +433,7 @@ typedef enum { QAOA_PROBLEM_LABS = 0, QAOA_PROBLEM_MAXCUT = 1 } qaoa_problem;
 typedef struct {
     int max_inflight;  /* GPU work units (streams) at once, 1..64           */
     int max_queue;     /* pending requests accepted before QAOA_ERR_BUSY    */
-    int small_batch;   /* most n <= 12 requests packed into one launch      */
+    int small_batch;   /* most n <= 12 requests packed into one batch       */
 } qaoa_server_config;
 
 typedef struct {

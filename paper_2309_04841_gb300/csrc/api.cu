@@ -2,16 +2,19 @@
 //
 // The planner turns one call into a short sequence of kernel launches on the
 // caller's stream:
-//   n <= 12        : single-CTA kernels with the whole state on chip;
-//   n >  12 (tiled): the qubits split into k groups, a LOW group (the TB
+//   on chip (small_path)  : n <= 12 index bits, one CTA with the whole state;
+//   tiled                 : the qubits split into k groups, a LOW group (the TB
 //                    lowest qubits, one contiguous tile) and HIGH groups
 //                    (TB - c qubits each beside 2^c contiguous amplitudes,
-//                    c = 3..5); each layer passes over every group once, with
+//                    c = 2..5); each layer passes over every group once, with
 //                    the phase in the pass that opens the layer, and the
 //                    group order reversed every layer so that the last pass
 //                    of one layer and the first of the next are one pass
 //                    (k - 1 passes per layer).  The adjoint runs the same
-//                    kind of schedule backwards on (psi, lambda).
+//                    kind of schedule backwards on (psi, lambda).  Up to n = 19
+//                    tiles are small (mid_path); beyond, complex64 vectors are
+//                    streamed by TMA (tma_ok) and others by plain loads.
+// Costs with f(x) = f(~x) take n - 1 index bits (half vectors, comp_symmetric).
 // Nothing here allocates device memory: scratch lives in the caller's
 // workspace, per-layer constants travel in the kernel parameter blocks.
 #include <algorithm>

@@ -2,8 +2,8 @@
 // paper).  Objective (+ gradient) requests of different n and p arrive at any
 // time; a scheduler thread admits them as GPU slots and device memory free up
 // and runs admitted work concurrently:
-//   * n <= 12 requests are packed, many per launch, into k_small_batch
-//     (one CTA per request, state and lambda on chip);
+//   * n <= 12 requests are packed in batches of k_small_batch launches, one per
+//     number of index bits (one CTA per request, state and lambda on chip);
 //   * larger requests run qaoa_grad / qaoa_simulate on their own stream,
 //     several streams at once, so mid-size requests that cannot fill the GPU
 //     alone overlap with each other.
@@ -311,7 +311,7 @@ bool start_large(qaoa_server *S, Job *j, int u) {
   return true;
 }
 
-// Pack pending small jobs (n <= 12, p <= 128) into one launch on unit u.
+// Pack pending small jobs (n <= 12, p <= 128) into one batch on unit u.
 bool start_small_batch(qaoa_server *S, std::vector<Job *> &cand, int u) {
   Unit &U = S->units[u];
   std::vector<Job *> batch;

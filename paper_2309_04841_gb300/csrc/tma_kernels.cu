@@ -712,7 +712,6 @@ __device__ __forceinline__ float cost_val(int kind, uint32_t word) {
   return kind == kCostF32 ? __uint_as_float(word) : (float)(int)word;
 }
 
-// v <- v * exp(-i g f) (* the scale that the tables carry).
 // Cost-tile slot of register r's amplitude in round R (tt = thr_tile).
 template <class PL, int R, bool CP>
 __device__ __forceinline__ uint32_t cost_slot(uint32_t tt, int r) {
@@ -722,6 +721,7 @@ __device__ __forceinline__ uint32_t cost_slot(uint32_t tt, int r) {
     return tt | pdep(r, PL::reg(R));
 }
 
+// v <- v * exp(-i g f) (* the scale that the tables carry).
 template <class PL, int R, bool CP, int M>
 __device__ __forceinline__ void phase_round_m(float2 (&v)[PL::NREG], const CostWord *cb,
                                               const PhaseDigits &ph, const float2 *tab) {
