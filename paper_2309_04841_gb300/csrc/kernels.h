@@ -146,8 +146,9 @@ static_assert(comp_plan<PlanTmaF13High>() && comp_plan<PlanTmaB12High>() && comp
 // g f / 2pi, up to 2^-25 of it, is part of r, so from |g f / 2pi| = 2^36 on (penalties of
 // 1e12, say) nd = 0 takes the form that reduces r once more; nd = 1 (float32 costs below)
 // does without, 0.8% of a weighted MaxCut n = 28 gradient.  It is the pivots' arithmetic that costs
-// there: weighted MaxCut n = 28 pivots 658 -> 556 us forward and 1339 -> 1152 us
-// adjoint against sincospi and a scale multiply per amplitude.
+// there: weighted MaxCut n = 28 pivots 658 -> 559 us forward and 1339 -> 1161 us
+// adjoint against sincospi and a scale multiply per amplitude; the phase's error is
+// smaller (32 equal layers, beta = 0: 1.7e-6 -> 1.2e-6 rms).
 constexpr int kPhaseCopies = 16;
 constexpr int kPhaseMaxEntries = 112;
 constexpr int kPhaseTabEntries = kPhaseMaxEntries * kPhaseCopies;

@@ -137,3 +137,24 @@ def test_uint16_ways(Q, n, st, step):
     for (a, b, c) in ((400, 148, 12), (4001, 1503, 7), (15001, 12503, 7)):
         terms = [(a, (0, n - 1)), (b, (2,)), (c, (3, 4)), (a + b + c, ())]
         check(Q, n, terms, 100.0 / (2 * (a + b + c)), st, u16=True, step=step)
+
+
+# float32 costs on the streamed passes: table entry (2.4e-8 rms), sine and cosine of the rest (1.7e-8) and their product
+# (2.4e-8) repeat in each of 32 equal layers, 32 * 3.8e-8 = 1.2e-6; with the fraction of gamma f / 2 pi rounded to one
+# float (5e-8 where it is above a quarter turn) 1.8e-6.  1.4e-6 allowed on the mean of four gammas.
+@pytest.mark.parametrize("n", [21, 22])
+@pytest.mark.parametrize("kind", ["labs", "gnp"])
+def test_float_phases(Q, n, kind):
+    p = 32
+    if kind == "labs":
+        fd, gammas = Q.labs_costs(n).float(), (0.013, 0.0371, 0.077, 0.1)
+    else:
+        e, w = I.maxcut_gnp(n, 0.5, graph_seed=3, weight_seed=4)
+        fd, gammas = Q.maxcut_costs(n, e, w, Q.COST_F32), (0.11, 0.23, 0.37, 0.6)
+    s = Q.cost_stats_compute(fd)
+    f, rms = dev_np(fd).astype(float), []
+    for gamma in gammas:
+        x, _ = Q.simulate(fd, s, [gamma] * p, [0.0] * p, state_type=Q.C64)
+        d = dev_np(x) * 2.0 ** (n / 2) - np.exp(-1j * gamma * p * f)
+        rms.append(np.sqrt(np.mean(np.abs(d) ** 2)))
+    assert np.mean(rms) < 1.4e-6
