@@ -1340,6 +1340,18 @@ WalshTerms walsh_terms(int n, qaoa_cost_type ct, void *out, int e, int halve) {
   return P;
 }
 
+// Whether the transform is the faster one.  It costs nearly the same for any number of
+// terms (n = 24: int32 27 us, 64-bit sums 205), the loops over terms or edges from 23, 158
+// and 66 us on, and 5 to 10 us more for each: from 2 terms on in int32, from 23 on in 64-bit
+// sums (n = 24: 17 terms 164 against 204 us, 40 306 against 205; 17 edges 179 against 203,
+// 40 410 against 204).  Small vectors are bound by the call: the loops' parameter blocks cost
+// 12 us against 6 (int32 terms) and 17 against 16 (edges), but 12 against 16 for 64-bit terms
+// (n = 13, 40 terms: 12.7 against 16.5; 400: 25 against 19).
+bool walsh_pays(int n, size_t count, bool wide, bool edges) {
+  if (n <= 20 && (edges || !wide)) return true;
+  return count > (!wide ? 1u : n <= 17 ? 100u : n <= 19 ? 32u : 22u);
+}
+
 void walsh_add(WalshTerms &P, uint64_t mask, int64_t w) {
   P.mask[P.nterms] = (uint32_t)mask;
   P.w[P.nterms++] = w;
@@ -1497,7 +1509,8 @@ qaoa_status qaoa_precompute_costs(int n, const qaoa_term *terms, size_t n_terms,
       return fail(QAOA_ERR_INVALID_ARG, "float32 costs take at most 1024 terms per call");
   }
   const size_t nchunks = n_terms ? (n_terms + kTermChunk - 1) / kTermChunk : 1;
-  if (n >= kWalshBits && n <= 32 && mode != kTermF64) {  // sums in any order: by transform
+  if (n >= kWalshBits && n <= 32 && mode != kTermF64 && walsh_pays(n, n_terms, mode == kTermFixed, false)) {
+    // sums in any order: by transform
     for (size_t c = 0; c < nchunks; ++c) {
       const size_t k0 = c * kTermChunk, k1 = std::min(k0 + (size_t)kTermChunk, n_terms);
       WalshTerms P = walsh_terms(n, ct, d_costs, mode == kTermFixed ? e_fix : 0, 0);
@@ -1581,7 +1594,7 @@ qaoa_status qaoa_maxcut_costs(int n, const int32_t *edges, const double *w, size
     if (!std::isfinite(wv[e])) return fail(QAOA_ERR_INVALID_ARG, "maxcut_costs: non-finite weight");
   }
   // 2 f = sum w s_i s_j - sum w, by transform where the sums are exact (2 sum |w| in range)
-  if (n >= kWalshBits && n <= 32 && m < (size_t)kTermChunk) {
+  if (n >= kWalshBits && n <= 32 && m < (size_t)kTermChunk && walsh_pays(n, m, ct != QAOA_COST_I32, true)) {
     int e = 0;
     double tot = 0.0;
     bool whole = true;

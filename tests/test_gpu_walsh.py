@@ -38,3 +38,20 @@ def test_maxcut(Q, n):
         wi = np.zeros(len(e))
         wi[0], wi[-1] = top - 7, 7
         np.testing.assert_array_equal(dev_np(Q.maxcut_costs(n, e, wi)), oracle.maxcut_costs(n, e, wi).astype(np.int32))
+
+
+# the transform or the loops over terms and edges (walsh_pays): either side of each count, sizes of each rule
+@pytest.mark.parametrize("n", [13, 17, 18, 19, 20, 21])
+@pytest.mark.parametrize("count", [1, 2, 22, 23, 32, 33, 100, 101])
+def test_either_way(Q, n, count):
+    terms = I.random_terms(n, count, 7 * n + count, max_order=4, integer=True)
+    f = oracle.costs_terms_int(n, terms)
+    for ct, dt in ((Q.COST_I32, np.int32), (Q.COST_F32, np.float32), (Q.COST_F64, np.float64)):
+        np.testing.assert_array_equal(dev_np(Q.precompute_costs(n, terms, ct)), f.astype(dt))
+    r = np.random.RandomState(count)
+    e = r.randint(0, n, (count, 2)).astype(np.int32)
+    e[:, 1] = (e[:, 0] + 1 + r.randint(0, n - 1, count)) % n
+    w = np.floor(r.rand(count) * 8) + 1
+    g = oracle.maxcut_costs(n, e, w)
+    for ct, dt in ((Q.COST_I32, np.int32), (Q.COST_F32, np.float32), (Q.COST_F64, np.float64)):
+        np.testing.assert_array_equal(dev_np(Q.maxcut_costs(n, e, w, ct)), g.astype(dt))
