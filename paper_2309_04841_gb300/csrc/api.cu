@@ -1869,6 +1869,17 @@ std::vector<XyRound> xy_rounds(const XyOp &o) {
   return out;
 }
 
+// Whether a tile's gates run one at a time, a pair a thread, instead of in register
+// rounds, 16 amplitudes a thread.  A round needs four tile bits.  In complex128 a round's
+// registers (64 for 16 amplitudes) leave one CTA an SM, and on small tiles few threads at
+// work: rings n = 21 to 23 p = 6 2.79 -> 2.42, 4.92 -> 4.29 and 10.3 -> 8.65 ms one gate at a time,
+// n = 8 103 -> 66 us, complete graphs n = 8 230 -> 115 us, n = 10 392 -> 292; from n = 12 on
+// complete graphs are faster in rounds (1346 -> 1308 us) or equal.  complex64: rounds
+// always (complete graph n = 6 59 -> 47 us, n = 10 119 -> 84).
+bool xy_single(int tb, int graph, bool c128) {
+  return tb < 4 || (c128 ? graph == QAOA_XY_RING || tb <= 10 : false);
+}
+
 // The pair rotation by beta as three shears: beta reduced to [-pi/2, pi/2]
 // (a rotation by pi is the exact factor -1).
 void xy_beta(double beta, double &tb2, double &sb, int &neg) {
@@ -2024,6 +2035,7 @@ qaoa_status qaoa_simulate_xy(int n, const void *d_costs, qaoa_cost_type ct, cons
       P.sb = sb;
       P.neg = neg;
       P.nrounds = (int)rounds[k].size();
+      P.single = xy_single(P.tb, graph, c128);
       if (P.nrounds > kXyMaxRounds) return fail(QAOA_ERR_INVALID_ARG, "internal: too many XY rounds");
       std::copy(rounds[k].begin(), rounds[k].end(), P.rounds);
       LAUNCH("xy_tile", 2.0 * es * N + (P.has_phase ? cost_bytes(ct) * N : 0.0), s,

@@ -293,6 +293,7 @@ struct XyPass {
   double tb2, sb;            // tan(b/2), sin(b) of the layer's beta reduced to |b| <= pi/2
   int neg;                   // the reduction took out a factor -1
   int nrounds;
+  int single;  // a gate at a time in shared memory (xy_single)
   XyRound rounds[kXyMaxRounds];
   PhaseDigits ph;  // complex64 integer costs: digit tables (mode 0), else computed
 };

@@ -166,7 +166,8 @@ __device__ __forceinline__ C2 xy_phased(const XyPass &P, const float2 *tab, bool
 // PF (complex64): the next tile's amplitudes are loaded into registers while
 // the gates run on the current one in shared memory; otherwise the tile is
 // loaded just before its gates.
-template <typename C2, bool PF>
+// SINGLE: no rounds, a gate at a time, a pair a thread (xy_single in api.cu).
+template <typename C2, bool PF, bool SINGLE>
 __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_constant__ XyPass P) {
   using R = typename XyR<C2>::R;
   extern __shared__ __align__(16) unsigned char xy_smem[];
@@ -174,6 +175,7 @@ __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_consta
   C2 *psi = reinterpret_cast<C2 *>(P.psi);
   const uint32_t TE = 1u << P.tb;
   float2 *tab = reinterpret_cast<float2 *>(xy_smem + (size_t)TE * sizeof(C2));
+  auto slot = [](uint32_t i) { return SINGLE ? i : xy_slot(i); };
   const R th = (R)P.tb2, sn = (R)P.sb;
   const bool neg = P.neg != 0;
   const bool table = P.has_phase && P.ph.mode == 0;
@@ -206,8 +208,8 @@ __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_consta
             v0 = xy_phased(P, tab, table, v0, x);
             v1 = xy_phased(P, tab, table, v1, x + 1);
           }
-          s[xy_slot(t)] = v0;
-          s[xy_slot(t + 1)] = v1;
+          s[slot(t)] = v0;
+          s[slot(t + 1)] = v1;
         }
       }
       __syncthreads();
@@ -221,23 +223,23 @@ __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_consta
           v0 = xy_phased(P, tab, table, v0, x);
           v1 = xy_phased(P, tab, table, v1, x + 1);
         }
-        s[xy_slot(t)] = v0;
-        s[xy_slot(t + 1)] = v1;
+        s[slot(t)] = v0;
+        s[slot(t + 1)] = v1;
       }
       __syncthreads();
     }
     for (int k = 0; k < P.nrounds; ++k) {
       const XyRound rd = P.rounds[k];
-      if (P.tb >= 4) {
+      if constexpr (!SINGLE) {
         uint32_t e[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) e[j] = xy_slot(1u << rd.bit[j]);
+        for (int j = 0; j < 4; ++j) e[j] = slot(1u << rd.bit[j]);
         for (uint32_t i = threadIdx.x; i < (TE >> 4); i += blockDim.x) {
           uint32_t o = i;
 #pragma unroll
           for (int j = 0; j < 4; ++j) o = ((o >> rd.bit[j]) << (rd.bit[j] + 1)) | (o & ((1u << rd.bit[j]) - 1u));
           C2 v[16];
-          o = xy_slot(o);  // (linear over XOR)
+          o = slot(o);  // (linear over XOR)
           auto at = [&](int q) -> C2 & {
             return s[o ^ ((q & 1) ? e[0] : 0u) ^ ((q & 2) ? e[1] : 0u) ^ ((q & 4) ? e[2] : 0u) ^ ((q & 8) ? e[3] : 0u)];
           };
@@ -256,20 +258,22 @@ __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_consta
           for (int q = 0; q < 16; ++q) at(q) = v[q];
         }
         __syncthreads();
-      } else {  // fewer than four qubits: a gate at a time
+      } else {
+        const uint32_t bits = rd.bit[0] | rd.bit[1] << 8 | rd.bit[2] << 16 | (uint32_t)rd.bit[3] << 24;
+#pragma unroll 1
         for (int g = 0; g < 6; ++g)
           if ((rd.mask >> g) & 1) {
-            const int a = rd.bit[xy_gate_a(g)], b = rd.bit[xy_gate_b(g)];
+            const int a = (bits >> (8 * xy_gate_a(g))) & 255u, b = (bits >> (8 * xy_gate_b(g))) & 255u;
             for (uint32_t i = threadIdx.x; i < (TE >> 2); i += blockDim.x) {
               const uint32_t t0 = insert2_32(i, a, b);
-              xy_pair<C2, R>(s[xy_slot(t0 | (1u << a))], s[xy_slot(t0 | (1u << b))], th, sn, neg);
+              xy_pair<C2, R>(s[slot(t0 | (1u << a))], s[slot(t0 | (1u << b))], th, sn, neg);
             }
             __syncthreads();
           }
       }
     }
     for (uint32_t t = 2 * threadIdx.x; t < TE; t += 2 * blockDim.x) {
-      st2(psi + xy_index(P, T, t), s[xy_slot(t)], s[xy_slot(t + 1)]);
+      st2(psi + xy_index(P, T, t), s[slot(t)], s[slot(t + 1)]);
     }
     __syncthreads();
   }
@@ -291,34 +295,33 @@ unsigned grid_n(uint64_t work, int nsm) {
 
 }  // namespace
 
-cudaError_t launch_xy_tile(const XyPass &P, bool c128, cudaStream_t s, int nsm) {
+template <typename C2, bool PF, bool SINGLE>
+static cudaError_t launch_xy_tile_t(const XyPass &P, cudaStream_t s, int nsm) {
   const size_t tabb = (size_t)kPhaseTabEntries * sizeof(float2);
-  const size_t smem = ((size_t)1 << P.tb) * (c128 ? 16 : 8) + (P.has_phase && P.ph.mode == 0 ? tabb : 0);
-  static int per_sm[2] = {0, 0};  // resident CTAs per SM (registers, shared memory)
-  if (!per_sm[0]) {
-    const size_t m64 = ((size_t)1 << kXyMaxTb) * 8 + tabb, m128 = ((size_t)1 << kXyMaxTb) * 16;
-    cudaError_t e = cudaFuncSetAttribute(k_xy_tile<float2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)m64);
+  const size_t smem = sizeof(C2) << P.tb, most = (sizeof(C2) << kXyMaxTb) + (sizeof(C2) == 8 ? tabb : 0);
+  auto kern = k_xy_tile<C2, PF, SINGLE>;
+  static int per_sm = 0;  // resident CTAs per SM (registers, shared memory)
+  if (!per_sm) {
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_xy_tile<double2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m128);
-    if (e != cudaSuccess) return e;
-    int b64 = 0, b128 = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b128, k_xy_tile<double2, false>, 256, m128) != cudaSuccess ||
-        b128 < 1)
-      b128 = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b64, k_xy_tile<float2, true>, 256, m64) != cudaSuccess ||
-        b64 < 1)
-      b64 = 1;
-    per_sm[1] = b128;
-    per_sm[0] = b64;
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, 256, most) != cudaSuccess || b < 1) b = 1;
+    per_sm = b;
   }
-  const uint64_t cap = (uint64_t)nsm * per_sm[c128 ? 1 : 0];
+  const uint64_t cap = (uint64_t)nsm * per_sm;
   const unsigned grid = (unsigned)(P.ntiles < cap ? P.ntiles : cap);
-  if (c128)
-    k_xy_tile<double2, false><<<grid, 256, smem, s>>>(P);
-  else
-    k_xy_tile<float2, true><<<grid, 256, smem, s>>>(P);
+  kern<<<grid, 256, smem + (P.has_phase && P.ph.mode == 0 ? tabb : 0), s>>>(P);
   return cudaGetLastError();
+}
+
+cudaError_t launch_xy_tile(const XyPass &P, bool c128, cudaStream_t s, int nsm) {
+  if (!P.single && P.tb < 4) return cudaErrorInvalidValue;  // a round holds four tile bits
+  if (c128)
+    return P.single ? launch_xy_tile_t<double2, false, true>(P, s, nsm) : launch_xy_tile_t<double2, false, false>(P, s, nsm);
+  // prefetching the next tile into registers pays on tiles that fill the CTA; the smallest ones
+  // are bound by fetching that code (ring n = 6 p = 6 33 -> 28 us of device time without)
+  if (P.single) return launch_xy_tile_t<float2, false, true>(P, s, nsm);
+  return P.tb > 9 ? launch_xy_tile_t<float2, true, false>(P, s, nsm) : launch_xy_tile_t<float2, false, false>(P, s, nsm);
 }
 
 cudaError_t launch_dicke(void *psi, bool c128, int n, int k, double amp, cudaStream_t s, int nsm) {

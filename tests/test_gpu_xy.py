@@ -127,3 +127,18 @@ def test_complete_graph_blocks(Q, n, st):
     state, _ = Q.simulate_xy(fd, stats, g, b, Q.dicke_state(n, n // 2, stype), Q.XY_COMPLETE)
     ref = oracle.simulate_xy(n, f, g, b, oracle.dicke(n, n // 2), Q.XY_COMPLETE)
     assert np.linalg.norm(dev_np(state).astype(np.complex128) - ref) <= TOL[st][0] * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n", [3, 4, 5, 9, 10, 11, 12, 13])
+@pytest.mark.parametrize("st,tol", [("c64", 5e-6), ("c128", 1e-13)])
+@pytest.mark.parametrize("graph", [1, 2])
+def test_tile_forms_vs_oracle(Q, n, st, tol, graph):
+    # gates one at a time or in register rounds, with and without the next tile's prefetch: either side of each line;
+    # roundings of up to 2 * 66 gates, 2 each, as in test_gpu_half.py
+    f = oracle.labs_costs(n).astype(float)
+    fd = Q.labs_costs(n)
+    k = n // 2
+    psi0 = dev_np(Q.dicke_state(n, k, state_type=Q.C128))
+    g, b = I.angles(2, n, 0, 0.2), I.angles(2, 30 + n)
+    x, _ = Q.simulate_xy(fd, Q.cost_stats_compute(fd), g, b, Q.dicke_state(n, k, state_type=Q.C64 if st == "c64" else Q.C128), graph)
+    assert np.linalg.norm(dev_np(x) - oracle.simulate_xy(n, f, g, b, psi0, graph)) < tol
