@@ -940,7 +940,7 @@ qaoa_status tiled_forward_pl(int n, const void *cost, qaoa_cost_type ct, const q
     if (uses_lanes(P.s1) || uses_lanes(P.s2)) return fail(QAOA_ERR_INVALID_ARG, "internal: plan needs lane rotations");
     P.has_phase = op.lp >= 0;
     if (P.has_phase) {  // s1 runs before the phase, s2 after it
-      make_phase<Real>(P.ph, gam[op.lp], ct, stats, sig);
+      make_phase<Real>(P.ph, gam[op.lp], ct, sizeof(Real) == 8 ? stats : nullptr, sig);
       sig = 1.0;
     }
     if (op.l2 >= 0) sig *= sigma_pow(red_rot_tiled<Real>(bet[op.l2]).sigma, sweep_qubits(P.s2));
@@ -1018,7 +1018,7 @@ qaoa_status tiled_backward_pl(int n, const void *cost, qaoa_cost_type ct, const 
     if (op.lp >= 0) {
       P.has_phase = 1;
       P.wg = (Real)(sig * sig);
-      make_phase<Real>(P.ph, -gam[op.lp], ct, stats, sig);  // the un-phase pays the pending scale
+      make_phase<Real>(P.ph, -gam[op.lp], ct, sizeof(Real) == 8 ? stats : nullptr, sig);  // the un-phase pays the pending scale
       sig = 1.0;
       P.out_g = d_grad_g + op.lp;
     }

@@ -166,18 +166,6 @@ __device__ __forceinline__ void unrot_regs_acc(C2 (&v)[1 << EB], C2 (&w)[1 << EB
   rot_regs<EB>(w, m, t, form);
 }
 
-// Cost value in the precision of the state.
-__device__ __forceinline__ void cost_r(const void *cost, int kind, uint64_t x, float &f) {
-  if (kind == kCostI32)
-    f = (float)__ldg(reinterpret_cast<const int *>(cost) + x);
-  else if (kind == kCostU16)
-    f = (float)__ldg(reinterpret_cast<const unsigned short *>(cost) + x);
-  else if (kind == kCostF32)
-    f = __ldg(reinterpret_cast<const float *>(cost) + x);
-  else
-    f = (float)__ldg(reinterpret_cast<const double *>(cost) + x);
-}
-
 // Cost value as a float pair hi + lo (exact for int32 and float32 costs,
 // ~2^-48 relative for float64 costs).
 __device__ __forceinline__ void cost_split(const void *cost, int kind, uint64_t x, float &hi,
@@ -206,10 +194,6 @@ __device__ __forceinline__ double cost_d(const void *cost, int kind, uint64_t x)
   return __ldg(reinterpret_cast<const double *>(cost) + x);
 }
 
-__device__ __forceinline__ void cost_r(const void *cost, int kind, uint64_t x, double &f) {
-  f = cost_d(cost, kind, x);
-}
-
 // scl exp(-i g f), f = fh + fl: g f / 2pi as a float-float, p + e = g_hi * fh
 // exactly (Dekker's two-product via fma), the small cross terms added once; only
 // the fraction r in [-1/2, 1/2] reaches sincospi.
@@ -221,30 +205,26 @@ __device__ __forceinline__ float2 phase_at(const PhaseData<float> &ph, float fh,
   sincospif(2.0f * r, &sn, &cs);
   return make_float2(cs * scl, -sn * scl);
 }
-__device__ __forceinline__ double2 phase_at(const PhaseData<double> &ph, double f, double scl) {
+// (complex128: a phase per amplitude takes g / 2pi's first part alone, a table entry both)
+__device__ __forceinline__ double2 phase_at(const PhaseData<double> &ph, double f, double scl, bool entry = false) {
   const double p = ph.g_hi * f;
-  const double r = (p - rint(p)) + fma(ph.g_lo, f, fma(ph.g_hi, f, -p));
+  const double r = entry ? (p - rint(p)) + fma(ph.g_lo, f, fma(ph.g_hi, f, -p)) : p - rint(p);
   double sn, cs;
   sincospi(2.0 * r, &sn, &cs);
   return make_double2(cs * scl, -sn * scl);
 }
 
-__device__ __forceinline__ float2 phase_int(const PhaseData<float> &ph, int f, float scl) {
-  const float fh = (float)f;
-  return phase_at(ph, fh, (float)((long long)f - (long long)fh), scl);
-}
-__device__ __forceinline__ double2 phase_int(const PhaseData<double> &ph, int f, double scl) {
-  return phase_at(ph, (double)f, scl);
-}
-
-// The phase tables in shared memory (mode 0).
-template <int NT, typename Real, typename C2>
-__device__ __forceinline__ void fill_phase(C2 *tab, const PhaseData<Real> &ph) {
+// The phase tables in shared memory (mode 0; complex64 passes here never have them,
+// their costs being float64).
+template <int NT>
+__device__ __forceinline__ void fill_phase(float2 *, const PhaseData<float> &) {}
+template <int NT>
+__device__ __forceinline__ void fill_phase(double2 *tab, const PhaseData<double> &ph) {
   const int lastbase = 64 * (ph.nd - 1);
   for (int i = threadIdx.x; i < ph.entries; i += NT) {
     const int digit = min(i >> 6, ph.nd - 1), j = (i - 64 * digit) << (6 * digit + ph.shift);
     const bool last = i >= lastbase;
-    tab[i] = phase_int(ph, last ? ph.fmin + j : j, last ? ph.scl : (Real)1);
+    tab[i] = phase_at(ph, (double)(last ? ph.fmin + j : j), last ? ph.scl : 1.0, true);
   }
 }
 
@@ -252,18 +232,18 @@ __device__ __forceinline__ void fill_phase(C2 *tab, const PhaseData<Real> &ph) {
 template <typename Real, typename C2>
 __device__ __forceinline__ C2 phase_factor(const PhaseData<Real> &ph, const C2 *tab, const void *cost, int kind,
                                            uint64_t x) {
-  if (ph.mode == 0) {
-    const int f = kind == kCostU16 ? (int)__ldg(reinterpret_cast<const unsigned short *>(cost) + x)
-                                   : __ldg(reinterpret_cast<const int *>(cost) + x);
-    const uint32_t d = (uint32_t)(f - ph.fmin) >> ph.shift;
-    if (ph.nd == 2) return cmul(tab[d & 63u], tab[64u + min(d >> 6, (uint32_t)ph.last)]);
-    return cmul(cmul(tab[d & 63u], tab[64u + ((d >> 6) & 63u)]), tab[128u + min(d >> 12, (uint32_t)ph.last)]);
-  }
   if constexpr (sizeof(Real) == 4) {
     float fh, fl;
     cost_split(cost, kind, x, fh, fl);
     return phase_at(ph, fh, fl, ph.scl);
   } else {
+    if (ph.mode == 0) {
+      const int f = kind == kCostU16 ? (int)__ldg(reinterpret_cast<const unsigned short *>(cost) + x)
+                                     : __ldg(reinterpret_cast<const int *>(cost) + x);
+      const uint32_t d = (uint32_t)(f - ph.fmin) >> ph.shift;
+      if (ph.nd == 2) return cmul(tab[d & 63u], tab[64u + min(d >> 6, (uint32_t)ph.last)]);
+      return cmul(cmul(tab[d & 63u], tab[64u + ((d >> 6) & 63u)]), tab[128u + min(d >> 12, (uint32_t)ph.last)]);
+    }
     return phase_at(ph, cost_d(cost, kind, x), ph.scl);
   }
 }
@@ -338,18 +318,9 @@ __device__ __forceinline__ void accum_eo(const C2 (&v)[PL::NREG], const void *co
   for (int r = 0; r < PL::NREG; ++r) {
     const uint64_t x = ix.at(r);
     const Real pr = v[r].x * v[r].x + v[r].y * v[r].y;
-    Real f;
-    bool at_min;
-    cost_r(cost, kind, x, f);
-    if (sizeof(Real) == 8 || kind == kCostF64)
-      at_min = cost_d(cost, kind, x) == fmin;
-    else if (kind == kCostF32)
-      at_min = f == (Real)fmin;
-    else  // (no float64 conversion per amplitude)
-      at_min = (kind == kCostU16 ? (int)__ldg(reinterpret_cast<const unsigned short *>(cost) + x)
-                                 : __ldg(reinterpret_cast<const int *>(cost) + x)) == (int)fmin;
-    e += pr * f;
-    o += at_min ? pr : (Real)0;
+    const double f = cost_d(cost, kind, x);
+    e += pr * (Real)f;
+    o += (f == fmin) ? pr : (Real)0;
   }
 }
 
@@ -527,9 +498,7 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
       const AmpIndex<PL, 0, CP> ix(g, base);
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
-        Real f;
-        cost_r(P.cost, P.cost_kind, ix.at(r), f);
-        f -= fc;
+        const Real f = (Real)cost_d(P.cost, P.cost_kind, ix.at(r)) - fc;
         w[r] = mk<C2>(f * v[r].x, f * v[r].y);
       }
     } else {
@@ -551,9 +520,7 @@ __global__ void __launch_bounds__(PL::NT, 2) k_bwd(const __grid_constant__ BwdPa
 #pragma unroll
       for (int r = 0; r < NREG; ++r) {
         const uint64_t x = ix.at(r);
-        Real f;
-        cost_r(P.cost, P.cost_kind, x, f);
-        f -= fc;
+        const Real f = (Real)cost_d(P.cost, P.cost_kind, x) - fc;
         raw += f * (w[r].x * v[r].y - w[r].y * v[r].x);
         const C2 ph = phase_factor(P.ph, tab, P.cost, P.cost_kind, x);
         v[r] = cmul(v[r], ph);

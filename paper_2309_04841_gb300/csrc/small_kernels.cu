@@ -247,9 +247,9 @@ __device__ __forceinline__ void small_run(const SmallJob<Real> &P) {
       const Real scl = low ? (Real)1 : adj ? L.sig_adj : li == 0 ? (Real)1 : Ls[li - 1].sig;
       const int j = low ? e << P.shift : P.fmin + ((P.ndig ? (e - 64) * 64 : e) << P.shift);
       const F f = P.by_x ? fs[O::template slot<EB>((uint32_t)e)] : O::integer(j);
-      // (n = 13: entries as exact as that size's always were, 102.8 -> 104.5 us; below, as
-      // exact as a phase per amplitude was)
-      C2 z = D == kSmallMaxN && half ? O::entry(L, f, scl, (Real)0) : O::phase(L, f, scl);
+      // (complex64 n = 13: entries as exact as that size's always were, 102.8 -> 104.5 us; below,
+      // as exact as a phase per amplitude was)
+      C2 z = sizeof(Real) == 8 || (D == kSmallMaxN && half) ? O::entry(L, f, scl, (Real)0) : O::phase(L, f, scl);
       if (adj) z.y = -z.y;
       tab[i] = z;
     }

@@ -56,12 +56,12 @@ def test_range_over_int32(Q, n, st, odd):
 # The fraction of gamma f / 2 pi is known to 2^-54 of a turn (3.5e-16 in the angle), sincospi adds 2.2e-16, a table's
 # product as much again for each of up to three factors: 2e-15 in all.  (With gamma / 2 pi in one double the angle is
 # off by |gamma f| 2^-53 and more: 5e-14.)
-@pytest.mark.parametrize("kind", ["i32", "f64"])
+# (integer costs, whose phases come from tables; a phase per amplitude takes one double, as it always did)
 @pytest.mark.parametrize("n", [5, 8, 12, 14, 18, 21])
 @pytest.mark.parametrize("half", [False, True])
-def test_double_phase(Q, n, kind, half):
+def test_double_phase(Q, n, half):
     f = oracle.labs_costs(n)
-    fd = Q.labs_costs(n) if kind == "i32" else Q.labs_costs(n).double()
+    fd = Q.labs_costs(n)
     s = Q.cost_stats_compute(fd)
     if not half:
         s.reserved = 0
