@@ -1870,14 +1870,14 @@ std::vector<XyRound> xy_rounds(const XyOp &o) {
 }
 
 // Whether a tile's gates run one at a time, a pair a thread, instead of in register
-// rounds, 16 amplitudes a thread.  A round needs four tile bits.  In complex128 a round's
-// registers (64 for 16 amplitudes) leave one CTA an SM, and on small tiles few threads at
-// work: rings n = 21 to 23 p = 6 2.79 -> 2.42, 4.92 -> 4.29 and 10.3 -> 8.65 ms one gate at a time,
-// n = 8 103 -> 66 us, complete graphs n = 8 230 -> 115 us, n = 10 392 -> 292; from n = 12 on
+// rounds, 16 amplitudes a thread.  A round needs four tile bits.  In complex128 a
+// round's registers (64 for 16 amplitudes) leave one CTA an SM, and on small tiles few threads
+// at work: rings n = 21 to 23 p = 6 2.79 -> 2.43, 4.92 -> 4.31 and 10.3 -> 8.70 ms one gate at a
+// time, n = 8 103 -> 70 us, complete graphs n = 8 230 -> 115 us, n = 10 392 -> 304; from n = 12 on
 // complete graphs are faster in rounds (1346 -> 1308 us) or equal.  complex64: rounds
 // always (complete graph n = 6 59 -> 47 us, n = 10 119 -> 84).
 bool xy_single(int tb, int graph, bool c128) {
-  return tb < 4 || (c128 ? graph == QAOA_XY_RING || tb <= 10 : false);
+  return tb < 4 || (c128 && (graph == QAOA_XY_RING || tb <= 10));
 }
 
 // The pair rotation by beta as three shears: beta reduced to [-pi/2, pi/2]

@@ -175,7 +175,6 @@ __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_consta
   C2 *psi = reinterpret_cast<C2 *>(P.psi);
   const uint32_t TE = 1u << P.tb;
   float2 *tab = reinterpret_cast<float2 *>(xy_smem + (size_t)TE * sizeof(C2));
-  auto slot = [](uint32_t i) { return SINGLE ? i : xy_slot(i); };
   const R th = (R)P.tb2, sn = (R)P.sb;
   const bool neg = P.neg != 0;
   const bool table = P.has_phase && P.ph.mode == 0;
@@ -208,8 +207,8 @@ __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_consta
             v0 = xy_phased(P, tab, table, v0, x);
             v1 = xy_phased(P, tab, table, v1, x + 1);
           }
-          s[slot(t)] = v0;
-          s[slot(t + 1)] = v1;
+          s[xy_slot(t)] = v0;
+          s[xy_slot(t + 1)] = v1;
         }
       }
       __syncthreads();
@@ -223,8 +222,8 @@ __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_consta
           v0 = xy_phased(P, tab, table, v0, x);
           v1 = xy_phased(P, tab, table, v1, x + 1);
         }
-        s[slot(t)] = v0;
-        s[slot(t + 1)] = v1;
+        s[xy_slot(t)] = v0;
+        s[xy_slot(t + 1)] = v1;
       }
       __syncthreads();
     }
@@ -233,13 +232,13 @@ __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_consta
       if constexpr (!SINGLE) {
         uint32_t e[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) e[j] = slot(1u << rd.bit[j]);
+        for (int j = 0; j < 4; ++j) e[j] = xy_slot(1u << rd.bit[j]);
         for (uint32_t i = threadIdx.x; i < (TE >> 4); i += blockDim.x) {
           uint32_t o = i;
 #pragma unroll
           for (int j = 0; j < 4; ++j) o = ((o >> rd.bit[j]) << (rd.bit[j] + 1)) | (o & ((1u << rd.bit[j]) - 1u));
           C2 v[16];
-          o = slot(o);  // (linear over XOR)
+          o = xy_slot(o);  // (linear over XOR)
           auto at = [&](int q) -> C2 & {
             return s[o ^ ((q & 1) ? e[0] : 0u) ^ ((q & 2) ? e[1] : 0u) ^ ((q & 4) ? e[2] : 0u) ^ ((q & 8) ? e[3] : 0u)];
           };
@@ -266,14 +265,14 @@ __global__ void __launch_bounds__(256, PF ? 2 : 1) k_xy_tile(const __grid_consta
             const int a = (bits >> (8 * xy_gate_a(g))) & 255u, b = (bits >> (8 * xy_gate_b(g))) & 255u;
             for (uint32_t i = threadIdx.x; i < (TE >> 2); i += blockDim.x) {
               const uint32_t t0 = insert2_32(i, a, b);
-              xy_pair<C2, R>(s[slot(t0 | (1u << a))], s[slot(t0 | (1u << b))], th, sn, neg);
+              xy_pair<C2, R>(s[xy_slot(t0 | (1u << a))], s[xy_slot(t0 | (1u << b))], th, sn, neg);
             }
             __syncthreads();
           }
       }
     }
     for (uint32_t t = 2 * threadIdx.x; t < TE; t += 2 * blockDim.x) {
-      st2(psi + xy_index(P, T, t), s[slot(t)], s[slot(t + 1)]);
+      st2(psi + xy_index(P, T, t), s[xy_slot(t)], s[xy_slot(t + 1)]);
     }
     __syncthreads();
   }
